@@ -53,8 +53,8 @@ __global__ void k_dot(int64_t n, const float2* __restrict__ a, const float2* __r
     part.add_prod(a[i].x, b[i].x);
     part.add_prod(a[i].y, b[i].y);
   }
-  double v = part.value(), tot;
-  if (reduce_last_block<1>(&v, partials, counter, &tot)) *out = tot;
+  double tot;
+  if (reduce_last_block<1>(&part, partials, counter, &tot)) *out = tot;
 }
 
 // ||a - w o y||^2 in FP64 -> *out
@@ -66,8 +66,8 @@ __global__ void k_norm_wdiff(int64_t n, const float2* __restrict__ a, const floa
     part.add_prod(d.x, d.x);
     part.add_prod(d.y, d.y);
   }
-  double v = part.value(), tot;
-  if (reduce_last_block<1>(&v, partials, counter, &tot)) *out = tot;
+  double tot;
+  if (reduce_last_block<1>(&part, partials, counter, &tot)) *out = tot;
 }
 
 // Re <a - w o y, r> in FP64 -> *out
@@ -80,8 +80,8 @@ __global__ void k_dot_wdiff(int64_t n, const float2* __restrict__ a, const float
     part.add_prod(d.x, r[i].x);
     part.add_prod(d.y, r[i].y);
   }
-  double v = part.value(), tot;
-  if (reduce_last_block<1>(&v, partials, counter, &tot)) *out = tot;
+  double tot;
+  if (reduce_last_block<1>(&part, partials, counter, &tot)) *out = tot;
 }
 
 // out = a + b + c

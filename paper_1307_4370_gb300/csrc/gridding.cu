@@ -128,9 +128,8 @@ __global__ void __launch_bounds__(256) k_degrid(const float2* __restrict__ X, co
   }
   for (int i = ch.y + threadIdx.x + QV * NT; i < ch.z; i += NT) visit(i, __ldg(&uv[i]));
   if (MODE == kDegridSdmm) {
-    double acc2[2] = {part[0].value(), part[1].value()};
     double tot[2];
-    if (reduce_last_block<2>(acc2, partials + kCntL2 * 2 * kMaxPartials, &sc->counter[kCntL2], tot)) {
+    if (reduce_last_block<2>(part, partials + kCntL2 * 2 * kMaxPartials, &sc->counter[kCntL2], tot)) {
       sc->l2_dn2 = tot[0];
       sc->l2_res2 = tot[1];
       sc->nu = sqrt(tot[1]) / sc->eps;

@@ -348,8 +348,8 @@ __global__ void __launch_bounds__(256) k_row_inv(const float2* __restrict__ half
   if (MODE == kRowOutCgQ) {
     // per-block partials of gamma = <r, r> and delta = <Qr, r>; the kernel
     // that applies this step's update adds them and forms the step sizes
-    double acc[2] = {dst.part[0].value(), dst.part[1].value()};
-    block_reduce<2>(acc);
+    double acc[2];
+    block_reduce<2>(dst.part, acc);
     if (threadIdx.x == 0) {
       partials[kCntDot * 2 * kMaxPartials + blockIdx.x] = acc[0];
       partials[kCntDot * 2 * kMaxPartials + kMaxPartials + blockIdx.x] = acc[1];
@@ -463,8 +463,8 @@ __global__ void __launch_bounds__(NSIG * L / E, p2_rinv_minb(NSIG * L / E, MODE)
   dst.invL = 1.0f / (float)L;
   fft_p2<L, E, NSIG, false, false, true>(sm, twt, src, dst);
   if (MODE == kRowOutCgQ) {
-    double acc[2] = {dst.part[0].value(), dst.part[1].value()};
-    block_reduce<2>(acc);
+    double acc[2];
+    block_reduce<2>(dst.part, acc);
     if (threadIdx.x == 0) {
       partials[kCntDot * 2 * kMaxPartials + blockIdx.x] = acc[0];
       partials[kCntDot * 2 * kMaxPartials + kMaxPartials + blockIdx.x] = acc[1];

@@ -43,81 +43,124 @@ struct FPair {
   __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
 
+// FP64 adds are the scarce resource of these reductions: GB300 starts about
+// two per clock and SM, so one warp-wide add occupies the SM's FP64 unit for
+// 16 clocks, and the ten of a warp's shuffle tree over two values, for every
+// warp of a block, cost more than the kernel's own work (degridding with the
+// norms of the l2 branch at 1024^2, M = 2^21: 98 us against 63 us without).
+// So the lanes of a warp are summed as float pairs by error-free TwoSum
+// merges (FP32 unit; the dropped terms are below 2^-47 of one warp's sum,
+// itself a 10^-3..10^-5 part of the total, i.e. at the rounding of an FP64
+// total), and only the sums across warps and blocks are FP64.  A warp that
+// holds a value which could overflow the pair (or is not finite) takes the
+// FP64 tree instead.
+constexpr float kPairMax = 1.2676506e30f;  // 2^100: 32 such values stay far below FP32's maximum
+
 // Tree over the first `valid` lanes of a warp whose first `present` lanes
 // exist (any block size, including a partial last warp); every present lane
 // calls it, and the result is valid in lane 0.
-template <bool MAX>
 __device__ __forceinline__ double warp_tree(double v, int lane, int present, int valid) {
   const unsigned mask = present >= 32 ? 0xffffffffu : ((1u << present) - 1u);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
+    if (o >= valid) continue;  // (uniform) nothing to add at this distance
     const double t = __shfl_down_sync(mask, v, o);
-    if (lane + o < valid) v = MAX ? fmax(v, t) : v + t;
+    if (lane + o < valid) v += t;
   }
   return v;
 }
 
-// Sum (or max) of NV values over the block; the result is valid in thread 0.
-template <int NV, bool MAX = false>
-__device__ __forceinline__ void block_reduce(double* v) {
+__device__ __forceinline__ double warp_tree(FPair v, int lane, int present, int valid) {
+  const unsigned mask = present >= 32 ? 0xffffffffu : ((1u << present) - 1u);
+  if (__any_sync(mask, !(fabsf(v.hi) < kPairMax))) return warp_tree(v.value(), lane, present, valid);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    if (o >= valid) continue;
+    const float h = __shfl_down_sync(mask, v.hi, o), l = __shfl_down_sync(mask, v.lo, o);
+    if (lane + o < valid) v.add(h, l);
+  }
+  return v.value();
+}
+
+// Sum of NV values (FPair or double) over the block; out is valid in thread 0.
+template <int NV, class V>
+__device__ __forceinline__ void block_reduce(const V* v, double* out) {
   __shared__ double sh[NV][32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int nw = (blockDim.x + 31) >> 5;
   const int mylanes = min(32, (int)blockDim.x - wid * 32);
 #pragma unroll
-  for (int k = 0; k < NV; ++k) v[k] = warp_tree<MAX>(v[k], lane, mylanes, mylanes);
+  for (int k = 0; k < NV; ++k) out[k] = warp_tree(v[k], lane, mylanes, mylanes);
   __syncthreads();
   if (lane == 0) {
 #pragma unroll
-    for (int k = 0; k < NV; ++k) sh[k][wid] = v[k];
+    for (int k = 0; k < NV; ++k) sh[k][wid] = out[k];
   }
   __syncthreads();
   if (wid == 0) {
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      const double t = lane < nw ? sh[k][lane] : 0.0;
-      v[k] = warp_tree<MAX>(t, lane, mylanes, nw);
-    }
+    for (int k = 0; k < NV; ++k) out[k] = warp_tree(lane < nw ? sh[k][lane] : 0.0, lane, mylanes, nw);
   }
+}
+
+// Largest of one float per thread, over the block (valid in thread 0; any
+// block size).
+__device__ __forceinline__ float block_max(float v) {
+  __shared__ float sh[32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int nw = (blockDim.x + 31) >> 5;
+  const int mylanes = min(32, (int)blockDim.x - wid * 32);
+  const unsigned mask = mylanes >= 32 ? 0xffffffffu : ((1u << mylanes) - 1u);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float t = __shfl_down_sync(mask, v, o);
+    if (lane + o < mylanes) v = fmaxf(v, t);
+  }
+  __syncthreads();
+  if (lane == 0) sh[wid] = v;
+  __syncthreads();
+  if (wid == 0)
+    for (int k = 0; k < nw; ++k) v = fmaxf(v, sh[k]);
+  return v;
+}
+
+// Takes a ticket after this block's thread 0 has written its partials; true
+// (in every thread) in the block that takes the last one.
+__device__ __forceinline__ bool last_block_ticket(unsigned int* counter, unsigned int nblk) {
+  __shared__ bool am_last;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    am_last = (atomicAdd(counter, 1u) == nblk - 1);
+  }
+  __syncthreads();
+  if (!am_last) return false;
+  __threadfence();
+  return true;
 }
 
 // Writes the block's NV partials, and in the last block to finish sums all
 // partials (fixed order) into total[0..NV).  Returns true in thread 0 of that
 // last block only.  partials holds NV x kMaxPartials doubles; the grid must
 // have at most kMaxPartials blocks.  The counter is reset for the next use.
-template <int NV, bool MAX = false>
-__device__ __forceinline__ bool reduce_last_block(double* v, double* partials, unsigned int* counter,
-                                                  double* total) {
-  __shared__ bool am_last;
+template <int NV, class V>
+__device__ __forceinline__ bool reduce_last_block(const V* v, double* partials, unsigned int* counter, double* total) {
   const unsigned int nblk = gridDim.x * gridDim.y * gridDim.z;
   const unsigned int bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-  block_reduce<NV, MAX>(v);
+  double acc[NV];
+  block_reduce<NV>(v, acc);
   if (threadIdx.x == 0) {
 #pragma unroll
-    for (int k = 0; k < NV; ++k) partials[k * kMaxPartials + bid] = v[k];
-    __threadfence();
-    const unsigned int ticket = atomicAdd(counter, 1u);
-    am_last = (ticket == nblk - 1);
+    for (int k = 0; k < NV; ++k) partials[k * kMaxPartials + bid] = acc[k];
   }
-  __syncthreads();
-  if (!am_last) return false;
-  __threadfence();
-  double acc[NV];
+  if (!last_block_ticket(counter, nblk)) return false;
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
     double s = 0.0;
-    for (unsigned int i = threadIdx.x; i < nblk; i += blockDim.x) {
-      const double t = __ldcg(&partials[k * kMaxPartials + i]);
-      s = MAX ? fmax(s, t) : s + t;
-    }
+    for (unsigned int i = threadIdx.x; i < nblk; i += blockDim.x) s += __ldcg(&partials[k * kMaxPartials + i]);
     acc[k] = s;
   }
-  block_reduce<NV, MAX>(acc);
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) total[k] = acc[k];
-    *counter = 0u;
-  }
+  block_reduce<NV>(acc, total);
+  if (threadIdx.x == 0) *counter = 0u;
   return threadIdx.x == 0;
 }
 
@@ -147,32 +190,44 @@ __device__ __forceinline__ CgStep cg_consume(const double* __restrict__ part, in
   if (nblk == 0) {  // formed by k_cg_scalars for this step (many partials)
     return CgStep{(float)sc->alpha, (float)sc->beta, sc->cg_step_first != 0};
   }
-  double v[2] = {0.0, 0.0};
-  for (int i = threadIdx.x; i < nblk; i += blockDim.x) {
-    v[0] += __ldcg(&part[i]);
-    v[1] += __ldcg(&part[kMaxPartials + i]);
-  }
-  block_reduce<2>(v);
-  if (threadIdx.x == 0) {
-    const double gamma = v[0], delta = v[1];
+  // the first warp adds the partials (fixed order) and forms the step sizes:
+  // one FP64 division each on lanes 0 and 1 while the partials arrive (the
+  // reciprocals of step j - 1's gamma and alpha), one after (gamma / den)
+  if (threadIdx.x < 32) {  // (blocks have at least two threads)
+    const int lane = threadIdx.x, present = min(32, (int)blockDim.x);
+    const unsigned mask = present >= 32 ? 0xffffffffu : ((1u << present) - 1u);
+    double v[2] = {0.0, 0.0};
     const int prev = (j - 1) & 1;
-    const double rho_p = j > 0 ? sc->cg_rho[prev] : 0.0, al_p = j > 0 ? sc->cg_alpha[prev] : 0.0;
-    const bool first = j == 0 || al_p == 0.0 || rho_p == 0.0;
-    const double beta = first ? 0.0 : gamma / rho_p;
-    const double den = first ? delta : delta - beta * gamma / al_p;
-    const double alpha = den > 0.0 ? gamma / den : 0.0;
-    s_al = (float)alpha;
-    s_be = (float)beta;
-    s_first = first ? 1 : 0;
-    if (blockIdx.x == 0) {
-      sc->cg_rho[j & 1] = gamma;
-      sc->cg_alpha[j & 1] = alpha;
-      sc->alpha = alpha;
-      sc->beta = beta;
-      sc->rho = gamma;
-      sc->pqp = den;
-      sc->cg_res = sqrt(gamma);
-      sc->cg_step_first = first ? 1 : 0;
+    double old = 0.0;  // gamma (even lanes) and alpha (odd lanes) of step j - 1
+    if (j > 0) old = (lane & 1) ? sc->cg_alpha[prev] : sc->cg_rho[prev];
+    for (int i = lane; i < nblk; i += present) {
+      v[0] += __ldcg(&part[i]);
+      v[1] += __ldcg(&part[kMaxPartials + i]);
+    }
+    const unsigned zero = __ballot_sync(mask, old == 0.0);
+    const double inv = 1.0 / old;
+    const double inv_al = __shfl_sync(mask, inv, 1);
+    v[0] = warp_tree(v[0], lane, present, min(present, nblk));
+    v[1] = warp_tree(v[1], lane, present, min(present, nblk));
+    if (lane == 0) {
+      const double gamma = v[0], delta = v[1];
+      const bool first = j == 0 || (zero & 3u) != 0u;
+      const double beta = first ? 0.0 : gamma * inv;
+      const double den = first ? delta : delta - beta * gamma * inv_al;
+      const double alpha = den > 0.0 ? gamma / den : 0.0;
+      s_al = (float)alpha;
+      s_be = (float)beta;
+      s_first = first ? 1 : 0;
+      if (blockIdx.x == 0) {
+        sc->cg_rho[j & 1] = gamma;
+        sc->cg_alpha[j & 1] = alpha;
+        sc->alpha = alpha;
+        sc->beta = beta;
+        sc->rho = gamma;
+        sc->pqp = den;
+        sc->cg_res = sqrt(gamma);
+        sc->cg_step_first = first ? 1 : 0;
+      }
     }
   }
   __syncthreads();

@@ -78,8 +78,9 @@ __global__ void k_dirac(const float2* __restrict__ x, float2* __restrict__ alpha
     else f1 += sara_prox(al, (size_t)j, pa, gamma);
   }
   if (MODE == kSaraProx) {
-    double f1d = (double)f1, tot;
-    if (reduce_last_block<1>(&f1d, partials + kCntF1 * 2 * kMaxPartials, &sc->counter[kCntF1], &tot))
+    const FPair f1p{f1, 0.f};
+    double tot;
+    if (reduce_last_block<1>(&f1p, partials + kCntF1 * 2 * kMaxPartials, &sc->counter[kCntF1], &tot))
       sc->f1 = tot;  // first contribution of this analysis
   }
 }
@@ -288,8 +289,9 @@ __global__ void __launch_bounds__(256) k_dwt_level(const float2* __restrict__ in
   }
   if (MODE == kSaraProx) {
     // this block's f1 partial; the first synthesis launch adds them all up
-    double f1d = (double)f1;
-    block_reduce<1>(&f1d);
+    const FPair f1p{f1, 0.f};
+    double f1d;
+    block_reduce<1>(&f1p, &f1d);
     if (threadIdx.x == 0)
       partials[kCntF1 * 2 * kMaxPartials + G.f1_off + blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)] =
           f1d;
@@ -314,8 +316,9 @@ __device__ __forceinline__ void sara_f1_finish(const double* __restrict__ part, 
     for (int u = 0; u < U; ++u) a[u] += t[u];
   }
   for (; i < n; i += nt) a[0] += __ldcg(&part[i]);
-  double v = ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
-  block_reduce<1>(&v);
+  const double mine = ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
+  double v;
+  block_reduce<1>(&mine, &v);
   if (threadIdx.x == 0) {
     sc->f1 = v;
     const double prev = sc->f1_prev;

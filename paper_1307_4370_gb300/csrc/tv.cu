@@ -129,8 +129,8 @@ __global__ void k_tv_finish(int n, const float2* __restrict__ b, const float2* _
     f1.add_prod(w ? w[k] : 1.0f, mag);
   }
   if (!z1) return;
-  double v = f1.value(), tot;
-  if (reduce_last_block<1>(&v, partials + kCntF1 * 2 * kMaxPartials, &sc->counter[kCntF1], &tot)) {
+  double tot;
+  if (reduce_last_block<1>(&f1, partials + kCntF1 * 2 * kMaxPartials, &sc->counter[kCntF1], &tot)) {
     sc->f1 = tot;
     const double prev = sc->f1_prev;
     sc->zeta = (prev != 0.0) ? fabs(tot - prev) / fabs(prev) : INFINITY;

@@ -42,8 +42,8 @@ __global__ void k_norm_diff(int64_t n, const float2* __restrict__ a, const float
     part.add_sq_diff(a[j].x, b[j].x);
     part.add_sq_diff(a[j].y, b[j].y);
   }
-  double acc = part.value(), tot;
-  if (reduce_last_block<1>(&acc, partials + kCntNorm * 2 * kMaxPartials, &sc->counter[kCntNorm], &tot))
+  double tot;
+  if (reduce_last_block<1>(&part, partials + kCntNorm * 2 * kMaxPartials, &sc->counter[kCntNorm], &tot))
     sc->norm2 = tot;
 }
 
@@ -96,8 +96,8 @@ __global__ void k_cg_apply(int64_t n, float2* __restrict__ x, float2* __restrict
     part.add_prod(rn.x, rn.x);
     part.add_prod(rn.y, rn.y);
   }
-  double acc = part.value(), tot;
-  if (reduce_last_block<1>(&acc, partials + kCntRho * 2 * kMaxPartials, &sc->counter[kCntRho], &tot))
+  double tot;
+  if (reduce_last_block<1>(&part, partials + kCntRho * 2 * kMaxPartials, &sc->counter[kCntRho], &tot))
     sc->cg_res = sqrt(tot);  // recurrence residual after the last update
 }
 
@@ -111,9 +111,18 @@ __global__ void k_cg_residual_init(int64_t n, const float2* __restrict__ b, cons
 __global__ void k_max_abs(int64_t n, const float2* __restrict__ a, double* partials, DevScalars* sc) {
   float mf = 0.f;
   GRID_STRIDE(j, n) mf = fmaxf(mf, sqrtf(fmaf(a[j].x, a[j].x, a[j].y * a[j].y)));
-  double m = (double)mf, tot;
-  if (reduce_last_block<1, true>(&m, partials + kCntMax * 2 * kMaxPartials, &sc->counter[kCntMax], &tot))
-    sc->amax = tot;
+  // (the maximum of FP32 moduli is one of them: no FP64 needed before the last store)
+  partials += kCntMax * 2 * kMaxPartials;
+  mf = block_max(mf);
+  if (threadIdx.x == 0) partials[blockIdx.x] = (double)mf;
+  if (!last_block_ticket(&sc->counter[kCntMax], gridDim.x)) return;
+  float t = 0.f;
+  for (unsigned int i = threadIdx.x; i < gridDim.x; i += blockDim.x) t = fmaxf(t, (float)__ldcg(&partials[i]));
+  t = block_max(t);
+  if (threadIdx.x == 0) {
+    sc->amax = (double)t;
+    sc->counter[kCntMax] = 0u;
+  }
 }
 
 // SDMM l2 branch (Algorithm 1 steps 7-9, i = 2) after the degridding kernel
@@ -150,7 +159,7 @@ __global__ void k_sdmm_l2(int64_t M, const float2* __restrict__ s2, float2* __re
 // caller-order visibilities, ||s2_i + z2_i - y_i||^2 and ||s2_i - y_i||^2
 // (gathered through the sorted positions; exact FP32 terms, FP64 sums).  One
 // CTA per chunk of a block; the last CTA to finish adds each block's chunk
-// partials in chunk order and forms its ball factor min(1, eps_i / ||.||) and
+// partials in a fixed order and forms its ball factor min(1, eps_i / ||.||) and
 // nu_i = ||y_i - Phi_i x_hat|| / eps_i (nu = the largest, nu_min the smallest).
 __global__ void __launch_bounds__(256) k_block_norms(const int4* __restrict__ bchunks, int nbchunks,
                                                      const int* __restrict__ pos, const float2* __restrict__ s2,
@@ -159,7 +168,6 @@ __global__ void __launch_bounds__(256) k_block_norms(const int4* __restrict__ bc
                                                      const float* __restrict__ yscale, int R,
                                                      const double* __restrict__ beps, float* __restrict__ bscale,
                                                      double* partials, DevScalars* sc) {
-  __shared__ bool am_last;
   const int4 ch = bchunks[blockIdx.x];
   FPair part[2];
   for (int m = ch.y + threadIdx.x; m < ch.z; m += blockDim.x) {
@@ -179,34 +187,42 @@ __global__ void __launch_bounds__(256) k_block_norms(const int4* __restrict__ bc
     part[1].add_sq_diff(s.x, yy.x);
     part[1].add_sq_diff(s.y, yy.y);
   }
-  double v[2] = {part[0].value(), part[1].value()};
-  block_reduce<2>(v);
+  double v[2];
+  block_reduce<2>(part, v);
   if (threadIdx.x == 0) {
     partials[blockIdx.x] = v[0];
     partials[kMaxPartials + blockIdx.x] = v[1];
-    __threadfence();
-    am_last = atomicAdd(&sc->counter[kCntBlk], 1u) == (unsigned)(gridDim.x - 1);
   }
-  __syncthreads();
-  if (!am_last) return;
-  __threadfence();
+  if (!last_block_ticket(&sc->counter[kCntBlk], gridDim.x)) return;
+  __shared__ double s_nu[2][32];
   double numax = 0.0, numin = INFINITY;
-  for (int b = threadIdx.x; b < R; b += blockDim.x) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;  // 256 threads
+  // few blocks: a warp per block, a chunk per lane (one thread walking its 57
+  // chunks, four blocks of 235 k visibilities, kept the kernel at 57 us, each
+  // load behind the previous add); many: a thread per block
+  const bool by_warp = R <= 64;
+  const int nper = by_warp ? nw : (int)blockDim.x, me = by_warp ? wid : (int)threadIdx.x;
+  for (int b = me; b < R; b += nper) {
     // chunks of block b: from its first chunk up to the next block's first
-    int k0 = 0;
-    {
-      int lo = 0, hi = nbchunks;  // first chunk whose block is >= b
+    auto first_of = [&](int want) {  // first chunk whose block is >= want
+      int lo = 0, hi = nbchunks;
       while (lo < hi) {
         const int mid = (lo + hi) >> 1;
-        if (bchunks[mid].x < b) lo = mid + 1;
+        if (bchunks[mid].x < want) lo = mid + 1;
         else hi = mid;
       }
-      k0 = lo;
-    }
+      return lo;
+    };
+    const int k0 = first_of(b), k1 = first_of(b + 1);
     double dn2 = 0.0, res2 = 0.0;
-    for (int k = k0; k < nbchunks && bchunks[k].x == b; ++k) {
+    for (int k = k0 + (by_warp ? lane : 0); k < k1; k += by_warp ? 32 : 1) {
       dn2 += __ldcg(&partials[k]);
       res2 += __ldcg(&partials[kMaxPartials + k]);
+    }
+    if (by_warp) {
+      dn2 = warp_tree(dn2, lane, 32, 32);
+      res2 = warp_tree(res2, lane, 32, 32);
+      if (lane > 0) continue;
     }
     const double e = beps[b];
     const double nd = sqrt(dn2);
@@ -215,12 +231,23 @@ __global__ void __launch_bounds__(256) k_block_norms(const int4* __restrict__ bc
     numax = fmax(numax, nu);
     numin = fmin(numin, nu);
   }
-  double mx[1] = {numax}, mn[1] = {-numin};
-  block_reduce<1, true>(mx);
-  block_reduce<1, true>(mn);
+  __syncwarp();
+  for (int o = 16; o > 0; o >>= 1) {
+    numax = fmax(numax, __shfl_xor_sync(0xffffffffu, numax, o));
+    numin = fmin(numin, __shfl_xor_sync(0xffffffffu, numin, o));
+  }
+  if (lane == 0) {
+    s_nu[0][wid] = numax;
+    s_nu[1][wid] = numin;
+  }
+  __syncthreads();
   if (threadIdx.x == 0) {
-    sc->nu = mx[0];
-    sc->nu_min = -mn[0];
+    for (int k = 1; k < nw; ++k) {
+      numax = fmax(numax, s_nu[0][k]);
+      numin = fmin(numin, s_nu[1][k]);
+    }
+    sc->nu = numax;
+    sc->nu_min = numin;
     sc->counter[kCntBlk] = 0u;
   }
 }
@@ -228,8 +255,13 @@ __global__ void __launch_bounds__(256) k_block_norms(const int4* __restrict__ bc
 // Reweighting (§3.3): w = delta / (delta + |alpha|).
 __global__ void k_reweight(int64_t n, const float2* __restrict__ alpha, float* __restrict__ w, int round,
                            const DevScalars* sc) {
-  const double amax = sc->amax;
-  const float delta = (float)fmax(pow(10.0, -(double)round) * amax, 1e-6 * amax);
+  __shared__ float s_delta;  // one FP64 power per block (every thread forming it held the kernel at 86 us, 256^2)
+  if (threadIdx.x == 0) {
+    const double amax = sc->amax;
+    s_delta = (float)fmax(pow(10.0, -(double)round) * amax, 1e-6 * amax);
+  }
+  __syncthreads();
+  const float delta = s_delta;
   GRID_STRIDE(j, n) {
     if (delta == 0.f) {
       w[j] = 1.0f;
