@@ -423,8 +423,8 @@ void purify_batch_destroy(purify_batch* batch);
  * (y, w, z2) are in the caller's order of the context's uv.  omega (D
  * float32) are the weights of f1, w (M float32) the visibility weights.
  * Complex entries are treated as real pairs (§4.1): the adjoint of an entry
- * is dL/dRe + i dL/dIm.  The calls synchronise `stream` (the CG step sizes
- * are formed on the host in FP64).  cg_iters is 0..64. */
+ * is dL/dRe + i dL/dIm.  The calls synchronise `stream`; the CG step sizes
+ * are formed on the device in FP64 and kept on the tape.  cg_iters is 0..64. */
 
 /* gamma = beta ||Psi^H Phi_w^H y_w||_inf (§4.4's rule for the weighted
  * problem) into *gamma (host).  y, wvis: M entries (device, caller order). */

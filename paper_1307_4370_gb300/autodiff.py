@@ -11,7 +11,7 @@
   per-visibility weights w (Phi_w = diag(w) Phi, y_w = diag(w) y; the
   weighting matrices §5 says fold into the measurement operator) and SARA
   weights omega.  Each iteration is the library's purify_diff_iteration
-  (CUDA kernels; the CG step sizes in FP64 on the host) and its backward
+  (CUDA kernels, the CG step sizes among them, in FP64) and its backward
   the library's purify_diff_iteration_vjp: CG reversed from the step sizes
   and vectors on the tape, and the Jacobians of the soft threshold, the
   l2-ball projection and the positivity projection.  The forward keeps the

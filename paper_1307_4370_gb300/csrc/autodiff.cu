@@ -5,7 +5,8 @@
 // run forward with a tape, and its vector-Jacobian product (reverse mode)
 // from that tape.  Every vector operation is a kernel of this file or one of
 // the library's operators (Phi, Phi^H, Psi, Psi^H); the scalar recurrences
-// of CG (a few doubles per step) run on the host.
+// of CG run on the device, in the last blocks of the kernels that form the
+// inner products (FP64), and stay on the tape.
 //
 // Forward, from the input state S = (x_hat, z1, z2, z3, x1, x2, x3), as the
 // oracle's Algorithm 1 steps 5-9 with S = 3:
@@ -33,6 +34,27 @@ namespace {
 
 unsigned dblocks(int64_t n) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 2048)); }
 
+// Header of the device tape: the scalars of the iteration, written and read
+// by the kernels (no inner product goes through the host: one read and
+// synchronisation per product kept the 256^2 gradient at 24 ms).
+struct TapeHeader {
+  double alpha[64], beta[64], rho[65], pi[64];
+  double nd;      // ||a2 - y_w||
+  double cball;   // min(1, eps / nd)
+  int32_t steps;  // CG steps run (rho = 0 ends the solve)
+  int32_t k;
+};
+
+// Scalars of the reverse pass that one kernel leaves for the next.
+struct BwdScalars {
+  double rhob;   // adjoint of rho_{j+1}, complete
+  double rhobn;  // adjoint of rho_j without the step below's term
+  double betab;  // adjoint of beta_j
+  double xp;     // <x_bar, p_j>
+  double pib;    // adjoint of pi_j
+  double k2;     // c <d, rbar2> / ||d||^2 of the ball's Jacobian
+};
+
 // ---------------------------------------------------------------------------
 // Elementwise and reduction kernels
 // ---------------------------------------------------------------------------
@@ -57,23 +79,10 @@ __global__ void k_dot(int64_t n, const float2* __restrict__ a, const float2* __r
   if (reduce_last_block<1>(&part, partials, counter, &tot)) *out = tot;
 }
 
-// ||a - w o y||^2 in FP64 -> *out
-__global__ void k_norm_wdiff(int64_t n, const float2* __restrict__ a, const float* __restrict__ w,
-                             const float2* __restrict__ y, double* partials, unsigned* counter, double* out) {
-  FPair part;
-  DGRID(i, n) {
-    const float2 d = csub(a[i], cscale(y[i], w[i]));
-    part.add_prod(d.x, d.x);
-    part.add_prod(d.y, d.y);
-  }
-  double tot;
-  if (reduce_last_block<1>(&part, partials, counter, &tot)) *out = tot;
-}
-
-// Re <a - w o y, r> in FP64 -> *out
+// Re <a - w o y, r> in FP64, and from it k2 = c <d, rbar2> / ||d||^2
 __global__ void k_dot_wdiff(int64_t n, const float2* __restrict__ a, const float* __restrict__ w,
                             const float2* __restrict__ y, const float2* __restrict__ r, double* partials,
-                            unsigned* counter, double* out) {
+                            unsigned* counter, const TapeHeader* __restrict__ H, BwdScalars* S) {
   FPair part;
   DGRID(i, n) {
     const float2 d = csub(a[i], cscale(y[i], w[i]));
@@ -81,7 +90,7 @@ __global__ void k_dot_wdiff(int64_t n, const float2* __restrict__ a, const float
     part.add_prod(d.y, r[i].y);
   }
   double tot;
-  if (reduce_last_block<1>(&part, partials, counter, &tot)) *out = tot;
+  if (reduce_last_block<1>(&part, partials, counter, &tot)) S->k2 = H->cball * tot / (H->nd * H->nd);
 }
 
 // out = a + b + c
@@ -90,33 +99,70 @@ __global__ void k_sum3(int64_t n, const float2* __restrict__ a, const float2* __
   DGRID(i, n) out[i] = cadd(cadd(a[i], b[i]), c[i]);
 }
 
-// out = u - (v + 2 p): the residual b - Q x0 with v = Phi_w^H Phi_w x0
+// r0 = p0 = u - (v + 2 x0): the residual b - Q x0 with v = Phi_w^H Phi_w x0;
+// rho_0 = <r0, r0> into the (zeroed) header
 __global__ void k_resid0(int64_t n, const float2* __restrict__ u, const float2* __restrict__ v,
-                         const float2* __restrict__ p, float2* __restrict__ out, float2* __restrict__ out2) {
+                         const float2* __restrict__ x, float2* __restrict__ r0, float2* __restrict__ p0, int k,
+                         double* partials, unsigned* counter, TapeHeader* H) {
+  FPair part;
   DGRID(i, n) {
-    const float2 r = make_float2(u[i].x - v[i].x - 2.f * p[i].x, u[i].y - v[i].y - 2.f * p[i].y);
-    out[i] = r;
-    if (out2) out2[i] = r;
+    const float2 r = make_float2(u[i].x - v[i].x - 2.f * x[i].x, u[i].y - v[i].y - 2.f * x[i].y);
+    r0[i] = r;
+    if (p0) p0[i] = r;
+    part.add_prod(r.x, r.x);
+    part.add_prod(r.y, r.y);
+  }
+  double tot;
+  if (reduce_last_block<1>(&part, partials, counter, &tot)) {
+    H->rho[0] = tot;
+    H->k = k;
   }
 }
 
-// q = v + 2 p (Q_w p from v = Phi_w^H Phi_w p)
-__global__ void k_plus2(int64_t n, const float2* __restrict__ v, const float2* __restrict__ p, float2* __restrict__ q) {
-  DGRID(i, n) q[i] = make_float2(fmaf(2.f, p[i].x, v[i].x), fmaf(2.f, p[i].y, v[i].y));
-}
-
-// x += alpha p; r_next = r - alpha q
-__global__ void k_cg_upd(int64_t n, float alpha, float2* __restrict__ x, const float2* __restrict__ p,
-                         const float2* __restrict__ r, const float2* __restrict__ q, float2* __restrict__ rn) {
+// CG step j after q = Q_w p left the block partials of pi_j = <q, p> (pqpart):
+// alpha_j = rho_j / pi_j (every block forms it, in the same order);
+// x += alpha p; r_{j+1} = r - alpha q; rho_{j+1} = <r_{j+1}, r_{j+1}>, beta_j.
+// rho_j = 0 ends the solve: nothing changes from there on.
+__global__ void k_cg_upd(int64_t n, const double* __restrict__ pqpart, int npq, int j, float2* __restrict__ x,
+                         const float2* __restrict__ p, const float2* __restrict__ r, const float2* __restrict__ q,
+                         float2* __restrict__ rn, double* partials, unsigned* counter, TapeHeader* H) {
+  __shared__ float s_alpha;
+  const double rho = H->rho[j];
+  if (threadIdx.x < 32) {
+    double v = 0.0;
+    for (int i = threadIdx.x; i < npq; i += 32) v += __ldcg(&pqpart[i]);
+    v = warp_tree(v, threadIdx.x, 32, 32);
+    if (threadIdx.x == 0) {
+      const double alpha = v > 0.0 && rho != 0.0 ? rho / v : 0.0;
+      s_alpha = (float)alpha;
+      if (blockIdx.x == 0) {
+        H->alpha[j] = alpha;
+        H->pi[j] = v;
+      }
+    }
+  }
+  __syncthreads();
+  const float alpha = s_alpha;
+  FPair part;
   DGRID(i, n) {
     x[i] = make_float2(fmaf(alpha, p[i].x, x[i].x), fmaf(alpha, p[i].y, x[i].y));
-    rn[i] = make_float2(fmaf(-alpha, q[i].x, r[i].x), fmaf(-alpha, q[i].y, r[i].y));
+    const float2 t = make_float2(fmaf(-alpha, q[i].x, r[i].x), fmaf(-alpha, q[i].y, r[i].y));
+    rn[i] = t;
+    part.add_prod(t.x, t.x);
+    part.add_prod(t.y, t.y);
+  }
+  double tot;
+  if (reduce_last_block<1>(&part, partials, counter, &tot)) {
+    H->rho[j + 1] = tot;
+    H->beta[j] = rho != 0.0 ? tot / rho : 0.0;
+    if (rho != 0.0) H->steps = j + 1;
   }
 }
 
-// p_next = r + beta p
-__global__ void k_cg_dir(int64_t n, float beta, const float2* __restrict__ r, const float2* __restrict__ p,
-                         float2* __restrict__ pn) {
+// p_{j+1} = r_{j+1} + beta_j p_j
+__global__ void k_cg_dir(int64_t n, const TapeHeader* __restrict__ H, int j, const float2* __restrict__ r,
+                         const float2* __restrict__ p, float2* __restrict__ pn) {
+  const float beta = (float)H->beta[j];
   DGRID(i, n) pn[i] = make_float2(fmaf(beta, p[i].x, r[i].x), fmaf(beta, p[i].y, r[i].y));
 }
 
@@ -137,17 +183,33 @@ __global__ void k_b1_fwd(int64_t n, float2* __restrict__ a1, const float2* __res
   }
 }
 
-// i = 2 forward, first half: a2 = w o s + z2 (s = Phi x_hat')
+// i = 2 forward, first half: a2 = w o s + z2 (s = Phi x_hat'), ||a2 - y_w|| and
+// the ball factor into the header
 __global__ void k_b2_a(int64_t n, const float2* __restrict__ s, const float* __restrict__ w,
-                       const float2* __restrict__ z2, float2* __restrict__ a2) {
-  DGRID(i, n) a2[i] = cadd(cscale(s[i], w[i]), z2[i]);
+                       const float2* __restrict__ z2, const float2* __restrict__ y, float2* __restrict__ a2,
+                       double eps, double* partials, unsigned* counter, TapeHeader* H) {
+  FPair part;
+  DGRID(i, n) {
+    const float2 a = cadd(cscale(s[i], w[i]), z2[i]);
+    a2[i] = a;
+    const float2 d = csub(a, cscale(y[i], w[i]));
+    part.add_prod(d.x, d.x);
+    part.add_prod(d.y, d.y);
+  }
+  double tot;
+  if (reduce_last_block<1>(&part, partials, counter, &tot)) {
+    const double nd = sqrt(tot);
+    H->nd = nd;
+    H->cball = nd > eps ? eps / nd : 1.0;
+  }
 }
 
 // i = 2 forward, second half: r2 = y_w + c (a2 - y_w), z2' = a2 - r2,
 // u2 = 2 r2 - a2, and t = w o u2 (gridded next)
 __global__ void k_b2_b(int64_t n, const float2* __restrict__ a2, const float* __restrict__ w,
-                       const float2* __restrict__ y, float c, float2* __restrict__ z2o, float2* __restrict__ u2,
-                       float2* __restrict__ t) {
+                       const float2* __restrict__ y, const TapeHeader* __restrict__ H, float2* __restrict__ z2o,
+                       float2* __restrict__ u2, float2* __restrict__ t) {
+  const float c = (float)H->cball;
   DGRID(i, n) {
     const float2 yw = cscale(y[i], w[i]);
     const float2 d = csub(a2[i], yw);
@@ -277,9 +339,10 @@ __global__ void k_b2_bwd1(int64_t n, const float2* __restrict__ g, const float* 
 // s2 = w o Phi x_hat': sbar2 = abar2, w_bar += Re(conj(Phi x_hat') abar2),
 // z2bar = abar2, t = w o abar2 (gridded into x_bar next)
 __global__ void k_b2_bwd2(int64_t n, const float2* __restrict__ a2, const float* __restrict__ w,
-                          const float2* __restrict__ y, int outside, float c, float k2, const float2* __restrict__ rb,
-                          float2* __restrict__ ab, const float2* __restrict__ phx, float* __restrict__ wb,
+                          const float2* __restrict__ y, int outside, float c, const BwdScalars* __restrict__ S,
+                          const float2* __restrict__ rb, float2* __restrict__ ab, const float2* __restrict__ phx, float* __restrict__ wb,
                           float2* __restrict__ z2b_i, float2* __restrict__ t) {
+  const float k2 = outside ? (float)S->k2 : 0.f;
   DGRID(i, n) {
     const float2 yw = cscale(y[i], w[i]);
     float2 db, cbar;
@@ -298,31 +361,77 @@ __global__ void k_b2_bwd2(int64_t n, const float2* __restrict__ a2, const float*
   }
 }
 
-// w_bar += f w o Re(conj(g) h) (the weights' term of <qbar, Q_w p>)
-__global__ void k_wbar_q(int64_t n, float f, const float* __restrict__ w, const float2* __restrict__ g,
-                         const float2* __restrict__ h, float* __restrict__ wb) {
-  DGRID(i, n) wb[i] += f * w[i] * (g[i].x * h[i].x + g[i].y * h[i].y);
+// <x_bar, p> for the last step run, before the reverse CG (S is zeroed first)
+__global__ void k_cgb_first(int64_t n, const float2* __restrict__ xb, const float2* __restrict__ p, double* partials,
+                            unsigned* counter, BwdScalars* S) {
+  FPair part;
+  DGRID(i, n) {
+    part.add_prod(xb[i].x, p[i].x);
+    part.add_prod(xb[i].y, p[i].y);
+  }
+  double tot;
+  if (reduce_last_block<1>(&part, partials, counter, &tot)) S->xp = tot;
 }
 
-// r_bar += p_bar + 2 rho_bar r
-__global__ void k_cgb_r(int64_t n, float2* __restrict__ rb, const float2* __restrict__ pb, float tr,
-                        const float2* __restrict__ r) {
-  DGRID(i, n) rb[i] = make_float2(rb[i].x + pb[i].x + tr * r[i].x, rb[i].y + pb[i].y + tr * r[i].y);
+// r_bar += p_bar + 2 rho_bar r; with q (step j): <r_bar, q_j> and from it the
+// adjoints of alpha_j, pi_j and rho_j
+__global__ void k_cgb_r(int64_t n, float2* __restrict__ rb, const float2* __restrict__ pb,
+                        const float2* __restrict__ r, const float2* __restrict__ q, int j, double* partials,
+                        unsigned* counter, const TapeHeader* __restrict__ H, BwdScalars* S) {
+  const float tr = (float)(2.0 * S->rhob);
+  FPair part;
+  DGRID(i, n) {
+    const float2 t = make_float2(rb[i].x + pb[i].x + tr * r[i].x, rb[i].y + pb[i].y + tr * r[i].y);
+    rb[i] = t;
+    if (q) {
+      part.add_prod(t.x, q[i].x);
+      part.add_prod(t.y, q[i].y);
+    }
+  }
+  if (!q) return;
+  double rq;
+  if (reduce_last_block<1>(&part, partials, counter, &rq)) {
+    const double rho = H->rho[j], rho1 = H->rho[j + 1], pq = H->pi[j];
+    const double alb = pq > 0.0 ? -rq + S->xp : 0.0;
+    S->rhobn = -S->betab * rho1 / (rho * rho) + (pq > 0.0 ? alb / pq : 0.0);
+    S->pib = pq > 0.0 ? -alb * rho / (pq * pq) : 0.0;
+  }
 }
 
 // q_bar = -alpha r_bar + pi_bar p
-__global__ void k_cgb_q(int64_t n, float alpha, const float2* __restrict__ rb, float pib, const float2* __restrict__ p,
-                        float2* __restrict__ qb) {
+__global__ void k_cgb_q(int64_t n, const TapeHeader* __restrict__ H, const BwdScalars* __restrict__ S, int j,
+                        const float2* __restrict__ rb, const float2* __restrict__ p, float2* __restrict__ qb) {
+  const float alpha = (float)H->alpha[j], pib = (float)S->pib;
   DGRID(i, n) qb[i] = make_float2(fmaf(-alpha, rb[i].x, pib * p[i].x), fmaf(-alpha, rb[i].y, pib * p[i].y));
 }
 
-// p_bar = beta p_bar + alpha x_bar + pi_bar q + (v + 2 q_bar), v = Phi_w^H Phi_w q_bar
-__global__ void k_cgb_p(int64_t n, float beta, float2* __restrict__ pb, float alpha, const float2* __restrict__ xb,
-                        float pib, const float2* __restrict__ q, const float2* __restrict__ v,
-                        const float2* __restrict__ qb) {
+// p_bar = beta p_bar + alpha x_bar + pi_bar q + (v + 2 q_bar), v = Phi_w^H Phi_w q_bar;
+// with pprev = p_{j-1}: beta_bar_{j-1} = <p_bar, p_{j-1}>, <x_bar, p_{j-1}> and
+// the rest of rho_j's adjoint for the step below
+__global__ void k_cgb_p(int64_t n, const TapeHeader* __restrict__ H, int j, float2* __restrict__ pb,
+                        const float2* __restrict__ xb, const float2* __restrict__ q, const float2* __restrict__ v,
+                        const float2* __restrict__ qb, const float2* __restrict__ pprev, double* partials,
+                        unsigned* counter, BwdScalars* S) {
+  const float beta = (float)H->beta[j], alpha = (float)H->alpha[j], pib = (float)S->pib;
+  FPair part[2];
   DGRID(i, n) {
-    pb[i] = make_float2(beta * pb[i].x + alpha * xb[i].x + pib * q[i].x + v[i].x + 2.f * qb[i].x,
-                        beta * pb[i].y + alpha * xb[i].y + pib * q[i].y + v[i].y + 2.f * qb[i].y);
+    const float2 x = xb[i];
+    const float2 t = make_float2(beta * pb[i].x + alpha * x.x + pib * q[i].x + v[i].x + 2.f * qb[i].x,
+                                 beta * pb[i].y + alpha * x.y + pib * q[i].y + v[i].y + 2.f * qb[i].y);
+    pb[i] = t;
+    if (pprev) {
+      const float2 p = pprev[i];
+      part[0].add_prod(t.x, p.x);
+      part[0].add_prod(t.y, p.y);
+      part[1].add_prod(x.x, p.x);
+      part[1].add_prod(x.y, p.y);
+    }
+  }
+  double tot[2];
+  if (reduce_last_block<2>(part, partials, counter, tot)) {
+    S->betab = tot[0];
+    S->xp = tot[1];
+    S->rhob = pprev ? S->rhobn + tot[0] / H->rho[j - 1] : S->rhobn;
   }
 }
 
@@ -350,14 +459,6 @@ __global__ void k_add(int64_t n, const float2* __restrict__ a, const float2* __r
 int64_t nN(const purify_ctx* c) { return (int64_t)c->n * c->n; }
 int64_t nD(const purify_ctx* c) { return (int64_t)c->q * c->n * c->n; }
 
-// Tape layout (device): a header of doubles, then complex vectors.
-struct TapeHeader {
-  double alpha[64], beta[64], rho[65], pi[64];
-  double nd;      // ||a2 - y_w||
-  double cball;   // min(1, eps / nd)
-  int32_t steps;  // CG steps run
-  int32_t k;
-};
 constexpr size_t kHdr = (sizeof(TapeHeader) + 255) / 256 * 256;
 
 struct Tape {
@@ -389,11 +490,12 @@ size_t tape_bytes(const purify_ctx* c, int k) {
 }
 
 // Scratch of the differentiation calls (allocated on first use): three
-// visibility-size and four image-size complex vectors, one coefficient-size.
-int diff_scratch(purify_ctx* c, float2** m, float2** im, float2** dv) {
+// visibility-size and four image-size complex vectors, one coefficient-size,
+// and the scalars of the reverse pass.
+int diff_scratch(purify_ctx* c, float2** m, float2** im, float2** dv, BwdScalars** bs = nullptr) {
   const int64_t N = nN(c), M = c->M, D = nD(c);
   if (!c->d_diff) {
-    if (cudaMalloc((void**)&c->d_diff, (size_t)(3 * M + 4 * N + D) * sizeof(float2)) != cudaSuccess) {
+    if (cudaMalloc((void**)&c->d_diff, (size_t)(3 * M + 4 * N + D) * sizeof(float2) + sizeof(BwdScalars)) != cudaSuccess) {
       cudaGetLastError();
       c->d_diff = nullptr;
       return PURIFY_E_ALLOC;
@@ -402,6 +504,7 @@ int diff_scratch(purify_ctx* c, float2** m, float2** im, float2** dv) {
   for (int i = 0; i < 3; ++i) m[i] = c->d_diff + i * M;
   for (int i = 0; i < 4; ++i) im[i] = c->d_diff + 3 * M + i * N;
   *dv = c->d_diff + 3 * M + 4 * N;
+  if (bs) *bs = reinterpret_cast<BwdScalars*>(c->d_diff + 3 * M + 4 * N + D);
   return PURIFY_OK;
 }
 
@@ -440,12 +543,24 @@ int host_dot(purify_ctx* c, int64_t n, const float2* a, const float2* b, double*
     if (int _rc = check_cuda(cudaGetLastError())) return _rc; \
   } while (0)
 
-// v = Phi_w^H Phi_w p (without the 2p); g (M) receives Phi p, t (M) is scratch
-int apply_ww(purify_ctx* c, const float2* p, const float* w, float2* g, float2* t, float2* v, cudaStream_t s) {
-  const int64_t M = c->M;
-  if (int rc = phi_into(c, p, g, s)) return rc;
-  LAUNCH((k_wmul<<<dblocks(M), 256, 0, s>>>(M, g, w, 2, t)));
-  return phi_adj_into(c, t, v, s);
+// Phi_w^H Phi_w p: the degridding leaves g = Phi p (caller order, may be
+// NULL), w^2 g in sorted order (t, gridded next) and, with wb, the weights'
+// adjoint wb += hf w Re(conj(g) h); `ra` is the last row pass's output
+int apply_ww(purify_ctx* c, const float2* p, const float* w, float2* g, float2* t, RowOutMode mode,
+             const RowOutArgs& ra, cudaStream_t s, const float2* h = nullptr, float hf = 0.f, float* wb = nullptr) {
+  RowInArgs ia{};
+  ia.in = p;
+  if (int rc = phi_forward_grid(c, kRowInPlain, ia, s)) return rc;
+  DegridArgs da{};
+  da.out = g;
+  da.w = w;
+  da.t = t;
+  da.h = h;
+  da.hf = hf;
+  da.wb = wb;
+  if (int rc = degrid(c, kDegridWeighted, da, s)) return rc;
+  if (int rc = grid_adjoint(c, kGridSorted, t, s)) return rc;
+  return phi_adjoint_image(c, mode, ra, s);
 }
 
 struct DiffArgs {
@@ -476,45 +591,37 @@ int diff_forward(purify_ctx* c, const DiffArgs& A, float2* const* in, float2* co
   if (int rc = diff_scratch(c, m, im, &dv)) return rc;
   if (!tape_mem) return PURIFY_E_INVALID_ARG;  // the forward keeps its vectors on the tape
   Tape T = tape_views(c, k, tape_mem);
-  TapeHeader H;
-  std::memset(&H, 0, sizeof(H));
-  H.k = k;
+  TapeHeader* H = static_cast<TapeHeader*>(tape_mem);  // (device)
+  double* part = c->d_partials + kCntNorm * 2 * kMaxPartials;
+  unsigned* cnt = &c->d_sc->counter[kCntNorm];
+  if (int rc = check_cuda(cudaMemsetAsync(tape_mem, 0, sizeof(TapeHeader), s))) return rc;
   // ---- step 5: b = x1 + x2 + x3; r0 = b - Q_w x0; CG from x0 = x_hat
   float2* b = im[0];
   float2* x = out[0];
   LAUNCH((k_sum3<<<dblocks(N), 256, 0, s>>>(N, in[4], in[5], in[6], b)));
   if (int rc = check_cuda(cudaMemcpyAsync(x, in[0], N * sizeof(float2), cudaMemcpyDeviceToDevice, s))) return rc;
-  if (int rc = apply_ww(c, x, A.w, T.PhiX0, m[0], im[1], s)) return rc;
-  LAUNCH((k_resid0<<<dblocks(N), 256, 0, s>>>(N, b, im[1], x, T.R, T.P)));
-  double rho;
-  if (int rc = host_dot(c, N, T.R, T.R, &rho, s)) return rc;
-  H.rho[0] = rho;
-  int steps = 0;
-  for (int j = 0; j < k; ++j) {
-    if (rho == 0.0) break;  // as the oracle: nothing left to do
+  RowOutArgs ra{};
+  ra.out = im[1];
+  if (int rc = apply_ww(c, x, A.w, T.PhiX0, m[0], kRowOutPlain, ra, s)) return rc;
+  LAUNCH((k_resid0<<<dblocks(N), 256, 0, s>>>(N, b, im[1], x, T.R, k > 0 ? T.P : nullptr, k, part, cnt, H)));
+  // rho_0 = 0 (the zero state of the first iteration): no step is run, as in the oracle
+  double rho0 = 0.0;
+  if (k > 0) {
+    if (int rc = check_cuda(cudaMemcpyAsync(&rho0, &H->rho[0], sizeof(double), cudaMemcpyDeviceToHost, s))) return rc;
+    if (int rc = check_cuda(cudaStreamSynchronize(s))) return rc;
+  }
+  for (int j = 0; j < k && rho0 != 0.0; ++j) {
     float2* pj = T.P + (int64_t)j * N;
     float2* qj = T.Qp + (int64_t)j * N;
-    if (int rc = apply_ww(c, pj, A.w, T.PhiP + (int64_t)j * M, m[0], im[1], s)) return rc;
-    LAUNCH((k_plus2<<<dblocks(N), 256, 0, s>>>(N, im[1], pj, qj)));
-    double pq;
-    if (int rc = host_dot(c, N, pj, qj, &pq, s)) return rc;
-    const double alpha = pq > 0.0 ? rho / pq : 0.0;
-    LAUNCH((k_cg_upd<<<dblocks(N), 256, 0, s>>>(N, (float)alpha, x, pj, T.R + (int64_t)j * N, qj,
-                                                 T.R + (int64_t)(j + 1) * N)));
-    double rho_n;
-    if (int rc = host_dot(c, N, T.R + (int64_t)(j + 1) * N, T.R + (int64_t)(j + 1) * N, &rho_n, s)) return rc;
-    const double beta = rho_n / rho;
-    if (j + 1 < k)
-      LAUNCH((k_cg_dir<<<dblocks(N), 256, 0, s>>>(N, (float)beta, T.R + (int64_t)(j + 1) * N, pj,
-                                                  T.P + (int64_t)(j + 1) * N)));
-    H.alpha[j] = alpha;
-    H.beta[j] = beta;
-    H.pi[j] = pq;
-    H.rho[j + 1] = rho_n;
-    rho = rho_n;
-    steps = j + 1;
+    float2* rj = T.R + (int64_t)j * N;
+    // q = Q_w p with the block partials of <p, p> and <q, p>
+    ra.out = qj;
+    ra.p = pj;
+    if (int rc = apply_ww(c, pj, A.w, T.PhiP + (int64_t)j * M, m[0], kRowOutCgQ, ra, s)) return rc;
+    LAUNCH((k_cg_upd<<<dblocks(N), 256, 0, s>>>(N, c->d_partials + kCntDot * 2 * kMaxPartials + kMaxPartials,
+                                                cg_partial_blocks(c), j, x, pj, rj, qj, rj + N, part, cnt, H)));
+    if (j + 1 < k) LAUNCH((k_cg_dir<<<dblocks(N), 256, 0, s>>>(N, H, j, rj + N, pj, pj + N)));
   }
-  H.steps = steps;
   // ---- i = 1: a1 = Psi^H x_hat' + z1; z1', x1' = Psi (2 r1 - a1)
   SaraProxArgs pa{};
   if (int rc = sara_analysis(c, x, T.A1, kSaraPlain, pa, s)) return rc;
@@ -522,25 +629,11 @@ int diff_forward(purify_ctx* c, const DiffArgs& A, float2* const* in, float2* co
   if (int rc = sara_synthesis(c, T.U1, out[4], s)) return rc;
   // ---- i = 2: a2 = w o Phi x_hat' + z2; projection onto the ball around y_w
   if (int rc = phi_into(c, x, T.PhiXh, s)) return rc;
-  LAUNCH((k_b2_a<<<dblocks(M), 256, 0, s>>>(M, T.PhiXh, A.w, in[2], T.A2)));
-  double nd2;
-  {
-    double* slot = &c->d_sc->norm2;
-    LAUNCH((k_norm_wdiff<<<dblocks(M), 256, 0, s>>>(M, T.A2, A.w, A.y, c->d_partials + kCntNorm * 2 * kMaxPartials,
-                                                    &c->d_sc->counter[kCntNorm], slot)));
-    if (int rc = check_cuda(cudaMemcpyAsync(&nd2, slot, sizeof(double), cudaMemcpyDeviceToHost, s))) return rc;
-    if (int rc = check_cuda(cudaStreamSynchronize(s))) return rc;
-  }
-  const double nd = std::sqrt(nd2);
-  const double cb = nd > A.eps ? A.eps / nd : 1.0;
-  H.nd = nd;
-  H.cball = cb;
-  LAUNCH((k_b2_b<<<dblocks(M), 256, 0, s>>>(M, T.A2, A.w, A.y, (float)cb, out[2], T.U2, m[1])));
+  LAUNCH((k_b2_a<<<dblocks(M), 256, 0, s>>>(M, T.PhiXh, A.w, in[2], A.y, T.A2, A.eps, part, cnt, H)));
+  LAUNCH((k_b2_b<<<dblocks(M), 256, 0, s>>>(M, T.A2, A.w, A.y, H, out[2], T.U2, m[1])));
   if (int rc = phi_adj_into(c, m[1], out[5], s)) return rc;
   // ---- i = 3
   LAUNCH((k_b3_fwd<<<dblocks(N), 256, 0, s>>>(N, x, in[3], T.A3, out[3], out[6])));
-  // header last (host staging copy, then synchronise so H may go out of scope)
-  if (int rc = check_cuda(cudaMemcpyAsync(tape_mem, &H, sizeof(H), cudaMemcpyHostToDevice, s))) return rc;
   return check_cuda(cudaStreamSynchronize(s));
 }
 
@@ -549,9 +642,14 @@ int diff_backward(purify_ctx* c, const DiffArgs& A, float2* const* in, const voi
   const int64_t N = nN(c), M = c->M, D = nD(c);
   const int k = A.k;
   float2 *m[3], *im[4], *dv;
-  if (int rc = diff_scratch(c, m, im, &dv)) return rc;
+  BwdScalars* S = nullptr;
+  if (int rc = diff_scratch(c, m, im, &dv, &S)) return rc;
   Tape T = tape_views(c, k, const_cast<void*>(tape_mem));
-  TapeHeader H;
+  const TapeHeader* dH = static_cast<const TapeHeader*>(tape_mem);  // (device)
+  double* part = c->d_partials + kCntNorm * 2 * kMaxPartials;
+  unsigned* cnt = &c->d_sc->counter[kCntNorm];
+  if (int rc = check_cuda(cudaMemsetAsync(S, 0, sizeof(BwdScalars), s))) return rc;
+  TapeHeader H;  // (host: the step count and whether the projection was active)
   if (int rc = check_cuda(cudaMemcpyAsync(&H, tape_mem, sizeof(H), cudaMemcpyDeviceToHost, s))) return rc;
   if (int rc = check_cuda(cudaStreamSynchronize(s))) return rc;
   if (H.k != k) return PURIFY_E_INVALID_ARG;
@@ -570,18 +668,9 @@ int diff_backward(purify_ctx* c, const DiffArgs& A, float2* const* in, const voi
   if (int rc = phi_into(c, ob[5], m[0], s)) return rc;
   LAUNCH((k_b2_bwd1<<<dblocks(M), 256, 0, s>>>(M, m[0], A.w, T.U2, ob[2], m[1], m[2], wb)));
   const int outside = H.nd > A.eps ? 1 : 0;
-  float k2 = 0.f;
-  if (outside) {
-    // <d, rbar2>, d = a2 - y_w (FP64): the ball's Jacobian needs it
-    double* slot = &c->d_sc->norm2;
-    double dr;
-    LAUNCH((k_dot_wdiff<<<dblocks(M), 256, 0, s>>>(M, T.A2, A.w, A.y, m[1], c->d_partials + kCntNorm * 2 * kMaxPartials,
-                                                   &c->d_sc->counter[kCntNorm], slot)));
-    if (int rc = check_cuda(cudaMemcpyAsync(&dr, slot, sizeof(double), cudaMemcpyDeviceToHost, s))) return rc;
-    if (int rc = check_cuda(cudaStreamSynchronize(s))) return rc;
-    k2 = (float)(H.cball * dr / (H.nd * H.nd));
-  }
-  LAUNCH((k_b2_bwd2<<<dblocks(M), 256, 0, s>>>(M, T.A2, A.w, A.y, outside, (float)H.cball, k2, m[1], m[2], T.PhiXh,
+  if (outside)  // <d, rbar2>, d = a2 - y_w (FP64): the ball's Jacobian needs it
+    LAUNCH((k_dot_wdiff<<<dblocks(M), 256, 0, s>>>(M, T.A2, A.w, A.y, m[1], part, cnt, dH, S)));
+  LAUNCH((k_b2_bwd2<<<dblocks(M), 256, 0, s>>>(M, T.A2, A.w, A.y, outside, (float)H.cball, S, m[1], m[2], T.PhiXh,
                                                wb, ib[2], m[0])));
   if (int rc = phi_adj_into(c, m[0], im[1], s)) return rc;
   LAUNCH((k_add<<<dblocks(N), 256, 0, s>>>(N, xacc, im[1], xacc)));
@@ -592,36 +681,23 @@ int diff_backward(purify_ctx* c, const DiffArgs& A, float2* const* in, const voi
   float2* vN = dv;  // the coefficient-size scratch, used as one more image vector
   if (int rc = check_cuda(cudaMemsetAsync(rb, 0, N * sizeof(float2), s))) return rc;
   if (int rc = check_cuda(cudaMemsetAsync(pb, 0, N * sizeof(float2), s))) return rc;
-  double rhob = 0.0;  // adjoint of rho_{j+1}, carried down
+  RowOutArgs ra{};
+  ra.out = vN;
+  if (H.steps > 0)
+    LAUNCH((k_cgb_first<<<dblocks(N), 256, 0, s>>>(N, xacc, T.P + (int64_t)(H.steps - 1) * N, part, cnt, S)));
   for (int j = H.steps - 1; j >= 0; --j) {
     const float2* pj = T.P + (int64_t)j * N;
     const float2* qj = T.Qp + (int64_t)j * N;
-    const float2* rj1 = T.R + (int64_t)(j + 1) * N;
-    double betab = 0.0;  // p_bar_{j+1} is zero for the last step run
-    if (j < H.steps - 1) {
-      if (int rc = host_dot(c, N, pb, pj, &betab, s)) return rc;
-    }
-    const double rho_j = H.rho[j], rho_j1 = H.rho[j + 1], al = H.alpha[j], be = H.beta[j], pq = H.pi[j];
-    rhob += betab / rho_j;
-    LAUNCH((k_cgb_r<<<dblocks(N), 256, 0, s>>>(N, rb, pb, (float)(2.0 * rhob), rj1)));
-    double rq, xp;
-    if (int rc = host_dot(c, N, rb, qj, &rq, s)) return rc;
-    if (int rc = host_dot(c, N, xacc, pj, &xp, s)) return rc;
-    const double alb = pq > 0.0 ? -rq + xp : 0.0;
-    const double rhob_j = -betab * rho_j1 / (rho_j * rho_j) + (pq > 0.0 ? alb / pq : 0.0);
-    const double pib = pq > 0.0 ? -alb * rho_j / (pq * pq) : 0.0;
-    LAUNCH((k_cgb_q<<<dblocks(N), 256, 0, s>>>(N, (float)al, rb, (float)pib, pj, qb)));
-    // v = Phi_w^H Phi_w qbar (m0 = Phi qbar); w_bar += 2 w Re(conj(Phi qbar) Phi p_j)
-    if (int rc = apply_ww(c, qb, A.w, m[0], m[1], vN, s)) return rc;
-    LAUNCH((k_wbar_q<<<dblocks(M), 256, 0, s>>>(M, 2.f, A.w, m[0], T.PhiP + (int64_t)j * M, wb)));
-    LAUNCH((k_cgb_p<<<dblocks(N), 256, 0, s>>>(N, (float)be, pb, (float)al, xacc, (float)pib, qj, vN, qb)));
-    rhob = rhob_j;
+    LAUNCH((k_cgb_r<<<dblocks(N), 256, 0, s>>>(N, rb, pb, T.R + (int64_t)(j + 1) * N, qj, j, part, cnt, dH, S)));
+    LAUNCH((k_cgb_q<<<dblocks(N), 256, 0, s>>>(N, dH, S, j, rb, pj, qb)));
+    // v = Phi_w^H Phi_w qbar; w_bar += 2 w Re(conj(Phi qbar) Phi p_j)
+    if (int rc = apply_ww(c, qb, A.w, nullptr, m[1], kRowOutPlain, ra, s, T.PhiP + (int64_t)j * M, 2.f, wb)) return rc;
+    LAUNCH((k_cgb_p<<<dblocks(N), 256, 0, s>>>(N, dH, j, pb, xacc, qj, vN, qb, j > 0 ? pj - N : nullptr, part, cnt, S)));
   }
   // p_0 = r_0 and rho_0 = <r_0, r_0>
-  LAUNCH((k_cgb_r<<<dblocks(N), 256, 0, s>>>(N, rb, pb, (float)(2.0 * rhob), T.R)));
+  LAUNCH((k_cgb_r<<<dblocks(N), 256, 0, s>>>(N, rb, pb, T.R, nullptr, 0, part, cnt, dH, S)));
   // r_0 = b - Q_w x_0: b_bar = r_bar; x0_bar = x_bar - Q_w r_bar; w term
-  if (int rc = apply_ww(c, rb, A.w, m[0], m[1], vN, s)) return rc;
-  LAUNCH((k_wbar_q<<<dblocks(M), 256, 0, s>>>(M, -2.f, A.w, m[0], T.PhiX0, wb)));
+  if (int rc = apply_ww(c, rb, A.w, nullptr, m[1], kRowOutPlain, ra, s, T.PhiX0, -2.f, wb)) return rc;
   LAUNCH((k_cgb_end<<<dblocks(N), 256, 0, s>>>(N, xacc, vN, rb, ib[0], ib[4], ib[5], ib[6])));
   return check_cuda(cudaStreamSynchronize(s));
 }

@@ -455,7 +455,7 @@ GraphKey step_graph_key(const purify_sdmm_state* st);                          /
 // kRowInCgUpd: apply the pending CG vector update, then transform r;
 // kRowInCgFinish: apply it, then transform x.
 enum RowInMode { kRowInPlain = 0, kRowInCgUpd = 1, kRowInCgFinish = 2 };
-enum DegridOut { kDegridPerm = 0, kDegridSorted = 1, kDegridSdmm = 2 };
+enum DegridOut { kDegridPerm = 0, kDegridSorted = 1, kDegridSdmm = 2, kDegridWeighted = 3 };
 enum GridIn { kGridPerm = 0, kGridSorted = 1, kGridGram = 2 };
 enum RowOutMode { kRowOutPlain = 0, kRowOutCgQ = 1, kRowOutSdmm = 2 };
 
@@ -475,6 +475,14 @@ struct DegridArgs {
   const float2* y;          // sdmm data (sorted) or NULL when bf16
   const uint16_t* yb;       // sdmm bf16 data
   const float* yscale;
+  // weighted (the differentiable iteration): out (caller order, may be NULL)
+  // = s = Phi x; t (sorted order) = w^2 s for the gridding that follows;
+  // with wb: wb += hf w Re(conj(s) h)
+  const float* w;           // M, caller order
+  float2* t;
+  const float2* h;          // M, caller order
+  float hf;
+  float* wb;                // M, caller order, or NULL
 };
 struct RowOutArgs {
   float2* out;          // plain: image; cg: w = Q r; sdmm: r0

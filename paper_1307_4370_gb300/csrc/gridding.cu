@@ -102,6 +102,15 @@ __global__ void __launch_bounds__(256) k_degrid(const float2* __restrict__ X, co
       a.out[perm[i]] = acc;
     } else if (MODE == kDegridSorted) {
       a.out[i] = acc;
+    } else if (MODE == kDegridWeighted) {
+      const int m = perm[i];
+      const float w = a.w[m];
+      if (a.out) a.out[m] = acc;
+      a.t[i] = cscale(acc, w * w);
+      if (a.wb) {
+        const float2 h = a.h[m];
+        a.wb[m] += a.hf * w * (acc.x * h.x + acc.y * h.y);
+      }
     } else {
       // SDMM: s2 = Phi x_hat, and the two FP64 norms of the l2 branch
       a.out[i] = acc;
@@ -600,6 +609,7 @@ static void degrid_J(purify_ctx* c, DegridOut mode, const DegridArgs& a, cudaStr
   } while (0)
   if (mode == kDegridPerm) DEG(kDegridPerm);
   else if (mode == kDegridSorted) DEG(kDegridSorted);
+  else if (mode == kDegridWeighted) DEG(kDegridWeighted);
   else DEG(kDegridSdmm);
 #undef DEG
 }
