@@ -767,7 +767,7 @@ static int purify_create_impl(purify_ctx** out, const purify_desc* d, const floa
   c->ks.lo = (float)(sc - (double)c->ks.hi);
   c->plan = make_plan(c->L);
   if (c->plan.nst < 0) { delete c; return PURIFY_E_UNSUPPORTED; }
-  c->fft_engine = (c->L >= 256 && c->L <= 4096 && (c->L & (c->L - 1)) == 0) ? 1 : 0;
+  c->fft_engine = fft_fixed_side(c->L) ? 1 : 0;
   make_daubechies(c->wf);
   if (d->tile != 0) {
     c->tileT = d->tile;

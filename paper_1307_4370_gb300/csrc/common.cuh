@@ -289,8 +289,8 @@ struct purify_ctx {
 
   float* d_deapod;      // n: 1 / g_hat((r - n/2) / 2n)
   float2* d_tw;         // L: exp(-2 pi i m / L)
-  int fft_engine;       // 1: compile-time power-of-two engine (L = 256 .. 4096), 0: generic Stockham
-  float2* d_twp[2];     // per-stage twiddle tables of the power-of-two engine (8 and 16 per thread)
+  int fft_engine;       // 1: compile-time engine (fft_fixed_side), 0: generic Stockham
+  float2* d_twp[2];     // per-stage twiddle tables of that engine (8 or 12, 16 or 24 per thread)
 
   // visibility table (sorted by grid tile of the first footprint cell)
   float2* d_uv;         // M sorted frequencies
@@ -491,7 +491,8 @@ struct RowOutArgs {
   float2* z3;           // sdmm
 };
 
-int fft_prepare(purify_ctx* c);  // tables of the power-of-two FFT engine (at context creation)
+bool fft_fixed_side(int L);      // the compile-time FFT engine has this grid side
+int fft_prepare(purify_ctx* c);  // its tables (at context creation)
 // cg_j: in the CG modes, the CG step whose update this pass applies (its
 // inner-product partials are in the kCntDot slot).
 int phi_forward_grid(purify_ctx* c, RowInMode mode, const RowInArgs& a, cudaStream_t s, int cg_j = 0);

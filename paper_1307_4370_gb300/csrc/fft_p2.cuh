@@ -1,14 +1,16 @@
-// Power-of-two FFT engine with the radices, strides and thread mapping fixed
-// at compile time (L = 2^p, 256 <= L <= 4096): the unitary DFT F of §5 eq.
-// opmodel, applied as 1-D transforms of the rows and of the columns of the
-// oversampled grid.
+// FFT engine with the radices, strides and thread mapping fixed at compile time
+// (L = 2^p, 128 <= L <= 4096, and L = 3 2^p, 192 <= L <= 3072): the unitary DFT
+// F of §5 eq. opmodel, applied as 1-D transforms of the rows and of the columns
+// of the oversampled grid.
 //
 // Same Stockham autosort formulation as fft.cuh (stage with radix R after
 // stages whose radices multiply to Ns: read R values L/R apart, twiddle by
 // exp(-2 pi i r k / (Ns R)), k = j mod Ns, R-point DFT, write Ns apart from
 // (j / Ns) Ns R + k; natural-order output), specialised so that
-//  * every index split is a shift or a mask, every loop is unrolled;
-//  * each thread runs E / R butterflies of a stage, E = elements per thread;
+//  * every index split is by a constant, every loop is unrolled;
+//  * each thread runs E / R butterflies of a stage, E = elements per thread
+//    (8 or 16; 12 or 24 where 3 divides L, whose first radix, 12 or 24, takes
+//    the factor 3 by a prime-factor map, without inner twiddles);
 //  * shared memory is padded by one complex value per 16, so the strided
 //    writes of the first stages and the strided reads of the column layout
 //    fall in distinct banks;
@@ -64,17 +66,59 @@ __device__ __forceinline__ void dft_small<16>(float2* v) {
   }
 }
 
-constexpr int p2_log2(int x) { return x <= 1 ? 0 : 1 + p2_log2(x >> 1); }
+// 3 Q-point DFT (Q = 4 or 8, coprime to 3): with j = (Q j1 + 3 j2) mod 3 Q and
+// k = (A k1 + 9 k2) mod 3 Q, A = 4 (Q = 4) or 16 (Q = 8) (A = 1 mod 3, 0 mod Q;
+// 9 = 0 mod 3, 1 mod Q), the transform is a Q-point DFT along j2 and a 3-point
+// one along j1 with no twiddles between (Good-Thomas prime-factor map).
+template <int Q>
+__device__ __forceinline__ void dft_3q(float2* v) {
+  constexpr int N = 3 * Q, A = Q == 4 ? 4 : 16;
+  float2 a[3][Q];
+#pragma unroll
+  for (int j1 = 0; j1 < 3; ++j1) {
+#pragma unroll
+    for (int j2 = 0; j2 < Q; ++j2) a[j1][j2] = v[(Q * j1 + 3 * j2) % N];
+    dft_small<Q>(a[j1]);
+  }
+#pragma unroll
+  for (int k2 = 0; k2 < Q; ++k2) {
+    float2 t[3] = {a[0][k2], a[1][k2], a[2][k2]};
+    dft_small<3>(t);
+#pragma unroll
+    for (int k1 = 0; k1 < 3; ++k1) v[(A * k1 + 9 * k2) % N] = t[k1];
+  }
+}
+template <>
+__device__ __forceinline__ void dft_small<12>(float2* v) { dft_3q<4>(v); }
+template <>
+__device__ __forceinline__ void dft_small<24>(float2* v) { dft_3q<8>(v); }
+
 constexpr int p2_min(int a, int b) { return a < b ? a : b; }
-// Radix of stage st: E until fewer than E remain.
+constexpr int p2_max(int a, int b) { return a > b ? a : b; }
+// First radix: E, or for L = 3 2^p and E = 24 the one of 24 and 12 that leaves
+// 8^a or 4 8^a (the pruned last stage needs a radix of at least 4).
+constexpr int p2_first(int L, int E) {
+  if (L % 3 != 0) return p2_min(E, L);
+  if (E == 12) return 12;
+  int rem = L / 24;
+  while (rem >= 8) rem /= 8;
+  return rem == 2 ? 12 : 24;
+}
+// Radix of stage st: after the first, E (8 or 4 of 24 or 12) until fewer remain.
 constexpr int p2_radix(int L, int E, int st) {
-  int rem = L;
-  for (int i = 0; i < st; ++i) rem /= p2_min(E, rem);
-  return p2_min(E, rem);
+  const int cap = L % 3 != 0 ? E : E / 3;
+  int rem = L, r = p2_first(L, E);
+  for (int i = 0; i < st; ++i) {
+    rem /= r;
+    r = p2_min(cap, rem);
+  }
+  return r;
 }
 constexpr int p2_nstages(int L, int E) {
   int n = 0;
-  for (int rem = L; rem > 1; rem /= p2_min(E, rem)) ++n;
+  for (int rem = L; rem > 1; rem /= p2_radix(L, E, n), ++n) {
+    if (p2_radix(L, E, n) <= 1) break;
+  }
   return n;
 }
 constexpr int p2_ns(int L, int E, int st) {
@@ -106,21 +150,22 @@ constexpr size_t p2_smem_bytes() { return (size_t)NSIG * (L + L / 16) * sizeof(f
 // Butterfly q of this thread in a stage with L/R butterflies per signal.
 template <int L, int R, int NSIG, bool SIG_FAST, int T>
 __device__ __forceinline__ void p2_map(int q, int& s, int& j) {
-  const int b = threadIdx.x + q * T;
-  constexpr int LR = L / R;
+  const unsigned b = threadIdx.x + q * T;
+  constexpr unsigned LR = L / R, NS = NSIG;
   if constexpr (SIG_FAST) {
-    s = b & (NSIG - 1);
-    j = b >> p2_log2(NSIG);
+    s = b % NS;
+    j = b / NS;
   } else {
-    s = b >> p2_log2(LR);
-    j = b & (LR - 1);
+    s = b / LR;
+    j = b % LR;
   }
 }
 
 // Middle stage st (1 <= st < nstages - 1): shared memory to shared memory.
 template <int L, int E, int NSIG, bool SIG_FAST, int ST>
 __device__ __forceinline__ void p2_stage_mid(float2* buf, const float2* __restrict__ twt) {
-  constexpr int R = p2_radix(L, E, ST), NS = p2_ns(L, E, ST), NB = E / R, T = NSIG * L / E;
+  constexpr int R = p2_radix(L, E, ST), NB = E / R, T = NSIG * L / E;
+  constexpr unsigned NS = p2_ns(L, E, ST);
   constexpr int LR = L / R;
   const float2* tw = twt + p2_twoff(L, E, ST);
   float2 v[NB][R];
@@ -128,7 +173,7 @@ __device__ __forceinline__ void p2_stage_mid(float2* buf, const float2* __restri
   for (int q = 0; q < NB; ++q) {
     int s, j;
     p2_map<L, R, NSIG, SIG_FAST, T>(q, s, j);
-    const int k = j & (NS - 1);
+    const int k = (unsigned)j % NS;
 #pragma unroll
     for (int r = 0; r < R; ++r) v[q][r] = buf[p2_at<L, NSIG, SIG_FAST>(s, j + r * LR)];
 #pragma unroll
@@ -140,8 +185,8 @@ __device__ __forceinline__ void p2_stage_mid(float2* buf, const float2* __restri
   for (int q = 0; q < NB; ++q) {
     int s, j;
     p2_map<L, R, NSIG, SIG_FAST, T>(q, s, j);
-    const int k = j & (NS - 1);
-    const int base = (j >> p2_log2(NS)) * NS * R + k;
+    const int k = (unsigned)j % NS;
+    const int base = (unsigned)j / NS * (NS * R) + k;
 #pragma unroll
     for (int r = 0; r < R; ++r) buf[p2_at<L, NSIG, SIG_FAST>(s, base + r * NS)] = v[q][r];
   }
@@ -167,7 +212,7 @@ __device__ __forceinline__ void fft_p2(float2* buf, const float2* __restrict__ t
   constexpr int T = NSIG * L / E;
   constexpr int NST = p2_nstages(L, E);
   static_assert(NST >= 2, "at least two stages");
-  static_assert((L & (L - 1)) == 0 && (NSIG & (NSIG - 1)) == 0, "powers of two");
+  static_assert(L % E == 0 && E % p2_radix(L, E, 0) == 0, "whole butterflies per thread");
   // ---- first stage: radix R0 = E, one butterfly per thread per signal set
   {
     constexpr int R = p2_radix(L, E, 0), NB = E / R, LR = L / R;

@@ -358,34 +358,33 @@ __global__ void __launch_bounds__(256) k_row_inv(const float2* __restrict__ half
 }
 
 // ---------------------------------------------------------------------------
-// The same four passes on power-of-two grids (L = 256 .. 4096) with the
-// compile-time engine of fft_p2.cuh: the zero padding of the forward passes
-// and the crop of the adjoint ones prune the first / last stage.
+// The same four passes with the compile-time engine of fft_p2.cuh (2^p and
+// 3 2^p grids): the zero padding of the forward passes and the crop of the
+// adjoint ones prune the first / last stage.
 // ---------------------------------------------------------------------------
-#ifndef P2_E_LARGE
-#define P2_E_LARGE 16
-#endif
-#ifndef P2_E_CG
-#define P2_E_CG 8
-#endif
-#ifndef P2_NS_COL
-#define P2_NS_COL (L == 2048 ? 8 : 4)  // at most 1024 threads: NS L / E
-#endif
-#ifndef P2_ROWCG_THREADS
-#define P2_ROWCG_THREADS 256
-#endif
-#ifndef P2_RINV_THREADS
-#define P2_RINV_THREADS 512
-#endif
+// Signals (rows, adjacent columns) per CTA.  The passes of small grids are
+// latency-bound, so rows are spread over about 128 CTAs before a CTA takes a
+// second one (at 512, 32 CTAs of eight rows: 6.7 us an inverse row pass
+// against ROWINV us for 128 of two), with at least a warp per CTA; the inverse row pass of the CG leaves one pair of
+// partial sums per CTA, which every CTA of the next pass adds up.
+constexpr int p2_rows(int L, int E, int max_threads) {
+  const int per = L / E;                        // threads per row
+  int ns = p2_max(1, L / 2 / 128);              // about 128 CTAs
+  while (ns * per < 32) ns *= 2;
+  while (ns > 1 && ns * per > max_threads) ns /= 2;
+  int p = 1;
+  while (p * 2 <= ns) p *= 2;                   // a power of two (divides n)
+  return p;
+}
 template <int L>
 struct P2Cfg {
-  static constexpr int E = L >= 1024 ? P2_E_LARGE : 8;             // plain row, column and inverse row passes
-  static constexpr int E_CG = P2_E_CG;                             // forward row pass with the CG update
-  static constexpr int NS_ROW = 256 / (L / E) > 0 ? 256 / (L / E) : 1;
-  static constexpr int NS_ROWCG = P2_ROWCG_THREADS / (L / E_CG) > 0 ? P2_ROWCG_THREADS / (L / E_CG) : 1;
-  static constexpr int NS_RINV =
-      P2_RINV_THREADS / (L / E) > 0 ? (P2_RINV_THREADS / (L / E) > 8 ? 8 : P2_RINV_THREADS / (L / E)) : 1;
-  static constexpr int NS_COL = P2_NS_COL;
+  static constexpr bool T3 = L % 3 == 0;
+  static constexpr int E = T3 ? 24 : (L >= 1024 || L == 128 ? 16 : 8);  // plain row, column and inverse row passes
+  static constexpr int E_CG = T3 ? 12 : 8;                              // forward row pass with the CG update
+  static constexpr int NS_ROW = p2_rows(L, E, 256);
+  static constexpr int NS_ROWCG = p2_rows(L, E_CG, 256);
+  static constexpr int NS_RINV = p2_rows(L, E, 512);
+  static constexpr int NS_COL = L == 2048 ? 8 : 4;  // at most 1024 threads: NS L / E
 };
 
 template <int L, int E, int NSIG, int MODE>
@@ -442,10 +441,12 @@ __global__ void __launch_bounds__(NSIG * L / E) k_col_inv_p2(const float2* __res
 
 // Register cap: two CTAs per SM for the CG and plain epilogues; the SDMM
 // epilogue (five operands per pixel) keeps its registers.
-constexpr int p2_rinv_minb(int T, int MODE) { return MODE == kRowOutSdmm ? 1 : (1024 / T > 1 ? 1024 / T : 1); }
+constexpr int p2_rinv_minb(int T, int E, int MODE) {
+  return MODE == kRowOutSdmm || E > 16 || 1024 / T <= 1 ? 1 : p2_min(1024 / T, 16);
+}
 
 template <int L, int E, int NSIG, int MODE>
-__global__ void __launch_bounds__(NSIG * L / E, p2_rinv_minb(NSIG * L / E, MODE)) k_row_inv_p2(const float2* __restrict__ half, RowOutArgs a,
+__global__ void __launch_bounds__(NSIG * L / E, p2_rinv_minb(NSIG * L / E, E, MODE)) k_row_inv_p2(const float2* __restrict__ half, RowOutArgs a,
                                                              const float* __restrict__ dz,
                                                              const float* __restrict__ beam,
                                                              const float2* __restrict__ twt, int n,
@@ -472,13 +473,24 @@ __global__ void __launch_bounds__(NSIG * L / E, p2_rinv_minb(NSIG * L / E, MODE)
   }
 }
 
-// Whether the grid side has the compile-time engine.
-static bool p2_side(int L) { return L == 256 || L == 512 || L == 1024 || L == 2048 || L == 4096; }
+// The grid sides of the compile-time engine.
+#define P2_SIDES(CASE)                                                            \
+  CASE(128) CASE(192) CASE(256) CASE(384) CASE(512) CASE(768) CASE(1024) CASE(1536) CASE(2048) CASE(3072) CASE(4096)
+
+bool fft_fixed_side(int L) {
+  switch (L) {
+#define P2_CASE(S) case S:
+    P2_SIDES(P2_CASE)
+#undef P2_CASE
+    return true;
+    default: return false;
+  }
+}
 
 // Concatenated twiddle tables of the engine for (L, E) (device, owned by the context).
 template <int L, int E>
 static int p2_table(purify_ctx* c, const float2** out) {
-  const int idx = (E == 16) ? 1 : 0;
+  const int idx = (E == 16 || E == 24) ? 1 : 0;
   if (!c->d_twp[idx]) {
     std::vector<float2> t(std::max(1, p2_twsize(L, E)));
     p2_twiddles<L, E>(t.data());
@@ -506,11 +518,9 @@ static int p2_prepare_L(purify_ctx* c) {
 int fft_prepare(purify_ctx* c) {
   if (c->fft_engine != 1) return PURIFY_OK;
   switch (c->L) {
-    case 256: return p2_prepare_L<256>(c);
-    case 512: return p2_prepare_L<512>(c);
-    case 1024: return p2_prepare_L<1024>(c);
-    case 2048: return p2_prepare_L<2048>(c);
-    case 4096: return p2_prepare_L<4096>(c);
+#define P2_CASE(S) case S: return p2_prepare_L<S>(c);
+    P2_SIDES(P2_CASE)
+#undef P2_CASE
     default: c->fft_engine = 0; return PURIFY_OK;
   }
 }
@@ -595,12 +605,10 @@ static int p2_adjoint(purify_ctx* c, RowOutMode mode, const RowOutArgs& a, cudaS
 // ---------------------------------------------------------------------------
 // Blocks of the inverse row pass, i.e. the CG inner-product partials it leaves.
 int cg_partial_blocks(const purify_ctx* c) {
-  switch (p2_side(c->L) ? c->L : 0) {
-    case 256: return c->n / P2Cfg<256>::NS_RINV;
-    case 512: return c->n / P2Cfg<512>::NS_RINV;
-    case 1024: return c->n / P2Cfg<1024>::NS_RINV;
-    case 2048: return c->n / P2Cfg<2048>::NS_RINV;
-    case 4096: return c->n / P2Cfg<4096>::NS_RINV;
+  switch (c->fft_engine == 1 ? c->L : 0) {
+#define P2_CASE(S) case S: return c->n / P2Cfg<S>::NS_RINV;
+    P2_SIDES(P2_CASE)
+#undef P2_CASE
     default: return c->n / row_shape(c).nsig;
   }
 }
@@ -627,12 +635,10 @@ int phi_forward_grid(purify_ctx* c, RowInMode mode, const RowInArgs& a, cudaStre
   const float* beam = c->beam_on ? c->d_beam : nullptr;
   if (c->fft_engine == 1) {
     switch (c->L) {
-      case 256: return p2_forward<256>(c, mode, a, s, cg_j, beam);
-      case 512: return p2_forward<512>(c, mode, a, s, cg_j, beam);
-      case 1024: return p2_forward<1024>(c, mode, a, s, cg_j, beam);
-      case 2048: return p2_forward<2048>(c, mode, a, s, cg_j, beam);
-      case 4096: return p2_forward<4096>(c, mode, a, s, cg_j, beam);
-      default: break;
+  #define P2_CASE(S) case S: return p2_forward<S>(c, mode, a, s, cg_j, beam);
+    P2_SIDES(P2_CASE)
+#undef P2_CASE
+    default: break;
     }
   }
   const FftShape rs = row_shape(c), cs = col_shape(c);
@@ -681,12 +687,10 @@ int phi_adjoint_image(purify_ctx* c, RowOutMode mode, const RowOutArgs& a, cudaS
   const float2* Xg = grid ? grid : c->d_grid;
   if (c->fft_engine == 1) {
     switch (c->L) {
-      case 256: return p2_adjoint<256>(c, mode, a, s, Xg, before_rows, beam);
-      case 512: return p2_adjoint<512>(c, mode, a, s, Xg, before_rows, beam);
-      case 1024: return p2_adjoint<1024>(c, mode, a, s, Xg, before_rows, beam);
-      case 2048: return p2_adjoint<2048>(c, mode, a, s, Xg, before_rows, beam);
-      case 4096: return p2_adjoint<4096>(c, mode, a, s, Xg, before_rows, beam);
-      default: break;
+  #define P2_CASE(S) case S: return p2_adjoint<S>(c, mode, a, s, Xg, before_rows, beam);
+    P2_SIDES(P2_CASE)
+#undef P2_CASE
+    default: break;
     }
   }
   const FftShape rs = row_shape(c), cs = col_shape(c);
