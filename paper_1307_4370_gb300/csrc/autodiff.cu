@@ -61,6 +61,7 @@ struct BwdScalars {
 // out = w^pw o in (complex by real), pw = 1 or 2
 __global__ void k_wmul(int64_t n, const float2* __restrict__ in, const float* __restrict__ w, int pw,
                        float2* __restrict__ out) {
+  pdl_sync(in, w, out);
   DGRID(i, n) {
     const float s = pw == 2 ? w[i] * w[i] : w[i];
     out[i] = cscale(in[i], s);
@@ -70,6 +71,7 @@ __global__ void k_wmul(int64_t n, const float2* __restrict__ in, const float* __
 // Re <a, b> in FP64 -> *out
 __global__ void k_dot(int64_t n, const float2* __restrict__ a, const float2* __restrict__ b, double* partials,
                       unsigned* counter, double* out) {
+  pdl_sync(a, b, partials, counter, out);
   FPair part;
   DGRID(i, n) {
     part.add_prod(a[i].x, b[i].x);
@@ -83,6 +85,7 @@ __global__ void k_dot(int64_t n, const float2* __restrict__ a, const float2* __r
 __global__ void k_dot_wdiff(int64_t n, const float2* __restrict__ a, const float* __restrict__ w,
                             const float2* __restrict__ y, const float2* __restrict__ r, double* partials,
                             unsigned* counter, const TapeHeader* __restrict__ H, BwdScalars* S) {
+  pdl_sync(a, w, y, r, partials, counter, H, S);
   FPair part;
   DGRID(i, n) {
     const float2 d = csub(a[i], cscale(y[i], w[i]));
@@ -96,6 +99,7 @@ __global__ void k_dot_wdiff(int64_t n, const float2* __restrict__ a, const float
 // out = a + b + c
 __global__ void k_sum3(int64_t n, const float2* __restrict__ a, const float2* __restrict__ b,
                        const float2* __restrict__ c, float2* __restrict__ out) {
+  pdl_sync(a, b, c, out);
   DGRID(i, n) out[i] = cadd(cadd(a[i], b[i]), c[i]);
 }
 
@@ -104,6 +108,7 @@ __global__ void k_sum3(int64_t n, const float2* __restrict__ a, const float2* __
 __global__ void k_resid0(int64_t n, const float2* __restrict__ u, const float2* __restrict__ v,
                          const float2* __restrict__ x, float2* __restrict__ r0, float2* __restrict__ p0, int k,
                          double* partials, unsigned* counter, TapeHeader* H) {
+  pdl_sync(u, v, x, r0, p0, partials, counter, H);
   FPair part;
   DGRID(i, n) {
     const float2 r = make_float2(u[i].x - v[i].x - 2.f * x[i].x, u[i].y - v[i].y - 2.f * x[i].y);
@@ -126,6 +131,7 @@ __global__ void k_resid0(int64_t n, const float2* __restrict__ u, const float2* 
 __global__ void k_cg_upd(int64_t n, const double* __restrict__ pqpart, int npq, int j, float2* __restrict__ x,
                          const float2* __restrict__ p, const float2* __restrict__ r, const float2* __restrict__ q,
                          float2* __restrict__ rn, double* partials, unsigned* counter, TapeHeader* H) {
+  pdl_sync(pqpart, x, p, r, q, rn, partials, counter, H);
   __shared__ float s_alpha;
   const double rho = H->rho[j];
   if (threadIdx.x < 32) {
@@ -162,6 +168,7 @@ __global__ void k_cg_upd(int64_t n, const double* __restrict__ pqpart, int npq, 
 // p_{j+1} = r_{j+1} + beta_j p_j
 __global__ void k_cg_dir(int64_t n, const TapeHeader* __restrict__ H, int j, const float2* __restrict__ r,
                          const float2* __restrict__ p, float2* __restrict__ pn) {
+  pdl_sync(H, r, p, pn);
   const float beta = (float)H->beta[j];
   DGRID(i, n) pn[i] = make_float2(fmaf(beta, p[i].x, r[i].x), fmaf(beta, p[i].y, r[i].y));
 }
@@ -171,6 +178,7 @@ __global__ void k_cg_dir(int64_t n, const TapeHeader* __restrict__ H, int j, con
 __global__ void k_b1_fwd(int64_t n, float2* __restrict__ a1, const float2* __restrict__ z1,
                          const float* __restrict__ om, float gamma, float2* __restrict__ z1o,
                          float2* __restrict__ u1) {
+  pdl_sync(a1, z1, om, z1o, u1);
   DGRID(i, n) {
     const float2 a = cadd(a1[i], z1[i]);
     a1[i] = a;
@@ -188,6 +196,7 @@ __global__ void k_b1_fwd(int64_t n, float2* __restrict__ a1, const float2* __res
 __global__ void k_b2_a(int64_t n, const float2* __restrict__ s, const float* __restrict__ w,
                        const float2* __restrict__ z2, const float2* __restrict__ y, float2* __restrict__ a2,
                        double eps, double* partials, unsigned* counter, TapeHeader* H) {
+  pdl_sync(s, w, z2, y, a2, partials, counter, H);
   FPair part;
   DGRID(i, n) {
     const float2 a = cadd(cscale(s[i], w[i]), z2[i]);
@@ -209,6 +218,7 @@ __global__ void k_b2_a(int64_t n, const float2* __restrict__ s, const float* __r
 __global__ void k_b2_b(int64_t n, const float2* __restrict__ a2, const float* __restrict__ w,
                        const float2* __restrict__ y, const TapeHeader* __restrict__ H, float2* __restrict__ z2o,
                        float2* __restrict__ u2, float2* __restrict__ t) {
+  pdl_sync(a2, w, y, H, z2o, u2, t);
   const float c = (float)H->cball;
   DGRID(i, n) {
     const float2 yw = cscale(y[i], w[i]);
@@ -224,6 +234,7 @@ __global__ void k_b2_b(int64_t n, const float2* __restrict__ a2, const float* __
 // i = 3 forward: a3 = x_hat' + z3, r3 = max(Re a3, 0), z3' = a3 - r3, x3' = 2 r3 - a3
 __global__ void k_b3_fwd(int64_t n, const float2* __restrict__ xh, const float2* __restrict__ z3,
                          float2* __restrict__ a3o, float2* __restrict__ z3o, float2* __restrict__ x3o) {
+  pdl_sync(xh, z3, a3o, z3o, x3o);
   DGRID(i, n) {
     const float2 a = cadd(xh[i], z3[i]);
     a3o[i] = a;
@@ -255,6 +266,7 @@ __device__ __forceinline__ float2 vjp_soft(float2 a, float lam, float2 rb, float
 
 __global__ void k_vjp_soft(int64_t n, const float2* __restrict__ a, const float* __restrict__ om, float gamma,
                            const float2* __restrict__ rb, float2* __restrict__ ab, float* __restrict__ omb) {
+  pdl_sync(a, om, rb, ab, omb);
   DGRID(i, n) {
     const float w = om ? om[i] : 1.f;
     float dlam;
@@ -266,6 +278,7 @@ __global__ void k_vjp_soft(int64_t n, const float2* __restrict__ a, const float*
 // Positivity r = max(Re a, 0) + 0i (eq. prox3): abar = (Re rbar [Re a > 0], 0).
 __global__ void k_vjp_pos(int64_t n, const float2* __restrict__ a, const float2* __restrict__ rb,
                           float2* __restrict__ ab) {
+  pdl_sync(a, rb, ab);
   DGRID(i, n) ab[i] = make_float2(a[i].x > 0.f ? rb[i].x : 0.f, 0.f);
 }
 
@@ -277,6 +290,7 @@ __global__ void k_vjp_pos(int64_t n, const float2* __restrict__ a, const float2*
 __global__ void k_vjp_ball(int64_t n, const float2* __restrict__ a, const float2* __restrict__ ctr, int outside,
                            float c, float k2, const float2* __restrict__ rb, float2* __restrict__ ab,
                            float2* __restrict__ cb) {
+  pdl_sync(a, ctr, rb, ab, cb);
   DGRID(i, n) {
     if (!outside) {
       ab[i] = rb[i];
@@ -295,6 +309,7 @@ __global__ void k_vjp_ball(int64_t n, const float2* __restrict__ a, const float2
 // z3bar = abar3 and xbar += abar3 (x_hat' feeds a3)
 __global__ void k_b3_bwd(int64_t n, const float2* __restrict__ a3, const float2* __restrict__ z3b_o,
                          const float2* __restrict__ x3b_o, float2* __restrict__ z3b_i, float2* __restrict__ xacc) {
+  pdl_sync(a3, z3b_o, x3b_o, z3b_i, xacc);
   DGRID(i, n) {
     const float2 zb = z3b_o[i], xb = x3b_o[i];
     const float rbx = 2.f * xb.x - zb.x;
@@ -310,6 +325,7 @@ __global__ void k_b3_bwd(int64_t n, const float2* __restrict__ a3, const float2*
 // holds z1bar' on entry), omega_bar += gamma dL/dlam
 __global__ void k_b1_bwd(int64_t n, const float2* __restrict__ a1, const float* __restrict__ om, float gamma,
                          const float2* __restrict__ ub, float2* __restrict__ z1b, float* __restrict__ omb) {
+  pdl_sync(a1, om, ub, z1b, omb);
   DGRID(i, n) {
     const float2 zb = z1b[i], u = ub[i];
     const float2 rb = make_float2(2.f * u.x - zb.x, 2.f * u.y - zb.y);
@@ -326,6 +342,7 @@ __global__ void k_b1_bwd(int64_t n, const float2* __restrict__ a1, const float* 
 __global__ void k_b2_bwd1(int64_t n, const float2* __restrict__ g, const float* __restrict__ w,
                           const float2* __restrict__ u2, const float2* __restrict__ z2b_o, float2* __restrict__ rb,
                           float2* __restrict__ ab, float* __restrict__ wb) {
+  pdl_sync(g, w, u2, z2b_o, rb, ab, wb);
   DGRID(i, n) {
     const float2 ub = cscale(g[i], w[i]);
     wb[i] += g[i].x * u2[i].x + g[i].y * u2[i].y;
@@ -342,6 +359,7 @@ __global__ void k_b2_bwd2(int64_t n, const float2* __restrict__ a2, const float*
                           const float2* __restrict__ y, int outside, float c, const BwdScalars* __restrict__ S,
                           const float2* __restrict__ rb, float2* __restrict__ ab, const float2* __restrict__ phx, float* __restrict__ wb,
                           float2* __restrict__ z2b_i, float2* __restrict__ t) {
+  pdl_sync(a2, w, y, S, rb, ab, phx, wb, z2b_i, t);
   const float k2 = outside ? (float)S->k2 : 0.f;
   DGRID(i, n) {
     const float2 yw = cscale(y[i], w[i]);
@@ -364,6 +382,7 @@ __global__ void k_b2_bwd2(int64_t n, const float2* __restrict__ a2, const float*
 // <x_bar, p> for the last step run, before the reverse CG (S is zeroed first)
 __global__ void k_cgb_first(int64_t n, const float2* __restrict__ xb, const float2* __restrict__ p, double* partials,
                             unsigned* counter, BwdScalars* S) {
+  pdl_sync(xb, p, partials, counter, S);
   FPair part;
   DGRID(i, n) {
     part.add_prod(xb[i].x, p[i].x);
@@ -378,6 +397,7 @@ __global__ void k_cgb_first(int64_t n, const float2* __restrict__ xb, const floa
 __global__ void k_cgb_r(int64_t n, float2* __restrict__ rb, const float2* __restrict__ pb,
                         const float2* __restrict__ r, const float2* __restrict__ q, int j, double* partials,
                         unsigned* counter, const TapeHeader* __restrict__ H, BwdScalars* S) {
+  pdl_sync(rb, pb, r, q, partials, counter, H, S);
   const float tr = (float)(2.0 * S->rhob);
   FPair part;
   DGRID(i, n) {
@@ -401,6 +421,7 @@ __global__ void k_cgb_r(int64_t n, float2* __restrict__ rb, const float2* __rest
 // q_bar = -alpha r_bar + pi_bar p
 __global__ void k_cgb_q(int64_t n, const TapeHeader* __restrict__ H, const BwdScalars* __restrict__ S, int j,
                         const float2* __restrict__ rb, const float2* __restrict__ p, float2* __restrict__ qb) {
+  pdl_sync(H, S, rb, p, qb);
   const float alpha = (float)H->alpha[j], pib = (float)S->pib;
   DGRID(i, n) qb[i] = make_float2(fmaf(-alpha, rb[i].x, pib * p[i].x), fmaf(-alpha, rb[i].y, pib * p[i].y));
 }
@@ -412,6 +433,7 @@ __global__ void k_cgb_p(int64_t n, const TapeHeader* __restrict__ H, int j, floa
                         const float2* __restrict__ xb, const float2* __restrict__ q, const float2* __restrict__ v,
                         const float2* __restrict__ qb, const float2* __restrict__ pprev, double* partials,
                         unsigned* counter, BwdScalars* S) {
+  pdl_sync(H, pb, xb, q, v, qb, pprev, partials, counter, S);
   const float beta = (float)H->beta[j], alpha = (float)H->alpha[j], pib = (float)S->pib;
   FPair part[2];
   DGRID(i, n) {
@@ -439,6 +461,7 @@ __global__ void k_cgb_p(int64_t n, const TapeHeader* __restrict__ H, int j, floa
 __global__ void k_cgb_end(int64_t n, const float2* __restrict__ xb, const float2* __restrict__ v,
                           const float2* __restrict__ rb, float2* __restrict__ xb0, float2* __restrict__ b1,
                           float2* __restrict__ b2, float2* __restrict__ b3) {
+  pdl_sync(xb, v, rb, xb0, b1, b2, b3);
   DGRID(i, n) {
     const float2 r = rb[i];
     xb0[i] = make_float2(xb[i].x - v[i].x - 2.f * r.x, xb[i].y - v[i].y - 2.f * r.y);
@@ -450,6 +473,7 @@ __global__ void k_cgb_end(int64_t n, const float2* __restrict__ xb, const float2
 
 // out = a + b
 __global__ void k_add(int64_t n, const float2* __restrict__ a, const float2* __restrict__ b, float2* __restrict__ out) {
+  pdl_sync(a, b, out);
   DGRID(i, n) out[i] = cadd(a[i], b[i]);
 }
 
@@ -528,7 +552,7 @@ int phi_adj_into(purify_ctx* c, const float2* u, float2* out, cudaStream_t s) {
 
 int host_dot(purify_ctx* c, int64_t n, const float2* a, const float2* b, double* out, cudaStream_t s) {
   double* slot = &c->d_sc->norm2;
-  k_dot<<<dblocks(n), 256, 0, s>>>(n, a, b, c->d_partials + kCntNorm * 2 * kMaxPartials, &c->d_sc->counter[kCntNorm],
+  pdl_launch(k_dot, LaunchCfg{dblocks(n), 256, 0, s}, n, a, b, c->d_partials + kCntNorm * 2 * kMaxPartials, &c->d_sc->counter[kCntNorm],
                                   slot);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   if (int rc = check_cuda(cudaGetLastError())) return rc;
@@ -598,12 +622,12 @@ int diff_forward(purify_ctx* c, const DiffArgs& A, float2* const* in, float2* co
   // ---- step 5: b = x1 + x2 + x3; r0 = b - Q_w x0; CG from x0 = x_hat
   float2* b = im[0];
   float2* x = out[0];
-  LAUNCH((k_sum3<<<dblocks(N), 256, 0, s>>>(N, in[4], in[5], in[6], b)));
+  LAUNCH((pdl_launch(k_sum3, LaunchCfg{dblocks(N), 256, 0, s}, N, in[4], in[5], in[6], b)));
   if (int rc = check_cuda(cudaMemcpyAsync(x, in[0], N * sizeof(float2), cudaMemcpyDeviceToDevice, s))) return rc;
   RowOutArgs ra{};
   ra.out = im[1];
   if (int rc = apply_ww(c, x, A.w, T.PhiX0, m[0], kRowOutPlain, ra, s)) return rc;
-  LAUNCH((k_resid0<<<dblocks(N), 256, 0, s>>>(N, b, im[1], x, T.R, k > 0 ? T.P : nullptr, k, part, cnt, H)));
+  LAUNCH((pdl_launch(k_resid0, LaunchCfg{dblocks(N), 256, 0, s}, N, b, im[1], x, T.R, k > 0 ? T.P : nullptr, k, part, cnt, H)));
   // rho_0 = 0 (the zero state of the first iteration): no step is run, as in the oracle
   double rho0 = 0.0;
   if (k > 0) {
@@ -618,22 +642,22 @@ int diff_forward(purify_ctx* c, const DiffArgs& A, float2* const* in, float2* co
     ra.out = qj;
     ra.p = pj;
     if (int rc = apply_ww(c, pj, A.w, T.PhiP + (int64_t)j * M, m[0], kRowOutCgQ, ra, s)) return rc;
-    LAUNCH((k_cg_upd<<<dblocks(N), 256, 0, s>>>(N, c->d_partials + kCntDot * 2 * kMaxPartials + kMaxPartials,
+    LAUNCH((pdl_launch(k_cg_upd, LaunchCfg{dblocks(N), 256, 0, s}, N, c->d_partials + kCntDot * 2 * kMaxPartials + kMaxPartials,
                                                 cg_partial_blocks(c), j, x, pj, rj, qj, rj + N, part, cnt, H)));
-    if (j + 1 < k) LAUNCH((k_cg_dir<<<dblocks(N), 256, 0, s>>>(N, H, j, rj + N, pj, pj + N)));
+    if (j + 1 < k) LAUNCH((pdl_launch(k_cg_dir, LaunchCfg{dblocks(N), 256, 0, s}, N, H, j, rj + N, pj, pj + N)));
   }
   // ---- i = 1: a1 = Psi^H x_hat' + z1; z1', x1' = Psi (2 r1 - a1)
   SaraProxArgs pa{};
   if (int rc = sara_analysis(c, x, T.A1, kSaraPlain, pa, s)) return rc;
-  LAUNCH((k_b1_fwd<<<dblocks(D), 256, 0, s>>>(D, T.A1, in[1], A.om, (float)A.gamma, out[1], T.U1)));
+  LAUNCH((pdl_launch(k_b1_fwd, LaunchCfg{dblocks(D), 256, 0, s}, D, T.A1, in[1], A.om, (float)A.gamma, out[1], T.U1)));
   if (int rc = sara_synthesis(c, T.U1, out[4], s)) return rc;
   // ---- i = 2: a2 = w o Phi x_hat' + z2; projection onto the ball around y_w
   if (int rc = phi_into(c, x, T.PhiXh, s)) return rc;
-  LAUNCH((k_b2_a<<<dblocks(M), 256, 0, s>>>(M, T.PhiXh, A.w, in[2], A.y, T.A2, A.eps, part, cnt, H)));
-  LAUNCH((k_b2_b<<<dblocks(M), 256, 0, s>>>(M, T.A2, A.w, A.y, H, out[2], T.U2, m[1])));
+  LAUNCH((pdl_launch(k_b2_a, LaunchCfg{dblocks(M), 256, 0, s}, M, T.PhiXh, A.w, in[2], A.y, T.A2, A.eps, part, cnt, H)));
+  LAUNCH((pdl_launch(k_b2_b, LaunchCfg{dblocks(M), 256, 0, s}, M, T.A2, A.w, A.y, H, out[2], T.U2, m[1])));
   if (int rc = phi_adj_into(c, m[1], out[5], s)) return rc;
   // ---- i = 3
-  LAUNCH((k_b3_fwd<<<dblocks(N), 256, 0, s>>>(N, x, in[3], T.A3, out[3], out[6])));
+  LAUNCH((pdl_launch(k_b3_fwd, LaunchCfg{dblocks(N), 256, 0, s}, N, x, in[3], T.A3, out[3], out[6])));
   return check_cuda(cudaStreamSynchronize(s));
 }
 
@@ -656,24 +680,24 @@ int diff_backward(purify_ctx* c, const DiffArgs& A, float2* const* in, const voi
   float2* xacc = im[0];  // adjoint of x_hat' (the CG output)
   if (int rc = check_cuda(cudaMemcpyAsync(xacc, ob[0], N * sizeof(float2), cudaMemcpyDeviceToDevice, s))) return rc;
   // ---- i = 3
-  LAUNCH((k_b3_bwd<<<dblocks(N), 256, 0, s>>>(N, T.A3, ob[3], ob[6], ib[3], xacc)));
+  LAUNCH((pdl_launch(k_b3_bwd, LaunchCfg{dblocks(N), 256, 0, s}, N, T.A3, ob[3], ob[6], ib[3], xacc)));
   // ---- i = 1: ubar = Psi^H x1bar'; z1bar; x_bar += Psi abar1
   if (int rc = check_cuda(cudaMemcpyAsync(ib[1], ob[1], D * sizeof(float2), cudaMemcpyDeviceToDevice, s))) return rc;
   SaraProxArgs pa{};
   if (int rc = sara_analysis(c, ob[4], dv, kSaraPlain, pa, s)) return rc;
-  LAUNCH((k_b1_bwd<<<dblocks(D), 256, 0, s>>>(D, T.A1, A.om, (float)A.gamma, dv, ib[1], omb)));
+  LAUNCH((pdl_launch(k_b1_bwd, LaunchCfg{dblocks(D), 256, 0, s}, D, T.A1, A.om, (float)A.gamma, dv, ib[1], omb)));
   if (int rc = sara_synthesis(c, ib[1], im[1], s)) return rc;
-  LAUNCH((k_add<<<dblocks(N), 256, 0, s>>>(N, xacc, im[1], xacc)));
+  LAUNCH((pdl_launch(k_add, LaunchCfg{dblocks(N), 256, 0, s}, N, xacc, im[1], xacc)));
   // ---- i = 2: g = Phi x2bar'; through the ball; x_bar += Phi^H (w o abar2)
   if (int rc = phi_into(c, ob[5], m[0], s)) return rc;
-  LAUNCH((k_b2_bwd1<<<dblocks(M), 256, 0, s>>>(M, m[0], A.w, T.U2, ob[2], m[1], m[2], wb)));
+  LAUNCH((pdl_launch(k_b2_bwd1, LaunchCfg{dblocks(M), 256, 0, s}, M, m[0], A.w, T.U2, ob[2], m[1], m[2], wb)));
   const int outside = H.nd > A.eps ? 1 : 0;
   if (outside)  // <d, rbar2>, d = a2 - y_w (FP64): the ball's Jacobian needs it
-    LAUNCH((k_dot_wdiff<<<dblocks(M), 256, 0, s>>>(M, T.A2, A.w, A.y, m[1], part, cnt, dH, S)));
-  LAUNCH((k_b2_bwd2<<<dblocks(M), 256, 0, s>>>(M, T.A2, A.w, A.y, outside, (float)H.cball, S, m[1], m[2], T.PhiXh,
+    LAUNCH((pdl_launch(k_dot_wdiff, LaunchCfg{dblocks(M), 256, 0, s}, M, T.A2, A.w, A.y, m[1], part, cnt, dH, S)));
+  LAUNCH((pdl_launch(k_b2_bwd2, LaunchCfg{dblocks(M), 256, 0, s}, M, T.A2, A.w, A.y, outside, (float)H.cball, S, m[1], m[2], T.PhiXh,
                                                wb, ib[2], m[0])));
   if (int rc = phi_adj_into(c, m[0], im[1], s)) return rc;
-  LAUNCH((k_add<<<dblocks(N), 256, 0, s>>>(N, xacc, im[1], xacc)));
+  LAUNCH((pdl_launch(k_add, LaunchCfg{dblocks(N), 256, 0, s}, N, xacc, im[1], xacc)));
   // ---- step 5: CG reversed (x_bar stays xacc through every step)
   float2* rb = im[1];
   float2* pb = im[2];
@@ -684,21 +708,21 @@ int diff_backward(purify_ctx* c, const DiffArgs& A, float2* const* in, const voi
   RowOutArgs ra{};
   ra.out = vN;
   if (H.steps > 0)
-    LAUNCH((k_cgb_first<<<dblocks(N), 256, 0, s>>>(N, xacc, T.P + (int64_t)(H.steps - 1) * N, part, cnt, S)));
+    LAUNCH((pdl_launch(k_cgb_first, LaunchCfg{dblocks(N), 256, 0, s}, N, xacc, T.P + (int64_t)(H.steps - 1) * N, part, cnt, S)));
   for (int j = H.steps - 1; j >= 0; --j) {
     const float2* pj = T.P + (int64_t)j * N;
     const float2* qj = T.Qp + (int64_t)j * N;
-    LAUNCH((k_cgb_r<<<dblocks(N), 256, 0, s>>>(N, rb, pb, T.R + (int64_t)(j + 1) * N, qj, j, part, cnt, dH, S)));
-    LAUNCH((k_cgb_q<<<dblocks(N), 256, 0, s>>>(N, dH, S, j, rb, pj, qb)));
+    LAUNCH((pdl_launch(k_cgb_r, LaunchCfg{dblocks(N), 256, 0, s}, N, rb, pb, T.R + (int64_t)(j + 1) * N, qj, j, part, cnt, dH, S)));
+    LAUNCH((pdl_launch(k_cgb_q, LaunchCfg{dblocks(N), 256, 0, s}, N, dH, S, j, rb, pj, qb)));
     // v = Phi_w^H Phi_w qbar; w_bar += 2 w Re(conj(Phi qbar) Phi p_j)
     if (int rc = apply_ww(c, qb, A.w, nullptr, m[1], kRowOutPlain, ra, s, T.PhiP + (int64_t)j * M, 2.f, wb)) return rc;
-    LAUNCH((k_cgb_p<<<dblocks(N), 256, 0, s>>>(N, dH, j, pb, xacc, qj, vN, qb, j > 0 ? pj - N : nullptr, part, cnt, S)));
+    LAUNCH((pdl_launch(k_cgb_p, LaunchCfg{dblocks(N), 256, 0, s}, N, dH, j, pb, xacc, qj, vN, qb, j > 0 ? pj - N : nullptr, part, cnt, S)));
   }
   // p_0 = r_0 and rho_0 = <r_0, r_0>
-  LAUNCH((k_cgb_r<<<dblocks(N), 256, 0, s>>>(N, rb, pb, T.R, nullptr, 0, part, cnt, dH, S)));
+  LAUNCH((pdl_launch(k_cgb_r, LaunchCfg{dblocks(N), 256, 0, s}, N, rb, pb, T.R, nullptr, 0, part, cnt, dH, S)));
   // r_0 = b - Q_w x_0: b_bar = r_bar; x0_bar = x_bar - Q_w r_bar; w term
   if (int rc = apply_ww(c, rb, A.w, nullptr, m[1], kRowOutPlain, ra, s, T.PhiX0, -2.f, wb)) return rc;
-  LAUNCH((k_cgb_end<<<dblocks(N), 256, 0, s>>>(N, xacc, vN, rb, ib[0], ib[4], ib[5], ib[6])));
+  LAUNCH((pdl_launch(k_cgb_end, LaunchCfg{dblocks(N), 256, 0, s}, N, xacc, vN, rb, ib[0], ib[4], ib[5], ib[6])));
   return check_cuda(cudaStreamSynchronize(s));
 }
 
@@ -786,7 +810,7 @@ int purify_diff_penalty(purify_ctx* c, const float* y, const float* wvis, double
   if (rc == PURIFY_OK) {
     // Phi_w^H y_w = Phi^H (w^2 o y), then Psi^H, then the largest modulus
     const int64_t M = c->M;
-    k_wmul<<<dblocks(M), 256, 0, s>>>(M, (const float2*)y, wvis, 2, m[0]);
+    pdl_launch(k_wmul, LaunchCfg{dblocks(M), 256, 0, s}, M, (const float2*)y, wvis, 2, m[0]);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     rc = check_cuda(cudaGetLastError());
     if (rc == PURIFY_OK) rc = phi_adj_into(c, m[0], im[0], s);
@@ -809,7 +833,7 @@ int purify_vjp_soft_threshold(int64_t count, const float* a, const float* w, flo
   if (!ok_dev(a) || !ok_dev(rbar) || !ok_dev(abar) || (w && !ok_dev(w)) || (wbar && !ok_dev(wbar)))
     return PURIFY_E_NOT_DEVICE_PTR;
   cudaStream_t s = (cudaStream_t)stream;
-  k_vjp_soft<<<dblocks(count), 256, 0, s>>>(count, (const float2*)a, w, gamma, (const float2*)rbar, (float2*)abar,
+  pdl_launch(k_vjp_soft, LaunchCfg{dblocks(count), 256, 0, s}, count, (const float2*)a, w, gamma, (const float2*)rbar, (float2*)abar,
                                             wbar);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return check_cuda(cudaGetLastError());
@@ -820,7 +844,7 @@ int purify_vjp_positive(int64_t count, const float* a, const float* rbar, float*
   if (count == 0) return PURIFY_OK;
   if (!ok_dev(a) || !ok_dev(rbar) || !ok_dev(abar)) return PURIFY_E_NOT_DEVICE_PTR;
   cudaStream_t s = (cudaStream_t)stream;
-  k_vjp_pos<<<dblocks(count), 256, 0, s>>>(count, (const float2*)a, (const float2*)rbar, (float2*)abar);
+  pdl_launch(k_vjp_pos, LaunchCfg{dblocks(count), 256, 0, s}, count, (const float2*)a, (const float2*)rbar, (float2*)abar);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return check_cuda(cudaGetLastError());
 }
@@ -850,7 +874,7 @@ int purify_vjp_l2ball(purify_ctx* c, int64_t count, const float* a, const float*
       const int outside = nd > eps ? 1 : 0;
       const double cb = outside ? eps / nd : 1.0;
       const float k2 = outside ? (float)(cb * (ar - yr) / nd2) : 0.f;
-      k_vjp_ball<<<dblocks(count), 256, 0, s>>>(count, A, Y, outside, (float)cb, k2, RB, (float2*)abar,
+      pdl_launch(k_vjp_ball, LaunchCfg{dblocks(count), 256, 0, s}, count, A, Y, outside, (float)cb, k2, RB, (float2*)abar,
                                                  (float2*)ybar);
       g_launches.fetch_add(1, std::memory_order_relaxed);
       rc = check_cuda(cudaGetLastError());

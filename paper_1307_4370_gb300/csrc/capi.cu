@@ -606,6 +606,7 @@ int cg_step(purify_ctx* c, float2* x, float2* r, float2* p, float2* sv, float2* 
   ia.p = p;
   ia.s = sv;
   ia.w = w;
+  ia.first = i == 0;  // (the first kernel of a captured iteration)
   TRY(phi_forward_grid(c, i == 0 ? kRowInPlain : kRowInCgUpd, ia, s, i - 1));  // applies step i - 1's update
   TRY(gram_grid(c, s));  // G^T G in one pass (the M samples are not stored)
   RowOutArgs ra{};
@@ -645,6 +646,7 @@ int enqueue_sdmm_step(purify_ctx* c, purify_sdmm_state* st, cudaStream_t s) {
   ia.p = st->p;
   ia.s = st->sv;
   ia.w = st->qp;
+  ia.first = k == 0;
   TRY(phi_forward_grid(c, k > 0 ? kRowInCgFinish : kRowInPlain, ia, s, k - 1));
   // steps 7-9: the branches are independent until the next residual (§4.5:
   // the proximity operators can run in parallel).  i = 1 (the prior) on the

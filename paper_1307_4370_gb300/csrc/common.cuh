@@ -205,6 +205,54 @@ inline void allow_smem(K kernel, size_t bytes) {
   if (bytes > 40 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
+// ---------------------------------------------------------------------------
+// Programmatic dependent launch.  The iteration is a chain of 65 short kernels
+// (3-15 us), so the launch latency of each is worth hiding behind its
+// predecessor: a kernel launched with pdl_launch may be set up while the CTAs
+// of the kernel before it on the stream are exiting, and waits in pdl_sync
+// until that kernel has completed and its writes are visible.  Every kernel
+// launched this way calls pdl_sync in every CTA before it reads or writes
+// anything another kernel of the chain touches; tables fixed at set-up may be
+// read before.  No kernel lets its successor start earlier
+// (griddepcontrol.launch_dependents): with that at the top of every kernel the
+// waiting CTAs took the slots of the two branches of an iteration (256^2
+// iteration 424 us, 332 without it, 351 with plain launches; 256^2 CG of ten
+// steps 426, 314 and 449 us).  So a kernel that passes pdl_sync follows all
+// earlier kernels of the chain, not only the last one.
+//
+// pdl_sync moves its pointer arguments past the wait: each gets an offset
+// (zero) that the wait's asm statement produces, so no access through a
+// __restrict__ or read-only pointer can be scheduled before it.
+// ---------------------------------------------------------------------------
+template <class... P>
+__device__ __forceinline__ void pdl_sync(P&... p) {
+  int zero;
+  asm volatile("griddepcontrol.wait;\n mov.u32 %0, 0;" : "=r"(zero)::"memory");
+  ((p += zero), ...);
+}
+
+struct LaunchCfg {
+  dim3 grid, block;
+  size_t smem;
+  cudaStream_t stream;
+  bool chained = true;  // false: a plain launch (the stream has just waited on another one)
+};
+
+template <class... P, class... A>
+inline void pdl_launch(void (*kernel)(P...), const LaunchCfg& c, A&&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = c.grid;
+  cfg.blockDim = c.block;
+  cfg.dynamicSmemBytes = c.smem;
+  cfg.stream = c.stream;
+  cfg.attrs = &at;
+  cfg.numAttrs = c.chained ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+
 constexpr int kMaxPartials = 32768;  // blocks per reduction (NV <= 2 values each)
 constexpr int kMaxBlocks = 4096;     // data blocks of the distributed form
 
@@ -460,6 +508,7 @@ enum GridIn { kGridPerm = 0, kGridSorted = 1, kGridGram = 2 };
 enum RowOutMode { kRowOutPlain = 0, kRowOutCgQ = 1, kRowOutSdmm = 2 };
 
 struct RowInArgs {
+  bool first;           // first kernel after a stream or graph boundary (plain launch)
   const float2* in;     // plain: the image to transform
   // CG (single-reduction form): the pending update of step i-1 is
   //   p = r + beta p; s = w + beta s; x += alpha p; r -= alpha s

@@ -21,6 +21,7 @@ __global__ void __launch_bounds__(256) k_degrid(const float2* __restrict__ X, co
                                                 const int* __restrict__ perm, DegridArgs a,
                                                 const int4* __restrict__ dchunks, KbPoly kb, KappaScale ks, int L,
                                                 int T, int tiles_1d, double* partials, DevScalars* sc) {
+  pdl_sync(X, uv, perm, dchunks, partials, sc);
   extern __shared__ float2 halo[];
   constexpr int NT = 256;
   const int W = T + J - 1, NW = W * W;
@@ -241,6 +242,7 @@ __global__ void __launch_bounds__(kGridThreads, MINB) k_grid(float2* __restrict_
                                                        const int* __restrict__ dense_tiles,
                                                        const float* __restrict__ H,
                                                        const int* __restrict__ gram_chunks, int dense_half) {
+  pdl_sync(X, Xin, perm, vis, list, chunks, tab, items, item_row, tile_slot0, tile_nchunk, tile_cnt, slots, sc, dense_tiles, H, gram_chunks);
   constexpr int NT = kGridThreads;
   constexpr int S = grid_wstride(J);  // [0 wr_0 .. wr_{J-1} 0 | 0 wc_0 .. wc_{J-1} 0 | pad]
   extern __shared__ __align__(128) float4 sm4[];
@@ -603,7 +605,7 @@ static void degrid_J(purify_ctx* c, DegridOut mode, const DegridArgs& a, cudaStr
   do {                                                                                                        \
     allow_smem(k_degrid<J, MD>, sm);                                                                          \
     PURIFY_LAUNCH(c, "degrid", s,                                                                             \
-                  (k_degrid<J, MD><<<c->ndchunks, threads, sm, s>>>(c->d_grid, c->d_uv, c->d_perm, a, c->d_dchunks, \
+                  (pdl_launch(k_degrid<J, MD>, LaunchCfg{c->ndchunks, threads, sm, s}, c->d_grid, c->d_uv, c->d_perm, a, c->d_dchunks, \
                                                                     c->kb, c->ks, c->L, c->tileT, c->tiles_1d,     \
                                                                     c->d_partials, c->d_sc)));                     \
   } while (0)
@@ -638,8 +640,7 @@ static void grid_JB(purify_ctx* c, GridIn mode, const float2* vis, size_t sm, cu
   do {                                                                                                         \
     allow_smem(k_grid<J, MD, MINB>, sm);                                                                       \
     PURIFY_LAUNCH(c, NAME, s,                                                                                  \
-                  (k_grid<J, MD, MINB><<<MD == kGridGram ? c->n_dense + c->n_gram_chunks : c->nchunks,       \
-                                         kGridThreads, sm, s>>>(                                               \
+                  (pdl_launch(k_grid<J, MD, MINB>, LaunchCfg{MD == kGridGram ? c->n_dense + c->n_gram_chunks : c->nchunks, kGridThreads, sm, s},                                                \
                       OUT, IN, c->d_perm, vis, c->d_list, c->d_chunks, c->d_chunk_tab, c->chunk_tab_stride,     \
                       c->d_items, c->d_item_row,                                                                \
                       c->d_tile_slot0, c->d_tile_nchunk,                                                        \

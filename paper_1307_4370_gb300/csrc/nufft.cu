@@ -147,6 +147,7 @@ __global__ void __launch_bounds__(256) k_row_fwd(RowInArgs a, float2* __restrict
                                                  const float* __restrict__ beam, const float2* __restrict__ tw,
                                                  FftPlan plan, int n, int nsig, DevScalars* sc,
                                                  const double* __restrict__ cgpart, int cg_nblk, int cg_j) {
+  pdl_sync(half, dz, beam, tw, sc, cgpart);
   extern __shared__ float2 sm[];
   const int L = plan.L;
   RowFwdSrc<MODE> src;
@@ -203,6 +204,7 @@ struct ColStoreDst {  // column c0 + s of an L x L grid
 template <int EPT>
 __global__ void __launch_bounds__(1024) k_col_fwd(const float2* __restrict__ half, float2* __restrict__ X,
                                                   const float2* __restrict__ tw, FftPlan plan, int n, int nsig) {
+  pdl_sync(half, X, tw);
   extern __shared__ float2 sm[];
   const int L = plan.L;
   const int c0 = blockIdx.x * nsig;
@@ -239,6 +241,7 @@ struct ColCropDst {
 template <int EPT>
 __global__ void __launch_bounds__(1024) k_col_inv(const float2* __restrict__ X, float2* __restrict__ half,
                                                   const float2* __restrict__ tw, FftPlan plan, int n, int nsig) {
+  pdl_sync(X, half, tw);
   extern __shared__ float2 sm[];
   const int L = plan.L;
   const int c0 = blockIdx.x * nsig;
@@ -332,6 +335,7 @@ __global__ void __launch_bounds__(256) k_row_inv(const float2* __restrict__ half
                                                  const float* __restrict__ dz, const float* __restrict__ beam,
                                                  const float2* __restrict__ tw, FftPlan plan, int n, int nsig,
                                                  double* partials, DevScalars* sc) {
+  pdl_sync(half, dz, beam, tw, partials, sc);
   extern __shared__ float2 sm[];
   const int L = plan.L;
   const int r0 = blockIdx.x * nsig;
@@ -394,6 +398,7 @@ __global__ void __launch_bounds__(NSIG * L / E) k_row_fwd_p2(RowInArgs a, float2
                                                              const float2* __restrict__ twt, int n, DevScalars* sc,
                                                              const double* __restrict__ cgpart, int cg_nblk,
                                                              int cg_j) {
+  pdl_sync(half, dz, beam, twt, sc, cgpart);
   extern __shared__ float2 sm[];
   RowFwdSrc<MODE> src;
   src.a = a;
@@ -422,6 +427,7 @@ __global__ void __launch_bounds__(NSIG * L / E) k_row_fwd_p2(RowInArgs a, float2
 template <int L, int E, int NSIG>
 __global__ void __launch_bounds__(NSIG * L / E) k_col_fwd_p2(const float2* __restrict__ half, float2* __restrict__ X,
                                                              const float2* __restrict__ twt, int n) {
+  pdl_sync(half, X, twt);
   extern __shared__ float2 sm[];
   const int c0 = blockIdx.x * NSIG;
   ColFwdSrc src{half, n, L, c0};
@@ -432,6 +438,7 @@ __global__ void __launch_bounds__(NSIG * L / E) k_col_fwd_p2(const float2* __res
 template <int L, int E, int NSIG>
 __global__ void __launch_bounds__(NSIG * L / E) k_col_inv_p2(const float2* __restrict__ X, float2* __restrict__ half,
                                                              const float2* __restrict__ twt, int n) {
+  pdl_sync(X, half, twt);
   extern __shared__ float2 sm[];
   const int c0 = blockIdx.x * NSIG;
   ColInvSrc src{X, L, c0};
@@ -451,6 +458,7 @@ __global__ void __launch_bounds__(NSIG * L / E, p2_rinv_minb(NSIG * L / E, E, MO
                                                              const float* __restrict__ beam,
                                                              const float2* __restrict__ twt, int n,
                                                              double* partials) {
+  pdl_sync(half, dz, beam, twt, partials);
   extern __shared__ float2 sm[];
   const int r0 = blockIdx.x * NSIG;
   RowInvSrc src{half, L, r0};
@@ -540,7 +548,7 @@ static int p2_forward(purify_ctx* c, RowInMode mode, const RowInArgs& a, cudaStr
     constexpr size_t sm = p2_smem_bytes<L, NS>();
     allow_smem(k_row_fwd_p2<L, C::E, NS, kRowInPlain>, sm);
     PURIFY_LAUNCH(c, "row_fwd", s,
-                  (k_row_fwd_p2<L, C::E, NS, kRowInPlain><<<n / NS, NS * L / C::E, sm, s>>>(
+                  (pdl_launch(k_row_fwd_p2<L, C::E, NS, kRowInPlain>, LaunchCfg{n / NS, NS * L / C::E, sm, s, !a.first},
                       a, c->d_half, c->d_deapod, beam, tw, n, c->d_sc, cgpart, cg_nblk, cg_j)));
   } else {
     constexpr int NS = C::NS_ROWCG;
@@ -549,7 +557,7 @@ static int p2_forward(purify_ctx* c, RowInMode mode, const RowInArgs& a, cudaStr
   do {                                                                                                    \
     allow_smem(k_row_fwd_p2<L, C::E_CG, NS, MD>, sm);                                                     \
     PURIFY_LAUNCH(c, "row_fwd", s,                                                                        \
-                  (k_row_fwd_p2<L, C::E_CG, NS, MD><<<n / NS, NS * L / C::E_CG, sm, s>>>(                  \
+                  (pdl_launch(k_row_fwd_p2<L, C::E_CG, NS, MD>, LaunchCfg{n / NS, NS * L / C::E_CG, sm, s},                   \
                       a, c->d_half, c->d_deapod, beam, twcg, n, c->d_sc, cgpart, cg_nblk, cg_j)));          \
   } while (0)
     if (mode == kRowInCgUpd) ROWCG(kRowInCgUpd);
@@ -561,7 +569,7 @@ static int p2_forward(purify_ctx* c, RowInMode mode, const RowInArgs& a, cudaStr
     constexpr size_t sm = p2_smem_bytes<L, NS>();
     allow_smem(k_col_fwd_p2<L, C::E, NS>, sm);
     PURIFY_LAUNCH(c, "col_fwd", s,
-                  (k_col_fwd_p2<L, C::E, NS><<<L / NS, NS * L / C::E, sm, s>>>(c->d_half, c->d_grid, tw, n)));
+                  (pdl_launch(k_col_fwd_p2<L, C::E, NS>, LaunchCfg{L / NS, NS * L / C::E, sm, s}, c->d_half, c->d_grid, tw, n)));
   }
   return check_cuda(cudaGetLastError());
 }
@@ -577,7 +585,7 @@ static int p2_adjoint(purify_ctx* c, RowOutMode mode, const RowOutArgs& a, cudaS
     constexpr int NS = C::NS_COL;
     constexpr size_t sm = p2_smem_bytes<L, NS>();
     allow_smem(k_col_inv_p2<L, C::E, NS>, sm);
-    PURIFY_LAUNCH(c, "col_inv", s, (k_col_inv_p2<L, C::E, NS><<<L / NS, NS * L / C::E, sm, s>>>(Xg, c->d_half, tw, n)));
+    PURIFY_LAUNCH(c, "col_inv", s, (pdl_launch(k_col_inv_p2<L, C::E, NS>, LaunchCfg{L / NS, NS * L / C::E, sm, s}, Xg, c->d_half, tw, n)));
   }
   if (before_rows) {
     const int rc = check_cuda(cudaStreamWaitEvent(s, before_rows, 0));
@@ -589,7 +597,7 @@ static int p2_adjoint(purify_ctx* c, RowOutMode mode, const RowOutArgs& a, cudaS
   do {                                                                                                     \
     allow_smem(k_row_inv_p2<L, C::E, NS, MD>, sm);                                                         \
     PURIFY_LAUNCH(c, "row_inv", s,                                                                         \
-                  (k_row_inv_p2<L, C::E, NS, MD><<<n / NS, NS * L / C::E, sm, s>>>(c->d_half, a, c->d_deapod, \
+                  (pdl_launch(k_row_inv_p2<L, C::E, NS, MD>, LaunchCfg{n / NS, NS * L / C::E, sm, s, !before_rows}, c->d_half, a, c->d_deapod, \
                                                                                      beam, tw, n,            \
                                                                                      c->d_partials)));       \
   } while (0)
@@ -621,12 +629,13 @@ int cg_consumer_blocks(const purify_ctx* c) {
 // One block: the step sizes of CG step j from the partials, for consumers
 // that read them (cg_consumer_blocks == 0).
 __global__ void __launch_bounds__(256) k_cg_scalars(const double* __restrict__ part, int nblk, int j, DevScalars* sc) {
+  pdl_sync(part, sc);
   cg_consume(part, nblk, j, sc);
 }
 
 int launch_cg_scalars(purify_ctx* c, int cg_j, cudaStream_t s) {
   PURIFY_LAUNCH(c, "cg_scalars", s,
-                (k_cg_scalars<<<1, 256, 0, s>>>(c->d_partials + kCntDot * 2 * kMaxPartials, cg_partial_blocks(c), cg_j,
+                (pdl_launch(k_cg_scalars, LaunchCfg{1, 256, 0, s}, c->d_partials + kCntDot * 2 * kMaxPartials, cg_partial_blocks(c), cg_j,
                                                c->d_sc)));
   return check_cuda(cudaGetLastError());
 }
@@ -651,7 +660,7 @@ int phi_forward_grid(purify_ctx* c, RowInMode mode, const RowInArgs& a, cudaStre
   do {                                                                                                     \
     allow_smem(k_row_fwd<E, MD>, smr);                                                                     \
     PURIFY_LAUNCH(c, "row_fwd", s,                                                                         \
-                  (k_row_fwd<E, MD><<<gr, rs.threads, smr, s>>>(a, c->d_half, c->d_deapod, beam, c->d_tw, c->plan, \
+                  (pdl_launch(k_row_fwd<E, MD>, LaunchCfg{gr, rs.threads, smr, s, !a.first}, a, c->d_half, c->d_deapod, beam, c->d_tw, c->plan, \
                                                                 c->n, rs.nsig, c->d_sc, cgpart, cg_nblk, cg_j)));   \
   } while (0)
   if (rs.ept == 8) {
@@ -671,11 +680,11 @@ int phi_forward_grid(purify_ctx* c, RowInMode mode, const RowInArgs& a, cudaStre
   if (cs.ept == 8) {
     allow_smem(k_col_fwd<8>, smc);
     PURIFY_LAUNCH(c, "col_fwd", s,
-                  (k_col_fwd<8><<<gc, cs.threads, smc, s>>>(c->d_half, c->d_grid, c->d_tw, c->plan, c->n, cs.nsig)));
+                  (pdl_launch(k_col_fwd<8>, LaunchCfg{gc, cs.threads, smc, s}, c->d_half, c->d_grid, c->d_tw, c->plan, c->n, cs.nsig)));
   } else {
     allow_smem(k_col_fwd<12>, smc);
     PURIFY_LAUNCH(c, "col_fwd", s,
-                  (k_col_fwd<12><<<gc, cs.threads, smc, s>>>(c->d_half, c->d_grid, c->d_tw, c->plan, c->n, cs.nsig)));
+                  (pdl_launch(k_col_fwd<12>, LaunchCfg{gc, cs.threads, smc, s}, c->d_half, c->d_grid, c->d_tw, c->plan, c->n, cs.nsig)));
   }
   return check_cuda(cudaGetLastError());
 }
@@ -700,11 +709,11 @@ int phi_adjoint_image(purify_ctx* c, RowOutMode mode, const RowOutArgs& a, cudaS
   if (cs.ept == 8) {
     allow_smem(k_col_inv<8>, smc);
     PURIFY_LAUNCH(c, "col_inv", s,
-                  (k_col_inv<8><<<gc, cs.threads, smc, s>>>(Xg, c->d_half, c->d_tw, c->plan, c->n, cs.nsig)));
+                  (pdl_launch(k_col_inv<8>, LaunchCfg{gc, cs.threads, smc, s}, Xg, c->d_half, c->d_tw, c->plan, c->n, cs.nsig)));
   } else {
     allow_smem(k_col_inv<12>, smc);
     PURIFY_LAUNCH(c, "col_inv", s,
-                  (k_col_inv<12><<<gc, cs.threads, smc, s>>>(Xg, c->d_half, c->d_tw, c->plan, c->n, cs.nsig)));
+                  (pdl_launch(k_col_inv<12>, LaunchCfg{gc, cs.threads, smc, s}, Xg, c->d_half, c->d_tw, c->plan, c->n, cs.nsig)));
   }
   // the row pass may read operands of another stream (the SDMM prior branch)
   if (before_rows) {
@@ -715,7 +724,7 @@ int phi_adjoint_image(purify_ctx* c, RowOutMode mode, const RowOutArgs& a, cudaS
   do {                                                                                                       \
     allow_smem(k_row_inv<E, MD>, smr);                                                                       \
     PURIFY_LAUNCH(c, "row_inv", s,                                                                           \
-                  (k_row_inv<E, MD><<<gr, rs.threads, smr, s>>>(c->d_half, a, c->d_deapod, beam, c->d_tw, c->plan, \
+                  (pdl_launch(k_row_inv<E, MD>, LaunchCfg{gr, rs.threads, smr, s, !before_rows}, c->d_half, a, c->d_deapod, beam, c->d_tw, c->plan, \
                                                                 c->n, rs.nsig, c->d_partials, c->d_sc)));     \
   } while (0)
   if (rs.ept == 8) {

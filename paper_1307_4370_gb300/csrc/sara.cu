@@ -70,6 +70,7 @@ __device__ __forceinline__ float sara_prox(float2 al, size_t j, const SaraProxAr
 template <int MODE>
 __global__ void k_dirac(const float2* __restrict__ x, float2* __restrict__ alpha, int64_t N, float scale,
                         SaraProxArgs pa, double* partials, DevScalars* sc) {
+  pdl_sync(x, alpha, partials, sc);
   float f1 = 0.f;
   const float gamma = (MODE == kSaraProx) ? (float)sc->gamma : 0.f;
   for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < N; j += (int64_t)gridDim.x * blockDim.x) {
@@ -259,6 +260,7 @@ __global__ void __launch_bounds__(256) k_dwt_level(const float2* __restrict__ in
                                                    float2* __restrict__ ll_out, float2* __restrict__ coef,
                                                    LevelGeom G, BasisList bl, WaveletFilters wf,
                                                    SaraProxArgs pa, double* partials, DevScalars* sc) {
+  pdl_sync(in, ll_out, coef, partials, sc);
   extern __shared__ float2 sm[];
   const int k = blockIdx.z;
   const float gamma = (MODE == kSaraProx) ? (float)sc->gamma : 0.f;
@@ -411,6 +413,7 @@ __global__ void __launch_bounds__(256) k_idwt_level(const float2* __restrict__ l
                                                     float2* __restrict__ x, int dirac_plane, LevelGeom G,
                                                     BasisList bl, WaveletFilters wf, const double* f1_part, int f1_n,
                                                     DevScalars* sc) {
+  pdl_sync(ll_in, ll_out, coef, x, f1_part, sc);
   extern __shared__ float2 sm[];
   // with f1 partials to sum, the first z slice is extra (dispatched first, so
   // that its block (0, 0), which forms f1 and zeta, overlaps the tiles)
@@ -511,11 +514,13 @@ __global__ void __launch_bounds__(256) k_idwt_level(const float2* __restrict__ l
 }
 
 __global__ void __launch_bounds__(256) k_f1_finish(const double* __restrict__ part, int n, DevScalars* sc) {
+  pdl_sync(part, sc);
   sara_f1_finish(part, n, sc);
 }
 
 // Dirac-only synthesis: x = alpha_0 / sqrt(q).
 __global__ void k_dirac_syn(const float2* __restrict__ a, float2* __restrict__ x, int64_t N, float scale) {
+  pdl_sync(a, x);
   for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < N; j += (int64_t)gridDim.x * blockDim.x)
     x[j] = cscale(a[j], scale);
 }
@@ -557,6 +562,7 @@ static int tile_for(int H, int64_t planes, int sms) {
 
 // Finish zeta when the dictionary has no wavelet plane (Dirac only).
 __global__ void k_finish_zeta(DevScalars* sc) {
+  pdl_sync(sc);
   const double prev = sc->f1_prev;
   sc->zeta = (prev != 0.0) ? fabs(sc->f1 - prev) / fabs(prev) : INFINITY;
   sc->f1_prev = sc->f1;
@@ -584,14 +590,14 @@ int sara_analysis(purify_ctx* c, const float2* x, float2* alpha, SaraMode mode, 
     int blocks = (int)std::min<int64_t>((N + 255) / 256, 1024);
     if (mode == kSaraPlain)
       PURIFY_LAUNCH(c, "dirac", s,
-                    (k_dirac<kSaraPlain><<<blocks, 256, 0, s>>>(x, alpha + (size_t)dirac_plane * N, N, scale, pa,
+                    (pdl_launch(k_dirac<kSaraPlain>, LaunchCfg{blocks, 256, 0, s, false}, x, alpha + (size_t)dirac_plane * N, N, scale, pa,
                                                                 c->d_partials, c->d_sc)));
     else
       PURIFY_LAUNCH(c, "dirac", s,
-                    (k_dirac<kSaraProx><<<blocks, 256, 0, s>>>(x, nullptr, N, scale, pa, c->d_partials, c->d_sc)));
+                    (pdl_launch(k_dirac<kSaraProx>, LaunchCfg{blocks, 256, 0, s, false}, x, nullptr, N, scale, pa, c->d_partials, c->d_sc)));
   }
   if (nb == 0) {
-    if (mode == kSaraProx) PURIFY_LAUNCH(c, "finish_zeta", s, (k_finish_zeta<<<1, 1, 0, s>>>(c->d_sc)));
+    if (mode == kSaraProx) PURIFY_LAUNCH(c, "finish_zeta", s, (pdl_launch(k_finish_zeta, LaunchCfg{1, 1, 0, s}, c->d_sc)));
     return check_cuda(cudaGetLastError());
   }
   int maxp = 1;
@@ -610,11 +616,11 @@ int sara_analysis(purify_ctx* c, const float2* x, float2* alpha, SaraMode mode, 
     const size_t sm = dwt_smem(TI, 2 * maxp);
     if (mode == kSaraPlain)
       PURIFY_LAUNCH(c, "dwt_level", s,
-                    (k_dwt_level<kSaraPlain><<<grid, 256, sm, s>>>(in, lev == 0, llo, alpha, G, bl, c->wf, pa,
+                    (pdl_launch(k_dwt_level<kSaraPlain>, LaunchCfg{grid, 256, sm, s, lev > 0}, in, lev == 0, llo, alpha, G, bl, c->wf, pa,
                                                                    c->d_partials, c->d_sc)));
     else
       PURIFY_LAUNCH(c, "dwt_level", s,
-                    (k_dwt_level<kSaraProx><<<grid, 256, sm, s>>>(in, lev == 0, llo, pa.z1, G, bl, c->wf, pa,
+                    (pdl_launch(k_dwt_level<kSaraProx>, LaunchCfg{grid, 256, sm, s, lev > 0}, in, lev == 0, llo, pa.z1, G, bl, c->wf, pa,
                                                                   c->d_partials, c->d_sc)));
   }
   if (mode == kSaraProx) {
@@ -622,7 +628,7 @@ int sara_analysis(purify_ctx* c, const float2* x, float2* alpha, SaraMode mode, 
       *f1_parts = f1_off;
     } else {  // no synthesis follows to finish f1: one block does
       PURIFY_LAUNCH(c, "f1_finish", s,
-                    (k_f1_finish<<<1, 256, 0, s>>>(c->d_partials + kCntF1 * 2 * kMaxPartials, f1_off, c->d_sc)));
+                    (pdl_launch(k_f1_finish, LaunchCfg{1, 256, 0, s}, c->d_partials + kCntF1 * 2 * kMaxPartials, f1_off, c->d_sc)));
     }
   }
   return check_cuda(cudaGetLastError());
@@ -636,7 +642,7 @@ int sara_synthesis(purify_ctx* c, const float2* alpha, float2* x, cudaStream_t s
   const float scale = 1.0f / sqrtf((float)c->q);
   if (nb == 0) {
     int blocks = (int)std::min<int64_t>((N + 255) / 256, 1024);
-    PURIFY_LAUNCH(c, "dirac", s, (k_dirac_syn<<<blocks, 256, 0, s>>>(alpha + (size_t)dirac_plane * N, x, N, scale)));
+    PURIFY_LAUNCH(c, "dirac", s, (pdl_launch(k_dirac_syn, LaunchCfg{blocks, 256, 0, s}, alpha + (size_t)dirac_plane * N, x, N, scale)));
     return check_cuda(cudaGetLastError());
   }
   int maxp = 1;
@@ -655,7 +661,7 @@ int sara_synthesis(purify_ctx* c, const float2* alpha, float2* x, cudaStream_t s
     dim3 grid(L / (2 * TO), L / (2 * TO), (lev == 0 ? 1 : nb) + (f1n > 0 ? 1 : 0));
     const size_t sm = idwt_smem(TO, maxp);
     PURIFY_LAUNCH(c, "idwt_level", s,
-                  (k_idwt_level<<<grid, 256, sm, s>>>(llin, from_plane, llo, alpha, x, dirac_plane, G, bl, c->wf,
+                  (pdl_launch(k_idwt_level, LaunchCfg{grid, 256, sm, s}, llin, from_plane, llo, alpha, x, dirac_plane, G, bl, c->wf,
                                                       c->d_partials + kCntF1 * 2 * kMaxPartials, f1n, c->d_sc)));
   }
   return check_cuda(cudaGetLastError());

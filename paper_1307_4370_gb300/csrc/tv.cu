@@ -49,6 +49,7 @@ __device__ __forceinline__ float tv_lambda(const DevScalars* sc, float lam) {
 __global__ void k_tv_init(int64_t N, const float2* __restrict__ xa, const float2* __restrict__ xb,
                           float2* __restrict__ b, float2* __restrict__ r, float2* __restrict__ s,
                           float2* __restrict__ p, float2* __restrict__ q) {
+  pdl_sync(xa, xb, b, r, s, p, q);
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x) {
     b[k] = xb ? cadd(xa[k], xb[k]) : xa[k];
     const float2 z = make_float2(0.f, 0.f);
@@ -64,6 +65,7 @@ __global__ void k_tv_fgp_step(int n, const float2* __restrict__ b, const float2*
                               const float2* __restrict__ s, float2* __restrict__ p, float2* __restrict__ q,
                               float2* __restrict__ r2, float2* __restrict__ s2, const float* __restrict__ w,
                               float cmom, const DevScalars* __restrict__ sc, float lam_host) {
+  pdl_sync(b, r, s, p, q, r2, s2, w, sc);
   const float lam = tv_lambda(sc, lam_host);
   const int64_t N = (int64_t)n * n;
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x) {
@@ -106,6 +108,7 @@ __global__ void k_tv_finish(int n, const float2* __restrict__ b, const float2* _
                             const float2* __restrict__ q, float2* __restrict__ out, float2* __restrict__ z1,
                             const float2* __restrict__ xhat, const float* __restrict__ w, double* partials,
                             DevScalars* sc, float lam_host) {
+  pdl_sync(b, p, q, out, z1, xhat, w, partials, sc);
   const float lam = tv_lambda(z1 ? sc : nullptr, lam_host);
   const int64_t N = (int64_t)n * n;
   FPair f1;
@@ -141,6 +144,7 @@ __global__ void k_tv_finish(int n, const float2* __restrict__ b, const float2* _
 // |grad x| per pixel, as complex (|grad x|, 0) so the complex max and
 // reweighting kernels apply.
 __global__ void k_tv_gradmag(int n, const float2* __restrict__ x, float2* __restrict__ g) {
+  pdl_sync(x, g);
   const int64_t N = (int64_t)n * n;
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x) {
     const int i = (int)k / n, j = (int)k - i * n;
@@ -173,7 +177,7 @@ static int tv_fgp(purify_ctx* c, float2* scratch, const float* w, int iters, con
     t = tn;
     const int a = k & 1;
     PURIFY_LAUNCH(c, "tv_fgp", s,
-                  (k_tv_fgp_step<<<tv_blocks(N), 256, 0, s>>>(c->n, b, r[a], sv[a], p, q, r[a ^ 1], sv[a ^ 1], w, cm,
+                  (pdl_launch(k_tv_fgp_step, LaunchCfg{tv_blocks(N), 256, 0, s}, c->n, b, r[a], sv[a], p, q, r[a ^ 1], sv[a ^ 1], w, cm,
                                                               sc, lam_host)));
   }
   return check_cuda(cudaGetLastError());
@@ -199,11 +203,11 @@ int tv_sdmm_branch(purify_ctx* c, purify_sdmm_state* st, cudaStream_t s) {
   float2* sc_buf = nullptr;
   TV_TRY(tv_scratch_ready(c, &sc_buf));
   PURIFY_LAUNCH(c, "tv_init", s,
-                (k_tv_init<<<tv_blocks(N), 256, 0, s>>>(N, st->xhat, st->z1, sc_buf, sc_buf + N, sc_buf + 2 * N,
+                (pdl_launch(k_tv_init, LaunchCfg{tv_blocks(N), 256, 0, s, false}, N, st->xhat, st->z1, sc_buf, sc_buf + N, sc_buf + 2 * N,
                                                         sc_buf + 5 * N, sc_buf + 6 * N)));
   TV_TRY(tv_fgp(c, sc_buf, st->w, st->fgp_iters, c->d_sc, 0.f, s));
   PURIFY_LAUNCH(c, "tv_finish", s,
-                (k_tv_finish<<<tv_blocks(N), 256, 0, s>>>(c->n, sc_buf, sc_buf + 5 * N, sc_buf + 6 * N, st->x1, st->z1,
+                (pdl_launch(k_tv_finish, LaunchCfg{tv_blocks(N), 256, 0, s}, c->n, sc_buf, sc_buf + 5 * N, sc_buf + 6 * N, st->x1, st->z1,
                                                           st->xhat, st->w, c->d_partials, c->d_sc, 0.f)));
   return check_cuda(cudaGetLastError());
 }
@@ -212,7 +216,7 @@ int tv_sdmm_branch(purify_ctx* c, purify_sdmm_state* st, cudaStream_t s) {
 int tv_gradmag(purify_ctx* c, const float2* x, float2** g, cudaStream_t s) {
   float2* sc_buf = nullptr;
   TV_TRY(tv_scratch_ready(c, &sc_buf));
-  PURIFY_LAUNCH(c, "tv_gradmag", s, (k_tv_gradmag<<<tv_blocks(((int64_t)c->n * c->n)), 256, 0, s>>>(c->n, x, sc_buf)));
+  PURIFY_LAUNCH(c, "tv_gradmag", s, (pdl_launch(k_tv_gradmag, LaunchCfg{tv_blocks(((int64_t)c->n * c->n)), 256, 0, s}, c->n, x, sc_buf)));
   *g = sc_buf;
   return check_cuda(cudaGetLastError());
 }
@@ -223,11 +227,11 @@ int tv_prox(purify_ctx* c, const float2* in, const float* w, float lam, int iter
   float2* sc_buf = nullptr;
   TV_TRY(tv_scratch_ready(c, &sc_buf));
   PURIFY_LAUNCH(c, "tv_init", s,
-                (k_tv_init<<<tv_blocks(N), 256, 0, s>>>(N, in, nullptr, sc_buf, sc_buf + N, sc_buf + 2 * N,
+                (pdl_launch(k_tv_init, LaunchCfg{tv_blocks(N), 256, 0, s}, N, in, nullptr, sc_buf, sc_buf + N, sc_buf + 2 * N,
                                                         sc_buf + 5 * N, sc_buf + 6 * N)));
   TV_TRY(tv_fgp(c, sc_buf, w, iters, nullptr, lam, s));
   PURIFY_LAUNCH(c, "tv_finish", s,
-                (k_tv_finish<<<tv_blocks(N), 256, 0, s>>>(c->n, sc_buf, sc_buf + 5 * N, sc_buf + 6 * N, out, nullptr,
+                (pdl_launch(k_tv_finish, LaunchCfg{tv_blocks(N), 256, 0, s}, c->n, sc_buf, sc_buf + 5 * N, sc_buf + 6 * N, out, nullptr,
                                                           nullptr, nullptr, nullptr, nullptr, lam)));
   return check_cuda(cudaGetLastError());
 }

@@ -24,6 +24,7 @@ static unsigned blocks_for(int64_t n, int threads = 256, int cap = 2048) {
 // §4.4 eq. prox1: a/|a| (|a| - gamma w)^+, with gamma from the host or the device.
 __global__ void k_soft(int64_t n, const float2* __restrict__ in, const float* __restrict__ w,
                        const double* gamma_dev, float gamma, float2* __restrict__ out) {
+  pdl_sync(in, w, gamma_dev, out);
   const float gm = gamma_dev ? (float)*gamma_dev : gamma;
   GRID_STRIDE(j, n) {
     const float2 a = in[j];
@@ -37,6 +38,7 @@ __global__ void k_soft(int64_t n, const float2* __restrict__ in, const float* __
 // ||a - b||^2 in FP64 -> sc->norm2
 __global__ void k_norm_diff(int64_t n, const float2* __restrict__ a, const float2* __restrict__ b,
                             double* partials, DevScalars* sc) {
+  pdl_sync(a, b, partials, sc);
   FPair part;  // per-thread exact sum of a few terms; FP64 across threads
   GRID_STRIDE(j, n) {
     part.add_sq_diff(a[j].x, b[j].x);
@@ -50,6 +52,7 @@ __global__ void k_norm_diff(int64_t n, const float2* __restrict__ a, const float
 // Projection onto {r : ||r - y|| <= eps} given ||in - y||^2 on the device.
 __global__ void k_l2_project(int64_t n, const float2* __restrict__ in, const float2* __restrict__ y, double eps,
                              const double* norm2, float2* __restrict__ out) {
+  pdl_sync(in, y, norm2, out);
   __shared__ float s_scale;  // one FP64 square root per block
   if (threadIdx.x == 0) {
     const double nd = sqrt(*norm2);
@@ -65,6 +68,7 @@ __global__ void k_l2_project(int64_t n, const float2* __restrict__ in, const flo
 
 // §4.4 eq. prox3 with complex entries as real pairs: max(Re a, 0).
 __global__ void k_positive(int64_t n, const float2* __restrict__ in, float2* __restrict__ out) {
+  pdl_sync(in, out);
   GRID_STRIDE(j, n) out[j] = make_float2(fmaxf(in[j].x, 0.f), 0.f);
 }
 
@@ -74,6 +78,7 @@ __global__ void k_positive(int64_t n, const float2* __restrict__ in, float2* __r
 __global__ void k_cg_apply(int64_t n, float2* __restrict__ x, float2* __restrict__ r, float2* __restrict__ p,
                            float2* __restrict__ sv, const float2* __restrict__ w, double* partials, DevScalars* sc,
                            int cg_nblk, int cg_j) {
+  pdl_sync(x, r, p, sv, w, partials, sc);
   const CgStep cs = cg_consume(partials + kCntDot * 2 * kMaxPartials, cg_nblk, cg_j, sc);
   const float al = cs.alpha, be = cs.beta;
   const bool first = cs.first;
@@ -104,11 +109,13 @@ __global__ void k_cg_apply(int64_t n, float2* __restrict__ x, float2* __restrict
 // r = b - Qx (the start of purify_cg_solve).
 __global__ void k_cg_residual_init(int64_t n, const float2* __restrict__ b, const float2* __restrict__ qx,
                                    float2* __restrict__ r, DevScalars* sc) {
+  pdl_sync(b, qx, r, sc);
   GRID_STRIDE(j, n) r[j] = csub(b[j], qx[j]);
 }
 
 // max |a_j| -> sc->amax
 __global__ void k_max_abs(int64_t n, const float2* __restrict__ a, double* partials, DevScalars* sc) {
+  pdl_sync(a, partials, sc);
   float mf = 0.f;
   GRID_STRIDE(j, n) mf = fmaxf(mf, sqrtf(fmaf(a[j].x, a[j].x, a[j].y * a[j].y)));
   // (the maximum of FP32 moduli is one of them: no FP64 needed before the last store)
@@ -135,6 +142,7 @@ __global__ void k_sdmm_l2(int64_t M, const float2* __restrict__ s2, float2* __re
                           const float2* __restrict__ y, const uint16_t* __restrict__ yb,
                           const float* __restrict__ yscale, float2* __restrict__ v, const DevScalars* sc,
                           const int* __restrict__ block_of, const float* __restrict__ bscale) {
+  pdl_sync(s2, z2, y, yb, yscale, v, sc, block_of, bscale);
   const float scale1 = (float)sc->l2_scale;
   GRID_STRIDE(i, M) {
     const float scale = block_of ? bscale[block_of[i]] : scale1;
@@ -168,6 +176,7 @@ __global__ void __launch_bounds__(256) k_block_norms(const int4* __restrict__ bc
                                                      const float* __restrict__ yscale, int R,
                                                      const double* __restrict__ beps, float* __restrict__ bscale,
                                                      double* partials, DevScalars* sc) {
+  pdl_sync(bchunks, pos, s2, z2, y, yb, yscale, beps, bscale, partials, sc);
   const int4 ch = bchunks[blockIdx.x];
   FPair part[2];
   for (int m = ch.y + threadIdx.x; m < ch.z; m += blockDim.x) {
@@ -255,6 +264,7 @@ __global__ void __launch_bounds__(256) k_block_norms(const int4* __restrict__ bc
 // Reweighting (§3.3): w = delta / (delta + |alpha|).
 __global__ void k_reweight(int64_t n, const float2* __restrict__ alpha, float* __restrict__ w, int round,
                            const DevScalars* sc) {
+  pdl_sync(alpha, w, sc);
   __shared__ float s_delta;  // one FP64 power per block (every thread forming it held the kernel at 86 us, 256^2)
   if (threadIdx.x == 0) {
     const double amax = sc->amax;
@@ -274,12 +284,14 @@ __global__ void k_reweight(int64_t n, const float2* __restrict__ alpha, float* _
 
 __global__ void k_gather(int64_t n, const float2* __restrict__ src, const int* __restrict__ perm,
                          float2* __restrict__ dst) {
+  pdl_sync(src, perm, dst);
   GRID_STRIDE(i, n) dst[i] = src[perm[i]];
 }
 
 // bf16 storage of y: one CTA per block of 4096 visibilities, scale = max |component|.
 __global__ void __launch_bounds__(256) k_quantize_bf16(int64_t M, const float2* __restrict__ y,
                                                        uint32_t* __restrict__ yb, float* __restrict__ yscale) {
+  pdl_sync(y, yb, yscale);
   __shared__ float wmax[8];
   const int64_t b0 = (int64_t)blockIdx.x * 4096;
   const int64_t b1 = min(b0 + 4096, M);
@@ -299,56 +311,58 @@ __global__ void __launch_bounds__(256) k_quantize_bf16(int64_t M, const float2* 
   }
 }
 
-__global__ void k_set_gamma(DevScalars* sc, double beta) { sc->gamma = beta * sc->amax; }
+__global__ void k_set_gamma(DevScalars* sc, double beta) {
+  pdl_sync(sc);
+  sc->gamma = beta * sc->amax; }
 
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
 int launch_soft_threshold(int64_t count, const float2* in, const float* w, const double* gamma_dev, float gamma,
                           float2* out, cudaStream_t s) {
-  PURIFY_LAUNCH(nullptr, "soft", s, (k_soft<<<blocks_for(count), 256, 0, s>>>(count, in, w, gamma_dev, gamma, out)));
+  PURIFY_LAUNCH(nullptr, "soft", s, (pdl_launch(k_soft, LaunchCfg{blocks_for(count), 256, 0, s}, count, in, w, gamma_dev, gamma, out)));
   return check_cuda(cudaGetLastError());
 }
 
 int launch_l2_norm_diff(purify_ctx* c, int64_t count, const float2* a, const float2* b, cudaStream_t s) {
-  PURIFY_LAUNCH(c, "norm_diff", s, (k_norm_diff<<<blocks_for(count), 256, 0, s>>>(count, a, b, c->d_partials, c->d_sc)));
+  PURIFY_LAUNCH(c, "norm_diff", s, (pdl_launch(k_norm_diff, LaunchCfg{blocks_for(count), 256, 0, s}, count, a, b, c->d_partials, c->d_sc)));
   return check_cuda(cudaGetLastError());
 }
 
 int launch_l2_project(int64_t count, const float2* in, const float2* y, double eps, const double* norm2_dev,
                       float2* out, cudaStream_t s) {
-  PURIFY_LAUNCH(nullptr, "l2_project", s, (k_l2_project<<<blocks_for(count), 256, 0, s>>>(count, in, y, eps, norm2_dev, out)));
+  PURIFY_LAUNCH(nullptr, "l2_project", s, (pdl_launch(k_l2_project, LaunchCfg{blocks_for(count), 256, 0, s}, count, in, y, eps, norm2_dev, out)));
   return check_cuda(cudaGetLastError());
 }
 
 int launch_positive(int64_t count, const float2* in, float2* out, cudaStream_t s) {
-  PURIFY_LAUNCH(nullptr, "positive", s, (k_positive<<<blocks_for(count), 256, 0, s>>>(count, in, out)));
+  PURIFY_LAUNCH(nullptr, "positive", s, (pdl_launch(k_positive, LaunchCfg{blocks_for(count), 256, 0, s}, count, in, out)));
   return check_cuda(cudaGetLastError());
 }
 
 int launch_cg_apply(purify_ctx* c, float2* x, float2* r, float2* p, float2* sv, const float2* w, int cg_j,
                     cudaStream_t s) {
   const int64_t N = (int64_t)c->n * c->n;
-  PURIFY_LAUNCH(c, "cg_apply", s, (k_cg_apply<<<blocks_for(N), 256, 0, s>>>(N, x, r, p, sv, w, c->d_partials, c->d_sc,
+  PURIFY_LAUNCH(c, "cg_apply", s, (pdl_launch(k_cg_apply, LaunchCfg{blocks_for(N), 256, 0, s}, N, x, r, p, sv, w, c->d_partials, c->d_sc,
                                                                            cg_consumer_blocks(c), cg_j)));
   return check_cuda(cudaGetLastError());
 }
 
 int launch_cg_residual_init(purify_ctx* c, const float2* b, const float2* qx, float2* r, cudaStream_t s) {
   const int64_t N = (int64_t)c->n * c->n;
-  PURIFY_LAUNCH(c, "cg_residual_init", s, (k_cg_residual_init<<<blocks_for(N), 256, 0, s>>>(N, b, qx, r, c->d_sc)));
+  PURIFY_LAUNCH(c, "cg_residual_init", s, (pdl_launch(k_cg_residual_init, LaunchCfg{blocks_for(N), 256, 0, s}, N, b, qx, r, c->d_sc)));
   return check_cuda(cudaGetLastError());
 }
 
 int launch_max_abs(purify_ctx* c, int64_t count, const float2* a, cudaStream_t s) {
-  PURIFY_LAUNCH(c, "max_abs", s, (k_max_abs<<<blocks_for(count), 256, 0, s>>>(count, a, c->d_partials, c->d_sc)));
+  PURIFY_LAUNCH(c, "max_abs", s, (pdl_launch(k_max_abs, LaunchCfg{blocks_for(count), 256, 0, s}, count, a, c->d_partials, c->d_sc)));
   return check_cuda(cudaGetLastError());
 }
 
 int launch_sdmm_l2_update(purify_sdmm_state* st, cudaStream_t s) {
   purify_ctx* c = st->ctx;
   const bool blk = st->nblocks > 0;
-  PURIFY_LAUNCH(st->ctx, "sdmm_l2", s, (k_sdmm_l2<<<blocks_for(c->M), 256, 0, s>>>(c->M, st->s2, st->z2, st->y_bf16 ? nullptr : st->y, st->yb,
+  PURIFY_LAUNCH(st->ctx, "sdmm_l2", s, (pdl_launch(k_sdmm_l2, LaunchCfg{blocks_for(c->M), 256, 0, s}, c->M, st->s2, st->z2, st->y_bf16 ? nullptr : st->y, st->yb,
                                              st->yscale, st->v, c->d_sc, blk ? st->d_block_of : nullptr,
                                              blk ? st->d_bscale : nullptr)));
   return check_cuda(cudaGetLastError());
@@ -357,7 +371,7 @@ int launch_sdmm_l2_update(purify_sdmm_state* st, cudaStream_t s) {
 int launch_block_norms(purify_sdmm_state* st, cudaStream_t s) {
   purify_ctx* c = st->ctx;
   PURIFY_LAUNCH(c, "block_norms", s,
-                (k_block_norms<<<st->nbchunks, 256, 0, s>>>(st->d_bchunks, st->nbchunks, st->d_pos, st->s2, st->z2,
+                (pdl_launch(k_block_norms, LaunchCfg{st->nbchunks, 256, 0, s}, st->d_bchunks, st->nbchunks, st->d_pos, st->s2, st->z2,
                                                             st->y_bf16 ? nullptr : st->y, st->yb, st->yscale,
                                                             st->nblocks, st->d_beps, st->d_bscale,
                                                             c->d_partials + kCntBlk * 2 * kMaxPartials, c->d_sc)));
@@ -365,23 +379,23 @@ int launch_block_norms(purify_sdmm_state* st, cudaStream_t s) {
 }
 
 int launch_reweight(purify_ctx* c, int64_t count, const float2* alpha, float* w, int round, cudaStream_t s) {
-  PURIFY_LAUNCH(c, "reweight", s, (k_reweight<<<blocks_for(count), 256, 0, s>>>(count, alpha, w, round, c->d_sc)));
+  PURIFY_LAUNCH(c, "reweight", s, (pdl_launch(k_reweight, LaunchCfg{blocks_for(count), 256, 0, s}, count, alpha, w, round, c->d_sc)));
   return check_cuda(cudaGetLastError());
 }
 
 int launch_gather_perm(int64_t M, const float2* src, const int* perm, float2* dst, cudaStream_t s) {
-  PURIFY_LAUNCH(nullptr, "gather", s, (k_gather<<<blocks_for(M), 256, 0, s>>>(M, src, perm, dst)));
+  PURIFY_LAUNCH(nullptr, "gather", s, (pdl_launch(k_gather, LaunchCfg{blocks_for(M), 256, 0, s}, M, src, perm, dst)));
   return check_cuda(cudaGetLastError());
 }
 
 int launch_quantize_bf16(int64_t M, const float2* y, uint16_t* yb, float* yscale, cudaStream_t s) {
   const int64_t blocks = (M + 4095) / 4096;
-  PURIFY_LAUNCH(nullptr, "quantize_bf16", s, (k_quantize_bf16<<<(unsigned)blocks, 256, 0, s>>>(M, y, reinterpret_cast<uint32_t*>(yb), yscale)));
+  PURIFY_LAUNCH(nullptr, "quantize_bf16", s, (pdl_launch(k_quantize_bf16, LaunchCfg{(unsigned)blocks, 256, 0, s}, M, y, reinterpret_cast<uint32_t*>(yb), yscale)));
   return check_cuda(cudaGetLastError());
 }
 
 int launch_set_gamma(purify_ctx* c, double beta, cudaStream_t s) {
-  PURIFY_LAUNCH(c, "set_gamma", s, (k_set_gamma<<<1, 1, 0, s>>>(c->d_sc, beta)));
+  PURIFY_LAUNCH(c, "set_gamma", s, (pdl_launch(k_set_gamma, LaunchCfg{1, 1, 0, s}, c->d_sc, beta)));
   return check_cuda(cudaGetLastError());
 }
 
