@@ -110,7 +110,8 @@ constexpr int p2_radix(int L, int E, int st) {
   int rem = L, r = p2_first(L, E);
   for (int i = 0; i < st; ++i) {
     rem /= r;
-    r = p2_min(cap, rem);
+    // (8, 4, 4 at 128: the pruned last stage needs a radix of at least 4)
+    r = rem == 2 * cap && cap == 8 ? 4 : p2_min(cap, rem);
   }
   return r;
 }

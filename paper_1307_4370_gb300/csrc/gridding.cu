@@ -5,6 +5,8 @@
 //              thread (SDMM mode: the FP64 norms of the l2 branch);
 //   k_grid     G^T as an atomic-free gather (and, in the Gram form, G^T G in
 //              one pass for the CG steps).
+#include <algorithm>
+
 #include "common.cuh"
 #include "reduce.cuh"
 
@@ -19,124 +21,140 @@ namespace purify {
 template <int J, int MODE>
 __global__ void __launch_bounds__(256) k_degrid(const float2* __restrict__ X, const float2* __restrict__ uv,
                                                 const int* __restrict__ perm, DegridArgs a,
-                                                const int4* __restrict__ dchunks, KbPoly kb, KappaScale ks, int L,
-                                                int T, int tiles_1d, double* partials, DevScalars* sc) {
+                                                const int4* __restrict__ dchunks, int nchunks, KbPoly kb, KappaScale ks,
+                                                int L, int T, int tiles_1d, double* partials, DevScalars* sc) {
   pdl_sync(X, uv, perm, dchunks, partials, sc);
   extern __shared__ float2 halo[];
   constexpr int NT = 256;
   const int W = T + J - 1, NW = W * W;
-  const int4 ch = dchunks[blockIdx.x];
-  const int tr = ch.x / tiles_1d, tc = ch.x - tr * tiles_1d;
-  const int R0 = tr * T, C0 = tc * T;
-  // the first frequencies of this thread, in flight with the halo loads
-  constexpr int QV = 4;
-  float2 uq[QV];
-#pragma unroll
-  for (int q = 0; q < QV; ++q) {
-    const int i = ch.y + threadIdx.x + q * NT;
-    if (i < ch.z) uq[q] = __ldg(&uv[i]);
-  }
-  // halo of the tile: eight cells per thread per round, all loads issued first
   const float inv_w = 1.0f / (float)W;
-  for (int k0 = 0; k0 < NW; k0 += 8 * NT) {
-    float2 v[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int k = k0 + threadIdx.x + q * NT;
-      if (k < NW) {
-        const int rr = quot_small(k, inv_w), cc = k - rr * W;  // W = T + J - 1 <= 71, k < 2^13
-        int r = R0 + rr, c = C0 + cc;
-        if (r >= L) r -= L;
-        if (c >= L) c -= L;
-        v[q] = __ldg(&X[(size_t)r * L + c]);
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int k = k0 + threadIdx.x + q * NT;
-      if (k < NW) halo[k] = v[q];
-    }
-  }
-  __syncthreads();
   FPair part[2];  // per-thread exact sums of a few terms; FP64 across threads
-  auto visit = [&](int i, float2 u) {
-    int k0r, k0c;
-    float fr, fc;
-    split_kappa(u.x, ks, k0r, fr);
-    split_kappa(u.y, ks, k0c, fc);
-    k0r -= J / 2 - 1;
-    k0c -= J / 2 - 1;
-    float wr[J], wc[J];
-    kb_weights<J>(kb, fr, wr);
-    kb_weights<J>(kb, fc, wc);
-    const int dr = wrap(k0r - R0, L), dc = wrap(k0c - C0, L);
-    float2 acc = make_float2(0.f, 0.f);
-    if (dr < T && dc < T) {
-      const float2* base = halo + dr * W + dc;
-      float2 wcc[J];  // the column weights as (w, w) pairs for the FFMA2s
+  // One chunk per CTA; in the SDMM mode a CTA takes every gridDim-th chunk
+  // (heavy chunks come first, so the shares are even): the norms' partial
+  // sums then end in a few hundred tickets and terms for the last CTA instead
+  // of one per chunk (1024^2, 6000 chunks, beside the prior branch: 119 -> 97 us).
+  for (int q0 = blockIdx.x; q0 < nchunks; q0 += gridDim.x) {
+    const int4 ch = dchunks[q0];
+    const int tr = ch.x / tiles_1d, tc = ch.x - tr * tiles_1d;
+    const int R0 = tr * T, C0 = tc * T;
+    // the first frequencies of this thread, in flight with the halo loads
+    constexpr int QV = 4;
+    float2 uq[QV];
 #pragma unroll
-      for (int b = 0; b < J; ++b) wcc[b] = make_float2(wc[b], wc[b]);
+    for (int q = 0; q < QV; ++q) {
+      const int i = ch.y + threadIdx.x + q * NT;
+      if (i < ch.z) uq[q] = __ldg(&uv[i]);
+    }
+    // halo of the tile: eight cells per thread per round, all loads issued first
+    for (int k0 = 0; k0 < NW; k0 += 8 * NT) {
+      float2 v[8];
 #pragma unroll
-      for (int aa = 0; aa < J; ++aa) {
-        float2 t = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int b = 0; b < J; ++b) t = __ffma2_rn(wcc[b], base[aa * W + b], t);
-        acc = caxpy(wr[aa], t, acc);
-      }
-    } else {
-      // not in this tile (never for a consistent table): read the grid directly
-#pragma unroll
-      for (int aa = 0; aa < J; ++aa) {
-        const float2* row = X + (size_t)wrap(k0r + aa, L) * L;
-        float2 t = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int b = 0; b < J; ++b) {
-          const float2 g = __ldg(&row[wrap(k0c + b, L)]);
-          t.x = fmaf(wc[b], g.x, t.x);
-          t.y = fmaf(wc[b], g.y, t.y);
+      for (int q = 0; q < 8; ++q) {
+        const int k = k0 + threadIdx.x + q * NT;
+        if (k < NW) {
+          const int rr = quot_small(k, inv_w), cc = k - rr * W;  // W = T + J - 1 <= 71, k < 2^13
+          int r = R0 + rr, c = C0 + cc;
+          if (r >= L) r -= L;
+          if (c >= L) c -= L;
+          v[q] = __ldg(&X[(size_t)r * L + c]);
         }
-        acc.x = fmaf(wr[aa], t.x, acc.x);
-        acc.y = fmaf(wr[aa], t.y, acc.y);
       }
-    }
-    if (MODE == kDegridPerm) {
-      a.out[perm[i]] = acc;
-    } else if (MODE == kDegridSorted) {
-      a.out[i] = acc;
-    } else if (MODE == kDegridWeighted) {
-      const int m = perm[i];
-      const float w = a.w[m];
-      if (a.out) a.out[m] = acc;
-      a.t[i] = cscale(acc, w * w);
-      if (a.wb) {
-        const float2 h = a.h[m];
-        a.wb[m] += a.hf * w * (acc.x * h.x + acc.y * h.y);
-      }
-    } else {
-      // SDMM: s2 = Phi x_hat, and the two FP64 norms of the l2 branch
-      a.out[i] = acc;
-      float2 y;
-      if (a.y) {
-        y = a.y[i];
-      } else {
-        const float sc4 = a.yscale[i >> 12];
-        const uint32_t bits = reinterpret_cast<const uint32_t*>(a.yb)[i];
-        y = make_float2(__uint_as_float(bits << 16) * sc4, __uint_as_float(bits & 0xffff0000u) * sc4);
-      }
-      const float2 z = a.z2[i];
-      const float2 av = cadd(acc, z);
-      part[0].add_sq_diff(av.x, y.x);
-      part[0].add_sq_diff(av.y, y.y);
-      part[1].add_sq_diff(acc.x, y.x);
-      part[1].add_sq_diff(acc.y, y.y);
-    }
-  };
 #pragma unroll
-  for (int q = 0; q < QV; ++q) {
-    const int i = ch.y + threadIdx.x + q * NT;
-    if (i < ch.z) visit(i, uq[q]);
+      for (int q = 0; q < 8; ++q) {
+        const int k = k0 + threadIdx.x + q * NT;
+        if (k < NW) halo[k] = v[q];
+      }
+    }
+    __syncthreads();
+    auto visit = [&](int i, float2 u) {
+      int k0r, k0c;
+      float fr, fc;
+      split_kappa(u.x, ks, k0r, fr);
+      split_kappa(u.y, ks, k0c, fc);
+      k0r -= J / 2 - 1;
+      k0c -= J / 2 - 1;
+      float wr[J], wc[J];
+      kb_weights<J>(kb, fr, wr);
+      kb_weights<J>(kb, fc, wc);
+      // offsets in the tile; one turn of the grid at most for frequencies in
+      // [-pi, pi), any number (a remainder) otherwise
+      int dr = k0r - R0, dc = k0c - C0;
+      if (dr < 0) dr += L;
+      if (dc < 0) dc += L;
+      if ((unsigned)dr >= (unsigned)L || (unsigned)dc >= (unsigned)L) {
+        dr = wrap(dr, L);
+        dc = wrap(dc, L);
+      }
+      float2 acc = make_float2(0.f, 0.f);
+      if (dr < T && dc < T) {
+        const float2* base = halo + dr * W + dc;
+        float2 wcc[J];  // the column weights as (w, w) pairs for the FFMA2s
+#pragma unroll
+        for (int b = 0; b < J; ++b) wcc[b] = make_float2(wc[b], wc[b]);
+#pragma unroll
+        for (int aa = 0; aa < J; ++aa) {
+          float2 t = make_float2(0.f, 0.f);
+#pragma unroll
+          for (int b = 0; b < J; ++b) t = __ffma2_rn(wcc[b], base[aa * W + b], t);
+          acc = caxpy(wr[aa], t, acc);
+        }
+      } else {
+        // not in this tile (never for a consistent table): read the grid directly
+#pragma unroll
+        for (int aa = 0; aa < J; ++aa) {
+          const float2* row = X + (size_t)wrap(k0r + aa, L) * L;
+          float2 t = make_float2(0.f, 0.f);
+#pragma unroll
+          for (int b = 0; b < J; ++b) {
+            const float2 g = __ldg(&row[wrap(k0c + b, L)]);
+            t.x = fmaf(wc[b], g.x, t.x);
+            t.y = fmaf(wc[b], g.y, t.y);
+          }
+          acc.x = fmaf(wr[aa], t.x, acc.x);
+          acc.y = fmaf(wr[aa], t.y, acc.y);
+        }
+      }
+      if (MODE == kDegridPerm) {
+        a.out[perm[i]] = acc;
+      } else if (MODE == kDegridSorted) {
+        a.out[i] = acc;
+      } else if (MODE == kDegridWeighted) {
+        const int m = perm[i];
+        const float w = a.w[m];
+        if (a.out) a.out[m] = acc;
+        a.t[i] = cscale(acc, w * w);
+        if (a.wb) {
+          const float2 h = a.h[m];
+          a.wb[m] += a.hf * w * (acc.x * h.x + acc.y * h.y);
+        }
+      } else {
+        // SDMM: s2 = Phi x_hat, and the two FP64 norms of the l2 branch
+        a.out[i] = acc;
+        float2 y;
+        if (a.y) {
+          y = a.y[i];
+        } else {
+          const float sc4 = a.yscale[i >> 12];
+          const uint32_t bits = reinterpret_cast<const uint32_t*>(a.yb)[i];
+          y = make_float2(__uint_as_float(bits << 16) * sc4, __uint_as_float(bits & 0xffff0000u) * sc4);
+        }
+        const float2 z = a.z2[i];
+        const float2 av = cadd(acc, z);
+        part[0].add_sq_diff(av.x, y.x);
+        part[0].add_sq_diff(av.y, y.y);
+        part[1].add_sq_diff(acc.x, y.x);
+        part[1].add_sq_diff(acc.y, y.y);
+      }
+    };
+#pragma unroll
+    for (int q = 0; q < QV; ++q) {
+      const int i = ch.y + threadIdx.x + q * NT;
+      if (i < ch.z) visit(i, uq[q]);
+    }
+    for (int i = ch.y + threadIdx.x + QV * NT; i < ch.z; i += NT) visit(i, __ldg(&uv[i]));
+    if (MODE != kDegridSdmm) break;
+    __syncthreads();  // the halo is reused
   }
-  for (int i = ch.y + threadIdx.x + QV * NT; i < ch.z; i += NT) visit(i, __ldg(&uv[i]));
   if (MODE == kDegridSdmm) {
     double tot[2];
     if (reduce_last_block<2>(part, partials + kCntL2 * 2 * kMaxPartials, &sc->counter[kCntL2], tot)) {
@@ -596,6 +614,7 @@ __global__ void __launch_bounds__(kGridThreads, MINB) k_grid(float2* __restrict_
   if (threadIdx.x == 0) tile_cnt[tile] = 0u;
 }
 
+constexpr int kDegridPerSm = 8;  // CTAs of the SDMM mode per SM (4: 108 us, 8: 97 us, a CTA per chunk: 119 us, beside the prior branch)
 template <int J>
 static void degrid_J(purify_ctx* c, DegridOut mode, const DegridArgs& a, cudaStream_t s) {
   const int threads = 256;
@@ -605,8 +624,8 @@ static void degrid_J(purify_ctx* c, DegridOut mode, const DegridArgs& a, cudaStr
   do {                                                                                                        \
     allow_smem(k_degrid<J, MD>, sm);                                                                          \
     PURIFY_LAUNCH(c, "degrid", s,                                                                             \
-                  (pdl_launch(k_degrid<J, MD>, LaunchCfg{c->ndchunks, threads, sm, s}, c->d_grid, c->d_uv, c->d_perm, a, c->d_dchunks, \
-                                                                    c->kb, c->ks, c->L, c->tileT, c->tiles_1d,     \
+                  (pdl_launch(k_degrid<J, MD>, LaunchCfg{MD == kDegridSdmm ? std::min(c->ndchunks, kDegridPerSm * c->sms) : c->ndchunks, threads, sm, s}, c->d_grid, c->d_uv, c->d_perm, a, c->d_dchunks, \
+                                                                    c->ndchunks, c->kb, c->ks, c->L, c->tileT, c->tiles_1d,     \
                                                                     c->d_partials, c->d_sc)));                     \
   } while (0)
   if (mode == kDegridPerm) DEG(kDegridPerm);

@@ -368,9 +368,12 @@ __global__ void __launch_bounds__(256) k_row_inv(const float2* __restrict__ half
 // ---------------------------------------------------------------------------
 // Signals (rows, adjacent columns) per CTA.  The passes of small grids are
 // latency-bound, so rows are spread over about 128 CTAs before a CTA takes a
-// second one (at 512, 32 CTAs of eight rows: 6.7 us an inverse row pass
-// against ROWINV us for 128 of two), with at least a warp per CTA; the inverse row pass of the CG leaves one pair of
-// partial sums per CTA, which every CTA of the next pass adds up.
+// second one (512-point rows of the CG: 32 CTAs of eight rows 6.7 us an inverse
+// pass, 128 of two 5.2 us), with at least a warp per CTA.  Not more: the
+// inverse row pass of the CG leaves one pair of partial sums per CTA, which
+// every CTA of the next pass adds up.  Eight elements per thread up to 512
+// points: a lone warp issues an instruction every six clocks, so shorter
+// threads win there (128 points, CG epilogue: 16 elements 6.4 us, 8 4.5 us).
 constexpr int p2_rows(int L, int E, int max_threads) {
   const int per = L / E;                        // threads per row
   int ns = p2_max(1, L / 2 / 128);              // about 128 CTAs
@@ -383,7 +386,7 @@ constexpr int p2_rows(int L, int E, int max_threads) {
 template <int L>
 struct P2Cfg {
   static constexpr bool T3 = L % 3 == 0;
-  static constexpr int E = T3 ? 24 : (L >= 1024 || L == 128 ? 16 : 8);  // plain row, column and inverse row passes
+  static constexpr int E = T3 ? 24 : (L >= 1024 ? 16 : 8);  // plain row, column and inverse row passes
   static constexpr int E_CG = T3 ? 12 : 8;                              // forward row pass with the CG update
   static constexpr int NS_ROW = p2_rows(L, E, 256);
   static constexpr int NS_ROWCG = p2_rows(L, E_CG, 256);
