@@ -36,15 +36,24 @@ struct LevelGeom {
   int f1_off;   // analysis, prox mode: index of this launch's first f1 partial
 };
 
+// Daubechies orders of the wavelet planes, four bits each (an array indexed by
+// the plane would be copied to local memory by every thread).
 struct BasisList {
-  int p[8];     // Daubechies order of wavelet plane k
+  unsigned packed;  // at most eight planes
+  __host__ __device__ int p(int k) const { return (int)(packed >> (4 * k)) & 15; }
+};
+
+// The filters as kernel parameters: each tap as the (w, w) pair of a packed
+// FP32x2 multiply-add, db_p from p (p - 1).
+struct WaveletTaps {
+  float2 h[72], g[72];
 };
 
 // Soft threshold + dual update for one final coefficient alpha at index j;
 // returns w |alpha| (its term of f1), summed per thread in FP32 (a few terms)
 // and across threads in FP64.
 // The same with z1_j and w_j already loaded.
-__device__ __forceinline__ float sara_prox_v(float2 al, float2 z, float w, size_t j, const SaraProxArgs& pa,
+__device__ __forceinline__ float sara_prox_v(float2 al, float2 z, float w, int j, float2* z1, float2* u1,
                                              float gamma) {
   const float2 a = cadd(al, z);
   // shrink factor (|a| - lam)^+ / |a| = max(1 - lam / |a|, 0), with 1 / |a|
@@ -53,15 +62,15 @@ __device__ __forceinline__ float sara_prox_v(float2 al, float2 z, float w, size_
   const float s = m2 > 0.0f ? fmaxf(fmaf(-gamma * w, rsqrtf(m2), 1.0f), 0.0f) : 0.0f;
   const float2 r1 = cscale(a, s);
   const float2 z1n = csub(a, r1);
-  pa.z1[j] = z1n;
-  pa.u1[j] = csub(r1, z1n);
+  z1[j] = z1n;
+  u1[j] = csub(r1, z1n);
   const float al2 = fmaf(al.x, al.x, al.y * al.y);
   return w * (al2 > 0.0f ? al2 * rsqrtf(al2) : 0.0f);
 }
 
 __device__ __forceinline__ float sara_prox(float2 al, size_t j, const SaraProxArgs& pa, float gamma) {
   const float w = pa.w ? pa.w[j] : 1.0f;
-  return sara_prox_v(al, pa.z1[j], w, j, pa, gamma);
+  return sara_prox_v(al, pa.z1[j], w, 0, pa.z1 + j, pa.u1 + j, gamma);
 }
 
 // ---------------------------------------------------------------------------
@@ -89,28 +98,28 @@ __global__ void k_dirac(const float2* __restrict__ x, float2* __restrict__ alpha
 // One wavelet plane of one analysis level, for the Daubechies order P fixed at
 // compile time (filters in registers, tap loops unrolled).  Returns this
 // thread's terms of f1 (prox mode).
-template <int P, int MODE>
+//
+// FAST (tiles of a multiple of four): a thread filters four adjacent outputs
+// of a row, then two of a column, from one window of inputs, (2P + 6) / 8 and
+// (2P + 2) / 4 shared-memory loads per output instead of P (one output pair
+// per thread: all four levels at 1024^2 83 us; 74 us so, issue-bound), and lanes take consecutive rows of an odd stride, so neither pass has
+// bank conflicts.
+template <int P, int MODE, bool FAST>
 __device__ __forceinline__ float dwt_plane(const float2* __restrict__ in, int in_shared, float2* __restrict__ ll_out,
-                                           float2* __restrict__ coef, const LevelGeom& G, const WaveletFilters& wf,
+                                           float2* __restrict__ coef, const LevelGeom& G, const WaveletTaps& wf,
                                            const SaraProxArgs& pa, int k, float gamma) {
   extern __shared__ float2 sm[];
   constexpr int taps = 2 * P;
   constexpr int hoff = P * (P - 1);  // db_p starts after db_1 .. db_(p-1): sum of 2q, q < p
-  float2 h[taps], g[taps];  // each tap as a (w, w) pair for the FFMA2s
-#pragma unroll
-  for (int m = 0; m < taps; ++m) {
-    const float hm = wf.h[hoff + m];
-    const float hr = wf.h[hoff + taps - 1 - m];
-    h[m] = make_float2(hm, hm);
-    g[m] = (m & 1) ? make_float2(-hr, -hr) : make_float2(hr, hr);
-  }
+  const float2 *h = wf.h + hoff, *g = wf.g + hoff;
   float f1 = 0.f;
   const int L = G.L, H = L / 2;
   const int TI = G.tile;
   const int I1 = blockIdx.y * TI, I2 = blockIdx.x * TI;
   const int RH = 2 * TI + taps - 2;  // input rows/cols the tile needs
+  const int RHS = RH | 1, RS = 2 * TI + 1;  // row strides (odd)
   float2* inb = sm;                  // RH x RH
-  float2* rowp = sm + RH * RH;       // RH x 2TI  ([a | d] per input row)
+  float2* rowp = sm + RH * RHS;      // RH x 2TI  ([a | d] per input row)
   const float2* src = in_shared ? in : in + (size_t)k * (G.n / 2) * (G.n / 2);
   const Div dTI = make_div(TI), d2TI = make_div(2 * TI);
   // input tile with its halo (periodic): warps take rows, lanes columns (RH <=
@@ -118,52 +127,71 @@ __device__ __forceinline__ float dwt_plane(const float2* __restrict__ in, int in
   // when L >= RH, and index by index (a remainder) otherwise
   {
     const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    auto wrapped = [&](int i) { return L >= RH ? (i >= L ? i - L : i) : i % L; };
+    const int cA = wrapped(2 * I2 + lane), cB = wrapped(2 * I2 + lane + 32);
+    const bool hasB = lane + 32 < RH, hasA = lane < RH;
     for (int rr0 = (threadIdx.x >> 5); rr0 < RH; rr0 += 4 * nw) {
       float2 v[4][2];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int rr = rr0 + q * nw;
         if (rr < RH) {
-          int r = 2 * I1 + rr;
-          r = (L >= RH) ? (r >= L ? r - L : r) : r % L;
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int cc = lane + 32 * h;
-            if (cc < RH) {
-              int c = 2 * I2 + cc;
-              c = (L >= RH) ? (c >= L ? c - L : c) : c % L;
-              v[q][h] = src[(size_t)r * L + c];
-            }
-          }
+          const float2* row = src + wrapped(2 * I1 + rr) * L;
+          if (hasA) v[q][0] = row[cA];
+          if (hasB) v[q][1] = row[cB];
         }
       }
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int rr = rr0 + q * nw;
         if (rr < RH) {
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int cc = lane + 32 * h;
-            if (cc < RH) inb[rr * RH + cc] = v[q][h];
-          }
+          if (hasA) inb[rr * RHS + lane] = v[q][0];
+          if (hasB) inb[rr * RHS + lane + 32] = v[q][1];
         }
       }
     }
   }
   __syncthreads();
   // rows: a[i2] = sum_m h[m] s[2 i2 + m], d[i2] = sum_m g[m] s[2 i2 + m]
-  for (int idx = threadIdx.x; idx < RH * TI; idx += blockDim.x) {
-    const int rr = udiv(idx, dTI), i2 = idx - rr * TI;
-    const float2* sp = inb + rr * RH + 2 * i2;
-    float2 a = make_float2(0.f, 0.f), d = make_float2(0.f, 0.f);
+  if constexpr (FAST) {
+    const float inv_rh = 1.0f / (float)RH;
+    for (int idx = threadIdx.x; idx < RH * (TI / 4); idx += blockDim.x) {
+      const int qq = quot_small(idx, inv_rh), rr = idx - qq * RH;
+      const float2* sp = inb + rr * RHS + 8 * qq;
+      float2 a[4], d[4];
 #pragma unroll
-    for (int m = 0; m < taps; ++m) {
-      const float2 v = sp[m];
-      a = __ffma2_rn(h[m], v, a);
-      d = __ffma2_rn(g[m], v, d);
+      for (int j = 0; j < 4; ++j) a[j] = d[j] = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int m = 0; m < taps + 6; ++m) {
+        const float2 v = sp[m];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (m - 2 * j >= 0 && m - 2 * j < taps) {
+            a[j] = __ffma2_rn(h[m - 2 * j], v, a[j]);
+            d[j] = __ffma2_rn(g[m - 2 * j], v, d[j]);
+          }
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        rowp[rr * RS + 4 * qq + j] = a[j];
+        rowp[rr * RS + TI + 4 * qq + j] = d[j];
+      }
     }
-    rowp[rr * (2 * TI) + i2] = a;
-    rowp[rr * (2 * TI) + TI + i2] = d;
+  } else {
+    for (int idx = threadIdx.x; idx < RH * TI; idx += blockDim.x) {
+      const int rr = udiv(idx, dTI), i2 = idx - rr * TI;
+      const float2* sp = inb + rr * RHS + 2 * i2;
+      float2 a = make_float2(0.f, 0.f), d = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int m = 0; m < taps; ++m) {
+        const float2 v = sp[m];
+        a = __ffma2_rn(h[m], v, a);
+        d = __ffma2_rn(g[m], v, d);
+      }
+      rowp[rr * RS + i2] = a;
+      rowp[rr * RS + TI + i2] = d;
+    }
   }
   __syncthreads();
   // columns, and the write-out of the four sub-bands
@@ -173,79 +201,93 @@ __device__ __forceinline__ float dwt_plane(const float2* __restrict__ in, int in
   // output with its prox operands loaded together
   constexpr int kMaxIdx = 2;  // TI * 2TI / 256
   float2 lov[kMaxIdx], hiv[kMaxIdx];
-  int idxv[kMaxIdx];
+  int i1v[kMaxIdx], kcv[kMaxIdx];  // coefficient row and column of [a | d], i1 = -1: none
 #pragma unroll
   for (int t = 0; t < kMaxIdx; ++t) {
     const int idx = threadIdx.x + t * blockDim.x;
-    idxv[t] = idx < TI * 2 * TI ? idx : -1;
-    float2 lo = make_float2(0.f, 0.f), hi = make_float2(0.f, 0.f);
-    if (idxv[t] >= 0) {
-      const int i1 = udiv(idx, d2TI), kc = idx - i1 * (2 * TI);
-      const float2* cp = rowp + (2 * i1) * (2 * TI) + kc;
+    if (FAST) {  // rows 2 j and 2 j + 1
+      const int j = udiv(threadIdx.x, d2TI);
+      i1v[t] = 2 * j < TI ? 2 * j + t : -1;
+      kcv[t] = threadIdx.x - j * (2 * TI);
+    } else {
+      const int i1 = udiv(idx, d2TI);
+      i1v[t] = idx < TI * 2 * TI ? i1 : -1;
+      kcv[t] = idx - i1 * (2 * TI);
+    }
+    lov[t] = hiv[t] = make_float2(0.f, 0.f);
+  }
+  if constexpr (FAST) {
+    if (i1v[0] >= 0) {
+      const float2* cp = rowp + (2 * i1v[0]) * RS + kcv[0];
+#pragma unroll
+      for (int m = 0; m < taps + 2; ++m) {
+        const float2 v = cp[m * RS];
+        if (m < taps) {
+          lov[0] = __ffma2_rn(h[m], v, lov[0]);
+          hiv[0] = __ffma2_rn(g[m], v, hiv[0]);
+        }
+        if (m >= 2) {
+          lov[1] = __ffma2_rn(h[m - 2], v, lov[1]);
+          hiv[1] = __ffma2_rn(g[m - 2], v, hiv[1]);
+        }
+      }
+    }
+  } else {
+#pragma unroll
+    for (int t = 0; t < kMaxIdx; ++t) {
+      if (i1v[t] < 0) continue;
+      const float2* cp = rowp + (2 * i1v[t]) * RS + kcv[t];
 #pragma unroll
       for (int m = 0; m < taps; ++m) {
-        const float2 v = cp[m * (2 * TI)];
-        lo = __ffma2_rn(h[m], v, lo);
-        hi = __ffma2_rn(g[m], v, hi);
+        const float2 v = cp[m * RS];
+        lov[t] = __ffma2_rn(h[m], v, lov[t]);
+        hiv[t] = __ffma2_rn(g[m], v, hiv[t]);
       }
     }
-    lov[t] = lo;
-    hiv[t] = hi;
   }
-  // destinations: LL = lo of a (top-left), LH = lo of d (top-right),
-  // HL = hi of a (bottom-left), HH = hi of d; on coarser levels LL goes to llk
-  size_t jo[2 * kMaxIdx];
-  float2 ao[2 * kMaxIdx];
-  bool to_plane[2 * kMaxIdx];
+  // destinations (offsets in the plane, at most 2048^2): LL = lo of a
+  // (top-left), LH = lo of d (top-right), HL = hi of a (H rows below), HH = hi
+  // of d; on levels before the last LL goes to llk
+  const int Hn = H * G.n;
+  float2* z1 = MODE == kSaraProx ? pa.z1 + (size_t)(G.plane0 + k) * G.n * G.n : nullptr;
+  const float* w = MODE == kSaraProx && pa.w ? pa.w + (size_t)(G.plane0 + k) * G.n * G.n : nullptr;
+  float2* u1 = MODE == kSaraProx ? pa.u1 + (size_t)(G.plane0 + k) * G.n * G.n : nullptr;
+  float2 zv[2 * kMaxIdx];
+  float wv[2 * kMaxIdx];
+  int off[kMaxIdx];
+  bool lo_out[kMaxIdx];
 #pragma unroll
   for (int t = 0; t < kMaxIdx; ++t) {
-    jo[2 * t] = jo[2 * t + 1] = 0;
-    to_plane[2 * t] = to_plane[2 * t + 1] = false;
-    ao[2 * t] = ao[2 * t + 1] = make_float2(0.f, 0.f);
-    if (idxv[t] < 0) continue;
-    const int i1 = udiv(idxv[t], d2TI), kc = idxv[t] - i1 * (2 * TI);
-    const int gi1 = I1 + i1;
-    const bool rowlow = kc < TI;
-    const int gi2 = I2 + (rowlow ? kc : kc - TI);
-    if (rowlow) {
-      if (G.last) {
-        jo[2 * t] = (size_t)gi1 * G.n + gi2;
-        ao[2 * t] = cscale(lov[t], G.scale);
-        to_plane[2 * t] = true;
-      } else {
-        llk[(size_t)gi1 * H + gi2] = lov[t];
+    off[t] = 0;
+    lo_out[t] = false;
+    if (i1v[t] < 0) continue;
+    const bool rowlow = kcv[t] < TI;
+    const int gi1 = I1 + i1v[t], gi2 = I2 + (rowlow ? kcv[t] : kcv[t] - TI);
+    off[t] = gi1 * G.n + (rowlow ? gi2 : H + gi2);
+    lo_out[t] = !rowlow || G.last;
+    if (!lo_out[t]) llk[gi1 * H + gi2] = lov[t];
+    if (MODE == kSaraProx) {  // the prox operands of every output, loaded together
+      if (lo_out[t]) {
+        zv[2 * t] = z1[off[t]];
+        wv[2 * t] = w ? w[off[t]] : 1.0f;
       }
-      jo[2 * t + 1] = (size_t)(H + gi1) * G.n + gi2;  // HL
-      ao[2 * t + 1] = cscale(hiv[t], G.scale);
+      zv[2 * t + 1] = z1[off[t] + Hn];
+      wv[2 * t + 1] = w ? w[off[t] + Hn] : 1.0f;
+    }
+  }
+#pragma unroll
+  for (int t = 0; t < kMaxIdx; ++t) {
+    if (i1v[t] < 0) continue;
+    const float2 lo = cscale(lov[t], G.scale), hi = cscale(hiv[t], G.scale);
+    if (MODE == kSaraPlain) {
+      if (lo_out[t]) plane[off[t]] = lo;
+      plane[off[t] + Hn] = hi;
     } else {
-      jo[2 * t] = (size_t)gi1 * G.n + H + gi2;                // LH
-      jo[2 * t + 1] = (size_t)(H + gi1) * G.n + H + gi2;      // HH
-      ao[2 * t] = cscale(lov[t], G.scale);
-      ao[2 * t + 1] = cscale(hiv[t], G.scale);
-      to_plane[2 * t] = true;
+      if (lo_out[t]) f1 += sara_prox_v(lo, zv[2 * t], wv[2 * t], off[t], z1, u1, gamma);
+      f1 += sara_prox_v(hi, zv[2 * t + 1], wv[2 * t + 1], off[t] + Hn, z1, u1, gamma);
     }
-    to_plane[2 * t + 1] = true;
   }
-  const size_t pbase = (size_t)(G.plane0 + k) * G.n * G.n;
-  if (MODE == kSaraPlain) {
-#pragma unroll
-    for (int o = 0; o < 2 * kMaxIdx; ++o)
-      if (to_plane[o]) plane[jo[o]] = ao[o];
-  } else {
-    float2 zv[2 * kMaxIdx];
-    float wv[2 * kMaxIdx];
-#pragma unroll
-    for (int o = 0; o < 2 * kMaxIdx; ++o) {
-      if (to_plane[o]) {
-        zv[o] = pa.z1[pbase + jo[o]];
-        wv[o] = pa.w ? pa.w[pbase + jo[o]] : 1.0f;
-      }
-    }
-#pragma unroll
-    for (int o = 0; o < 2 * kMaxIdx; ++o)
-      if (to_plane[o]) f1 += sara_prox_v(ao[o], zv[o], wv[o], pbase + jo[o], pa, gamma);
-  }
-    return f1;
+  return f1;
 }
 
 // ---------------------------------------------------------------------------
@@ -255,10 +297,10 @@ __device__ __forceinline__ float dwt_plane(const float2* __restrict__ in, int in
 //            ll_out + k * (n/2)^2, or to the plane on the last level.
 // CTA: coefficient tile [I1, I1 + TI) x [I2, I2 + TI) of the L/2 x L/2 sub-bands.
 // ---------------------------------------------------------------------------
-template <int MODE>
+template <int MODE, bool FAST>
 __global__ void __launch_bounds__(256) k_dwt_level(const float2* __restrict__ in, int in_shared,
                                                    float2* __restrict__ ll_out, float2* __restrict__ coef,
-                                                   LevelGeom G, BasisList bl, WaveletFilters wf,
+                                                   LevelGeom G, BasisList bl, const __grid_constant__ WaveletTaps wf,
                                                    SaraProxArgs pa, double* partials, DevScalars* sc) {
   pdl_sync(in, ll_out, coef, partials, sc);
   extern __shared__ float2 sm[];
@@ -269,24 +311,25 @@ __global__ void __launch_bounds__(256) k_dwt_level(const float2* __restrict__ in
     // the Dirac plane (first level only): alpha_0 = x / sqrt(q) on this CTA's
     // 2TI x 2TI block of pixels, with its prox update
     const int TI = G.tile, r0 = 2 * blockIdx.y * TI, c0 = 2 * blockIdx.x * TI;
+    const Div d2TI = make_div(2 * TI);
     const size_t base = (size_t)G.dirac * G.n * G.n;
     for (int e = threadIdx.x; e < 4 * TI * TI; e += blockDim.x) {
-      const int rr = e / (2 * TI), cc = e - rr * (2 * TI);
+      const int rr = udiv(e, d2TI), cc = e - rr * (2 * TI);
       const size_t j = (size_t)(r0 + rr) * G.n + c0 + cc;
       const float2 al = cscale(in[j], G.scale);
       if (MODE == kSaraPlain) coef[base + j] = al;
       else f1 += sara_prox(al, base + j, pa, gamma);
     }
   } else {
-    switch (bl.p[k]) {
-      case 1: f1 += dwt_plane<1, MODE>(in, in_shared, ll_out, coef, G, wf, pa, k, gamma); break;
-      case 2: f1 += dwt_plane<2, MODE>(in, in_shared, ll_out, coef, G, wf, pa, k, gamma); break;
-      case 3: f1 += dwt_plane<3, MODE>(in, in_shared, ll_out, coef, G, wf, pa, k, gamma); break;
-      case 4: f1 += dwt_plane<4, MODE>(in, in_shared, ll_out, coef, G, wf, pa, k, gamma); break;
-      case 5: f1 += dwt_plane<5, MODE>(in, in_shared, ll_out, coef, G, wf, pa, k, gamma); break;
-      case 6: f1 += dwt_plane<6, MODE>(in, in_shared, ll_out, coef, G, wf, pa, k, gamma); break;
-      case 7: f1 += dwt_plane<7, MODE>(in, in_shared, ll_out, coef, G, wf, pa, k, gamma); break;
-      default: f1 += dwt_plane<8, MODE>(in, in_shared, ll_out, coef, G, wf, pa, k, gamma); break;
+    switch (bl.p(k)) {
+      case 1: f1 += dwt_plane<1, MODE, FAST>(in, in_shared, ll_out, coef, G, wf, pa, k, gamma); break;
+      case 2: f1 += dwt_plane<2, MODE, FAST>(in, in_shared, ll_out, coef, G, wf, pa, k, gamma); break;
+      case 3: f1 += dwt_plane<3, MODE, FAST>(in, in_shared, ll_out, coef, G, wf, pa, k, gamma); break;
+      case 4: f1 += dwt_plane<4, MODE, FAST>(in, in_shared, ll_out, coef, G, wf, pa, k, gamma); break;
+      case 5: f1 += dwt_plane<5, MODE, FAST>(in, in_shared, ll_out, coef, G, wf, pa, k, gamma); break;
+      case 6: f1 += dwt_plane<6, MODE, FAST>(in, in_shared, ll_out, coef, G, wf, pa, k, gamma); break;
+      case 7: f1 += dwt_plane<7, MODE, FAST>(in, in_shared, ll_out, coef, G, wf, pa, k, gamma); break;
+      default: f1 += dwt_plane<8, MODE, FAST>(in, in_shared, ll_out, coef, G, wf, pa, k, gamma); break;
     }
   }
   if (MODE == kSaraProx) {
@@ -332,70 +375,128 @@ __device__ __forceinline__ void sara_f1_finish(const double* __restrict__ part, 
 // Column then row synthesis of one plane's coefficient windows (in shared
 // memory) for the Daubechies order P fixed at compile time; the finest level
 // accumulates into accum, coarser levels write their low-low output.
+//
+// FAST (even tiles): a thread forms four adjacent outputs (two of each parity)
+// of a column, then of a row, from one window of P + 1 coefficients, a quarter
+// of the shared-memory loads of one output per thread, which bound this kernel
+// (the four levels at 1024^2: 134 us with one output per
+// thread, 95 us so).
 constexpr int kIdwtMaxOut = 4;  // (2TO)^2 / blockDim outputs per thread: 1024 / 256
-template <int P>
+template <int P, bool FAST>
 __device__ __forceinline__ void idwt_filter(const float2* LLs, const float2* HLs, const float2* LHs,
                                             const float2* HHs, float2* As, float2* Ds, const LevelGeom& G,
-                                            const WaveletFilters& wf, int k, int K1, int K2,
+                                            const WaveletTaps& wf, int k, int K1, int K2,
                                             float2* __restrict__ ll_out, float2 (&accum)[kIdwtMaxOut]) {
-  constexpr int taps = 2 * P;
   constexpr int hoff = P * (P - 1);
-  float2 h[taps], g[taps];  // (w, w) pairs
-#pragma unroll
-  for (int m = 0; m < taps; ++m) {
-    const float hm = wf.h[hoff + m];
-    const float hr = wf.h[hoff + taps - 1 - m];
-    h[m] = make_float2(hm, hm);
-    g[m] = (m & 1) ? make_float2(-hr, -hr) : make_float2(hr, hr);
-  }
+  const float2 *h = wf.h + hoff, *g = wf.g + hoff;
   const int L = G.L;
   const int TO = G.tile;
-  const int CW = TO + P - 1;
-  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  const int nout = (2 * TO) * (2 * TO);
+  const int CW = TO + P - 1, CWS = CW | 1;  // As, Ds: odd row stride
   const Div d2TO = make_div(2 * TO);
-  // column synthesis: output row kappa1 in [0, 2TO), window column t2;
-  // taps of one parity: m = par + 2u, t1 = (k1 - par) / 2 - u + P - 1
-  for (int t2 = threadIdx.x >> 5; t2 < CW; t2 += nw)
-    for (int k1 = lane; k1 < 2 * TO; k1 += 32) {
-      const int idx = k1 * CW + t2;
-      const int par = k1 & 1;
-      const int tb = (k1 - par) / 2 + P - 1;
-      float2 av = make_float2(0.f, 0.f), dv = make_float2(0.f, 0.f);
+  // column synthesis: output row k1 in [0, 2TO), window column t2; taps of one
+  // parity: m = par + 2u, t1 = (k1 - par) / 2 - u + P - 1
+  if constexpr (FAST) {
+    const float inv_cw = 1.0f / (float)CW;
+    for (int idx = threadIdx.x; idx < (TO / 2) * CW; idx += blockDim.x) {
+      const int qq = quot_small(idx, inv_cw), t2 = idx - qq * CW;
+      float2 av[2][2], dv[2][2];  // [pair][parity]: output row 4 qq + 2 pair + parity
 #pragma unroll
-      for (int u = 0; u < P; ++u) {
-        const int t1 = tb - u;
-        const float2 hm = par ? h[2 * u + 1] : h[2 * u], gm = par ? g[2 * u + 1] : g[2 * u];
-        const float2 ll = LLs[t1 * CW + t2], hl = HLs[t1 * CW + t2];
-        const float2 lh = LHs[t1 * CW + t2], hh = HHs[t1 * CW + t2];
-        av = __ffma2_rn(hm, ll, __ffma2_rn(gm, hl, av));
-        dv = __ffma2_rn(hm, lh, __ffma2_rn(gm, hh, dv));
+      for (int e = 0; e < 2; ++e)
+#pragma unroll
+        for (int par = 0; par < 2; ++par) av[e][par] = dv[e][par] = make_float2(0.f, 0.f);
+      const int w0 = 2 * qq * CW + t2;
+#pragma unroll
+      for (int w = P; w >= 0; --w) {  // window row 2 qq + w
+        const float2 ll = LLs[w0 + w * CW], hl = HLs[w0 + w * CW], lh = LHs[w0 + w * CW], hh = HHs[w0 + w * CW];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int u = e + P - 1 - w;
+          if (u < 0 || u >= P) continue;
+#pragma unroll
+          for (int par = 0; par < 2; ++par) {
+            av[e][par] = __ffma2_rn(h[2 * u + par], ll, __ffma2_rn(g[2 * u + par], hl, av[e][par]));
+            dv[e][par] = __ffma2_rn(h[2 * u + par], lh, __ffma2_rn(g[2 * u + par], hh, dv[e][par]));
+          }
+        }
       }
-      As[idx] = av;
-      Ds[idx] = dv;
+#pragma unroll
+      for (int e = 0; e < 2; ++e)
+#pragma unroll
+        for (int par = 0; par < 2; ++par) {
+          As[(4 * qq + 2 * e + par) * CWS + t2] = av[e][par];
+          Ds[(4 * qq + 2 * e + par) * CWS + t2] = dv[e][par];
+        }
     }
+  } else {
+    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    for (int t2 = threadIdx.x >> 5; t2 < CW; t2 += nw)
+      for (int k1 = lane; k1 < 2 * TO; k1 += 32) {
+        const int par = k1 & 1;
+        const int tb = (k1 - par) / 2 + P - 1;
+        float2 av = make_float2(0.f, 0.f), dv = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < P; ++u) {
+          const int t1 = tb - u;
+          const float2 hm = par ? h[2 * u + 1] : h[2 * u], gm = par ? g[2 * u + 1] : g[2 * u];
+          const float2 ll = LLs[t1 * CW + t2], hl = HLs[t1 * CW + t2];
+          const float2 lh = LHs[t1 * CW + t2], hh = HHs[t1 * CW + t2];
+          av = __ffma2_rn(hm, ll, __ffma2_rn(gm, hl, av));
+          dv = __ffma2_rn(hm, lh, __ffma2_rn(gm, hh, dv));
+        }
+        As[k1 * CWS + t2] = av;
+        Ds[k1 * CWS + t2] = dv;
+      }
+  }
   __syncthreads();
   // row synthesis
+  float2* llk = ll_out + (size_t)k * (G.n / 2) * (G.n / 2);
+  if constexpr (FAST) {
+    const int qq = udiv(threadIdx.x, d2TO), k1 = threadIdx.x - qq * (2 * TO);
+    if (2 * qq < TO) {  // at most one group of four outputs per thread
+      float2 sv[2][2];
 #pragma unroll
-  for (int t = 0; t < kIdwtMaxOut; ++t) {
-    const int idx = threadIdx.x + t * blockDim.x;
-    if (idx >= nout) continue;
-    const int k1 = udiv(idx, d2TO), k2 = idx - k1 * (2 * TO);
-    const int par = k2 & 1;
-    const int tb = (k2 - par) / 2 + P - 1;
-    float2 sacc = make_float2(0.f, 0.f);
+      for (int e = 0; e < 2; ++e)
 #pragma unroll
-    for (int u = 0; u < P; ++u) {
-      const int t2 = tb - u;
-      const float2 hm = par ? h[2 * u + 1] : h[2 * u], gm = par ? g[2 * u + 1] : g[2 * u];
-      const float2 av = As[k1 * CW + t2], dv = Ds[k1 * CW + t2];
-      sacc = __ffma2_rn(hm, av, __ffma2_rn(gm, dv, sacc));
+        for (int par = 0; par < 2; ++par) sv[e][par] = make_float2(0.f, 0.f);
+      const int w0 = k1 * CWS + 2 * qq;
+#pragma unroll
+      for (int w = P; w >= 0; --w) {
+        const float2 av = As[w0 + w], dv = Ds[w0 + w];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int u = e + P - 1 - w;
+          if (u < 0 || u >= P) continue;
+#pragma unroll
+          for (int par = 0; par < 2; ++par)
+            sv[e][par] = __ffma2_rn(h[2 * u + par], av, __ffma2_rn(g[2 * u + par], dv, sv[e][par]));
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < 2; ++e)
+#pragma unroll
+        for (int par = 0; par < 2; ++par) {
+          if (G.last) accum[2 * e + par] = cadd(accum[2 * e + par], sv[e][par]);
+          else llk[(size_t)(K1 + k1) * L + K2 + 4 * qq + 2 * e + par] = sv[e][par];
+        }
     }
-    if (G.last) {
-      accum[t] = cadd(accum[t], sacc);
-    } else {
-      const int gk1 = K1 + k1, gk2 = K2 + k2;
-      if (gk1 < L && gk2 < L) ll_out[(size_t)k * (G.n / 2) * (G.n / 2) + (size_t)gk1 * L + gk2] = sacc;
+  } else {
+#pragma unroll
+    for (int t = 0; t < kIdwtMaxOut; ++t) {
+      const int idx = threadIdx.x + t * blockDim.x;
+      if (idx >= 4 * TO * TO) continue;
+      const int k1 = udiv(idx, d2TO), k2 = idx - k1 * (2 * TO);
+      const int par = k2 & 1;
+      const int tb = (k2 - par) / 2 + P - 1;
+      float2 sacc = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int u = 0; u < P; ++u) {
+        const int t2 = tb - u;
+        const float2 hm = par ? h[2 * u + 1] : h[2 * u], gm = par ? g[2 * u + 1] : g[2 * u];
+        const float2 av = As[k1 * CWS + t2], dv = Ds[k1 * CWS + t2];
+        sacc = __ffma2_rn(hm, av, __ffma2_rn(gm, dv, sacc));
+      }
+      if (G.last) accum[t] = cadd(accum[t], sacc);
+      else llk[(size_t)(K1 + k1) * L + K2 + k2] = sacc;
     }
   }
 }
@@ -408,10 +509,12 @@ __device__ __forceinline__ void idwt_filter(const float2* LLs, const float2* HLs
 // planes (plus the Dirac plane) into x, scaled by 1/sqrt(q).
 // CTA: output tile [K1, K1 + 2TO) x [K2, K2 + 2TO).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_idwt_level(const float2* __restrict__ ll_in, int ll_from_plane,
+template <bool FAST>
+__global__ void __launch_bounds__(256, 3) k_idwt_level(const float2* __restrict__ ll_in, int ll_from_plane,
                                                     float2* __restrict__ ll_out, const float2* __restrict__ coef,
                                                     float2* __restrict__ x, int dirac_plane, LevelGeom G,
-                                                    BasisList bl, WaveletFilters wf, const double* f1_part, int f1_n,
+                                                    BasisList bl, const __grid_constant__ WaveletTaps wf,
+                                                    const double* f1_part, int f1_n,
                                                     DevScalars* sc) {
   pdl_sync(ll_in, ll_out, coef, x, f1_part, sc);
   extern __shared__ float2 sm[];
@@ -435,46 +538,53 @@ __global__ void __launch_bounds__(256) k_idwt_level(const float2* __restrict__ l
 #pragma unroll
   for (int t = 0; t < kMaxOut; ++t) accum[t] = make_float2(0.f, 0.f);
   // the four coefficient windows of plane kk, loaded into registers (CW^2 <=
-  // 4 blockDim for TO <= 16, p <= 8): plane k + 1's loads are in flight while
+  // 23^2 <= 3 blockDim for TO <= 16, p <= 8): plane k + 1's loads are in flight while
   // plane k is synthesised
-  float2 v[4][4];
+  float2 v[3][4];
   auto issue = [&](int kk) {
-    const int pk = bl.p[kk];
+    const int pk = bl.p(kk);
     const int CWk = TO + pk - 1;
     const float2* plk = coef + (size_t)(G.plane0 + kk) * G.n * G.n;
     const float2* llk = ll_from_plane ? plk : ll_in + (size_t)kk * (G.n / 2) * (G.n / 2);
     const int lls = ll_from_plane ? G.n : H;
-    // window origin: coefficient K/2 - p + 1 (mod H), shifted to stay >= 0
-    const int o1 = K1 / 2 - pk + 1 + 8 * H, o2 = K2 / 2 - pk + 1 + 8 * H;
+    // window origin: coefficient K/2 - p + 1 (mod H); the window wraps at most
+    // once when H >= CW, and index by index (shifted to stay >= 0) otherwise
+    const int o1 = K1 / 2 - pk + 1, o2 = K2 / 2 - pk + 1;
+    const bool once = H >= CWk;
     const float rcw = 1.0f / (float)CWk;
+    auto wrapped = [&](int i) {
+      if (once) return i < 0 ? i + H : (i >= H ? i - H : i);
+      i += 8 * H;
+      return i - udiv(i, dH) * H;
+    };
+    const int Hn = H * G.n;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < 3; ++q) {
       const int e = threadIdx.x + q * blockDim.x;
       if (e < CWk * CWk) {
         const int t1 = quot_small(e, rcw), t2 = e - t1 * CWk;
-        int c1 = o1 + t1, c2 = o2 + t2;
-        c1 -= udiv(c1, dH) * H;
-        c2 -= udiv(c2, dH) * H;
-        v[q][0] = llk[(size_t)c1 * lls + c2];
-        v[q][1] = plk[(size_t)(H + c1) * G.n + c2];
-        v[q][2] = plk[(size_t)c1 * G.n + H + c2];
-        v[q][3] = plk[(size_t)(H + c1) * G.n + H + c2];
+        const int c1 = wrapped(o1 + t1), c2 = wrapped(o2 + t2);
+        const float2* pl = plk + c1 * G.n + c2;
+        v[q][0] = llk[c1 * lls + c2];
+        v[q][1] = pl[Hn];
+        v[q][2] = pl[H];
+        v[q][3] = pl[Hn + H];
       }
     }
   };
   issue(kbeg);
   for (int k = kbeg; k < kend; ++k) {
-    const int p = bl.p[k];
+    const int p = bl.p(k);
     const int CW = TO + p - 1;                 // coefficient window per axis
     float2* LLs = sm;                          // CW x CW each
     float2* HLs = LLs + CW * CW;
     float2* LHs = HLs + CW * CW;
     float2* HHs = LHs + CW * CW;
-    float2* As = HHs + CW * CW;                // 2TO x CW
-    float2* Ds = As + 2 * TO * CW;             // 2TO x CW
+    float2* As = HHs + CW * CW;
+    float2* Ds = As + 2 * TO * (CW | 1);       // 2TO x CW each, rows CW | 1 apart
     __syncthreads();
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < 3; ++q) {
       const int e = threadIdx.x + q * blockDim.x;
       if (e < CW * CW) {
         LLs[e] = v[q][0];
@@ -486,29 +596,35 @@ __global__ void __launch_bounds__(256) k_idwt_level(const float2* __restrict__ l
     __syncthreads();
     if (k + 1 < kend) issue(k + 1);
     switch (p) {
-      case 1: idwt_filter<1>(LLs, HLs, LHs, HHs, As, Ds, G, wf, k, K1, K2, ll_out, accum); break;
-      case 2: idwt_filter<2>(LLs, HLs, LHs, HHs, As, Ds, G, wf, k, K1, K2, ll_out, accum); break;
-      case 3: idwt_filter<3>(LLs, HLs, LHs, HHs, As, Ds, G, wf, k, K1, K2, ll_out, accum); break;
-      case 4: idwt_filter<4>(LLs, HLs, LHs, HHs, As, Ds, G, wf, k, K1, K2, ll_out, accum); break;
-      case 5: idwt_filter<5>(LLs, HLs, LHs, HHs, As, Ds, G, wf, k, K1, K2, ll_out, accum); break;
-      case 6: idwt_filter<6>(LLs, HLs, LHs, HHs, As, Ds, G, wf, k, K1, K2, ll_out, accum); break;
-      case 7: idwt_filter<7>(LLs, HLs, LHs, HHs, As, Ds, G, wf, k, K1, K2, ll_out, accum); break;
-      default: idwt_filter<8>(LLs, HLs, LHs, HHs, As, Ds, G, wf, k, K1, K2, ll_out, accum); break;
+      case 1: idwt_filter<1, FAST>(LLs, HLs, LHs, HHs, As, Ds, G, wf, k, K1, K2, ll_out, accum); break;
+      case 2: idwt_filter<2, FAST>(LLs, HLs, LHs, HHs, As, Ds, G, wf, k, K1, K2, ll_out, accum); break;
+      case 3: idwt_filter<3, FAST>(LLs, HLs, LHs, HHs, As, Ds, G, wf, k, K1, K2, ll_out, accum); break;
+      case 4: idwt_filter<4, FAST>(LLs, HLs, LHs, HHs, As, Ds, G, wf, k, K1, K2, ll_out, accum); break;
+      case 5: idwt_filter<5, FAST>(LLs, HLs, LHs, HHs, As, Ds, G, wf, k, K1, K2, ll_out, accum); break;
+      case 6: idwt_filter<6, FAST>(LLs, HLs, LHs, HHs, As, Ds, G, wf, k, K1, K2, ll_out, accum); break;
+      case 7: idwt_filter<7, FAST>(LLs, HLs, LHs, HHs, As, Ds, G, wf, k, K1, K2, ll_out, accum); break;
+      default: idwt_filter<8, FAST>(LLs, HLs, LHs, HHs, As, Ds, G, wf, k, K1, K2, ll_out, accum); break;
     }
   }
   if (G.last) {
 #pragma unroll
     for (int t = 0; t < kMaxOut; ++t) {
-      const int idx = threadIdx.x + t * blockDim.x;
-      if (idx >= nout) continue;
-      const int k1 = udiv(idx, d2TO), k2 = idx - k1 * (2 * TO);
-      const int gk1 = K1 + k1, gk2 = K2 + k2;
-      if (gk1 < L && gk2 < L) {
-        float2 s = accum[t];
-        const size_t j = (size_t)gk1 * G.n + gk2;
-        if (dirac_plane >= 0) s = cadd(s, coef[(size_t)dirac_plane * G.n * G.n + j]);
-        x[j] = cscale(s, G.scale);
+      int k1, k2;
+      if (FAST) {
+        const int qq = udiv(threadIdx.x, d2TO);
+        k1 = threadIdx.x - qq * (2 * TO);
+        k2 = 4 * qq + t;
+        if (k2 >= 2 * TO) continue;
+      } else {
+        const int idx = threadIdx.x + t * blockDim.x;
+        if (idx >= nout) continue;
+        k1 = udiv(idx, d2TO);
+        k2 = idx - k1 * (2 * TO);
       }
+      float2 s = accum[t];
+      const size_t j = (size_t)(K1 + k1) * G.n + K2 + k2;
+      if (dirac_plane >= 0) s = cadd(s, coef[(size_t)dirac_plane * G.n * G.n + j]);
+      x[j] = cscale(s, G.scale);
     }
   }
 }
@@ -536,7 +652,7 @@ static void basis_layout(const purify_ctx* c, int& dirac_plane, int& plane0, Bas
     if (c->bases[k] == 0) dirac_plane = k;
     else {
       if (nb == 0) plane0 = k;
-      bl.p[nb++] = c->bases[k];
+      bl.packed |= (unsigned)c->bases[k] << (4 * nb++);
     }
   }
 }
@@ -568,14 +684,27 @@ __global__ void k_finish_zeta(DevScalars* sc) {
   sc->f1_prev = sc->f1;
 }
 
+static WaveletTaps wavelet_taps(const WaveletFilters& wf) {
+  WaveletTaps t;
+  for (int p = 1; p <= 8; ++p) {
+    const float* h = wf.h + wf.off[p];
+    for (int m = 0; m < 2 * p; ++m) {
+      const float gm = (m & 1) ? -h[2 * p - 1 - m] : h[2 * p - 1 - m];
+      t.h[wf.off[p] + m] = make_float2(h[m], h[m]);
+      t.g[wf.off[p] + m] = make_float2(gm, gm);
+    }
+  }
+  return t;
+}
+
 static size_t dwt_smem(int TI, int taps) {
   const int RH = 2 * TI + taps - 2;
-  return (size_t)(RH * RH + RH * 2 * TI) * sizeof(float2);
+  return (size_t)(RH * (RH | 1) + RH * (2 * TI + 1)) * sizeof(float2);
 }
 
 static size_t idwt_smem(int TO, int p) {
   const int CW = TO + p - 1;
-  return (size_t)(4 * CW * CW + 2 * 2 * TO * CW) * sizeof(float2);
+  return (size_t)(4 * CW * CW + 2 * 2 * TO * (CW | 1)) * sizeof(float2);
 }
 
 int sara_analysis(purify_ctx* c, const float2* x, float2* alpha, SaraMode mode, const SaraProxArgs& pa,
@@ -601,7 +730,8 @@ int sara_analysis(purify_ctx* c, const float2* x, float2* alpha, SaraMode mode, 
     return check_cuda(cudaGetLastError());
   }
   int maxp = 1;
-  for (int k = 0; k < nb; ++k) maxp = std::max(maxp, bl.p[k]);
+  for (int k = 0; k < nb; ++k) maxp = std::max(maxp, bl.p(k));
+  const WaveletTaps taps = wavelet_taps(c->wf);
   int f1_off = 0;
   for (int lev = 0; lev < c->levels; ++lev) {
     const int L = c->n >> lev;
@@ -614,14 +744,19 @@ int sara_analysis(purify_ctx* c, const float2* x, float2* alpha, SaraMode mode, 
     f1_off += (int)(grid.x * grid.y * grid.z);
     if (mode == kSaraProx && f1_off > 2 * kMaxPartials) return PURIFY_E_SIZE;  // the kCntF1 slot holds 2 kMaxPartials
     const size_t sm = dwt_smem(TI, 2 * maxp);
-    if (mode == kSaraPlain)
-      PURIFY_LAUNCH(c, "dwt_level", s,
-                    (pdl_launch(k_dwt_level<kSaraPlain>, LaunchCfg{grid, 256, sm, s, lev > 0}, in, lev == 0, llo, alpha, G, bl, c->wf, pa,
-                                                                   c->d_partials, c->d_sc)));
-    else
-      PURIFY_LAUNCH(c, "dwt_level", s,
-                    (pdl_launch(k_dwt_level<kSaraProx>, LaunchCfg{grid, 256, sm, s, lev > 0}, in, lev == 0, llo, pa.z1, G, bl, c->wf, pa,
-                                                                  c->d_partials, c->d_sc)));
+    const LaunchCfg lc{grid, 256, sm, s, lev > 0};
+#define DWT(MD, FAST, COEF)                                                                                  \
+  PURIFY_LAUNCH(c, "dwt_level", s,                                                                           \
+                (pdl_launch(k_dwt_level<MD, FAST>, lc, in, lev == 0, llo, COEF, G, bl, taps, pa, c->d_partials, \
+                            c->d_sc)))
+    if (mode == kSaraPlain) {
+      if (TI % 4 == 0) DWT(kSaraPlain, true, alpha);
+      else DWT(kSaraPlain, false, alpha);
+    } else {
+      if (TI % 4 == 0) DWT(kSaraProx, true, pa.z1);
+      else DWT(kSaraProx, false, pa.z1);
+    }
+#undef DWT
   }
   if (mode == kSaraProx) {
     if (f1_parts) {
@@ -646,7 +781,8 @@ int sara_synthesis(purify_ctx* c, const float2* alpha, float2* x, cudaStream_t s
     return check_cuda(cudaGetLastError());
   }
   int maxp = 1;
-  for (int k = 0; k < nb; ++k) maxp = std::max(maxp, bl.p[k]);
+  for (int k = 0; k < nb; ++k) maxp = std::max(maxp, bl.p(k));
+  const WaveletTaps taps = wavelet_taps(c->wf);
   for (int lev = c->levels - 1; lev >= 0; --lev) {
     const int L = c->n >> lev;  // output side
     const int H = L / 2;
@@ -660,9 +796,14 @@ int sara_synthesis(purify_ctx* c, const float2* alpha, float2* x, cudaStream_t s
     const int f1n = (lev == c->levels - 1) ? f1_parts : 0;
     dim3 grid(L / (2 * TO), L / (2 * TO), (lev == 0 ? 1 : nb) + (f1n > 0 ? 1 : 0));
     const size_t sm = idwt_smem(TO, maxp);
-    PURIFY_LAUNCH(c, "idwt_level", s,
-                  (pdl_launch(k_idwt_level, LaunchCfg{grid, 256, sm, s}, llin, from_plane, llo, alpha, x, dirac_plane, G, bl, c->wf,
-                                                      c->d_partials + kCntF1 * 2 * kMaxPartials, f1n, c->d_sc)));
+    const LaunchCfg lc{grid, 256, sm, s};
+#define IDWT(FAST)                                                                                             \
+  PURIFY_LAUNCH(c, "idwt_level", s,                                                                            \
+                (pdl_launch(k_idwt_level<FAST>, lc, llin, from_plane, llo, alpha, x, dirac_plane, G, bl, taps, \
+                            c->d_partials + kCntF1 * 2 * kMaxPartials, f1n, c->d_sc)))
+    if (TO % 2 == 0) IDWT(true);
+    else IDWT(false);
+#undef IDWT
   }
   return check_cuda(cudaGetLastError());
 }
