@@ -307,15 +307,12 @@ void free_ctx(purify_ctx* c) {
 // G^T G as a stored stencil instead of gathering (measured on this GPU: the
 // stencil streams (2J - 1)^2 floats per cell from memory, the gather issues
 // ~1500 instructions per entry, and the two overlap in one launch).
-#ifndef PURIFY_DENSE_ENTRIES_PER_CELL
-#define PURIFY_DENSE_ENTRIES_PER_CELL 2.0
-#endif
-constexpr double kDenseEntriesPerCell = PURIFY_DENSE_ENTRIES_PER_CELL;
-// ... and one per cell, stored by half, when those stencils fit a quarter of L2
-#ifndef PURIFY_DENSE_ENTRIES_PER_CELL_L2
-#define PURIFY_DENSE_ENTRIES_PER_CELL_L2 1.0
-#endif
-constexpr double kDenseEntriesPerCellL2 = PURIFY_DENSE_ENTRIES_PER_CELL_L2;
+constexpr double kDenseEntriesPerCell = 2.0;
+// ... and one per cell, stored by half, when those stencils fit a quarter of
+// L2; with J <= 4 down to this many per cell and slice (all tiles of small grids)
+constexpr double kDenseEntriesPerCellL2 = 1.0;
+constexpr double kDenseEntriesPerSlice = 0.01;
+constexpr size_t kDenseAllBytes = (size_t)8 << 20;
 constexpr size_t kDenseL2Bytes = (size_t)32 << 20;
 
 // G^T G restricted to the cells of the dense tiles (§5: G^H G, precomputed
@@ -487,6 +484,7 @@ int setup_visibilities(purify_ctx* c, const float* uv_in, cudaStream_t s) {
   prm.L = c->L;
   prm.J = c->J;
   prm.T = T;
+  prm.home_T = c->homeT;
   prm.fixed_bytes = purify::grid_fixed_bytes(T, c->J);
   prm.entry_bytes = purify::grid_entry_bytes(c->J);
   prm.smem_budget = purify::kGridSmemBudget;
@@ -543,17 +541,35 @@ int setup_visibilities(purify_ctx* c, const float* uv_in, cudaStream_t s) {
   }
   // dense tiles of the Gram pass and their stored G^T G (see build_dense_gram)
   if (st == PURIFY_OK) {
-    // layout: the half stencil, with one entry per cell as the threshold,
-    // when those stencils fit a quarter of L2 (they stay resident across the
-    // CG steps; 256^2 workload: Gram 15.4 -> 12.8 us); the full stencil, two
-    // entries per cell, otherwise (HBM-streamed: 1024^2 half 136.8 us, full
-    // 130.9 us)
+    // layout: half stencils when those of the tiles with more than one entry
+    // per cell fit a quarter of L2 (they stay resident across the CG steps;
+    // 256^2 workload: Gram 15.4 -> 12.8 us); the full stencil, two entries per
+    // cell, otherwise (HBM-streamed: 1024^2 half 136.8 us, full 130.9 us).
+    // With J <= 4 (at most 25 slices) half stencils go down to the lowest
+    // threshold that still fits, bounded by where the two forms cost the same,
+    // near 0.01 entries per cell and slice (SDMM iteration, 256^2, M = 30000,
+    // J = 4: thresholds 1, 0.5, 0.25, 0: 306, 298, 271, 288 us), and small
+    // grids take them for every tile that has entries: a launch of stencils
+    // alone is shorter than one gather CTA (64^2, M = 2048: 209 -> 188 us;
+    // 128^2, M = 20000: 229 -> 215 us).  With J = 6 (61 slices) a lower
+    // threshold gains nothing (0.61: 256^2 330 -> 325 us, 96^2 274 -> 285 us,
+    // 384^2 515 -> 524 us).
     const size_t half_bytes = (size_t)dense_gram_slices(c->J) * (T + c->J - 1) * (T + 2 * (c->J - 1)) * 4;
-    int n_low = 0;
-    for (int t = 0; t < c->ntiles; ++t)
-      if ((double)(plan.list_off[t + 1] - plan.list_off[t]) > kDenseEntriesPerCellL2 * T * T) ++n_low;
-    c->dense_half = (size_t)n_low * half_bytes <= kDenseL2Bytes ? 1 : 0;
-    const double per_cell = c->dense_half ? kDenseEntriesPerCellL2 : kDenseEntriesPerCell;
+    auto denser_than = [&](double per_cell) {
+      size_t nt = 0;
+      for (int t = 0; t < c->ntiles; ++t)
+        if ((double)(plan.list_off[t + 1] - plan.list_off[t]) > per_cell * T * T) ++nt;
+      return nt;
+    };
+    c->dense_half = denser_than(kDenseEntriesPerCellL2) * half_bytes <= kDenseL2Bytes ? 1 : 0;
+    double per_cell = kDenseEntriesPerCell;
+    if (c->dense_half) {
+      if (c->J <= 4) per_cell = kDenseEntriesPerSlice * dense_gram_slices(c->J);
+      else per_cell = kDenseEntriesPerCellL2;
+      if (c->J <= 4 && denser_than(0.0) * half_bytes <= kDenseAllBytes) per_cell = 0.0;
+      while (per_cell < kDenseEntriesPerCellL2 && denser_than(per_cell) * half_bytes > kDenseL2Bytes)
+        per_cell = std::min(kDenseEntriesPerCellL2, 1.25 * per_cell);
+    }
     std::vector<int> dense;
     std::vector<char> is_dense(c->ntiles, 0);
     for (int t = 0; t < c->ntiles; ++t)
@@ -772,10 +788,15 @@ static int purify_create_impl(purify_ctx** out, const purify_desc* d, const floa
   c->fft_engine = fft_fixed_side(c->L) ? 1 : 0;
   make_daubechies(c->wf);
   if (d->tile != 0) {
-    c->tileT = d->tile;
+    c->tileT = c->homeT = d->tile;
   } else {
-    c->tileT = c->L >= 512 ? 32 : (c->L >= 64 ? 16 : 8);
-    while (c->tileT < c->J || c->L % c->tileT) c->tileT *= 2;
+    c->homeT = c->L >= 512 ? 32 : (c->L >= 64 ? 16 : 8);
+    while (c->homeT < c->J || c->L % c->homeT) c->homeT *= 2;
+    // gridding tiles of a 512 grid: 32 would leave 256 tiles, not two per SM
+    // (SDMM iteration at 256^2, M = 65536: tiles of 32 325 us, of 16 303 us; on
+    // 768 and larger grids 32 is the faster one, 384^2: 527 against 547 us).
+    // The sort keeps its tile: exported states and bf16 blocks follow it.
+    c->tileT = c->L == 512 ? 16 : c->homeT;
   }
   c->tiles_1d = c->L / c->tileT;
   c->ntiles = c->tiles_1d * c->tiles_1d;

@@ -343,7 +343,8 @@ struct purify_ctx {
   // visibility table (sorted by grid tile of the first footprint cell)
   float2* d_uv;         // M sorted frequencies
   int* d_perm;          // sorted position -> caller position
-  int tileT;            // tile side (cells)
+  int tileT;            // gridding tile side (cells)
+  int homeT;            // tile side of the visibility sort and the degridding
   int tiles_1d;         // L / tileT
   int ntiles;
   int4* d_list;         // per tile, the visibilities whose footprint meets it, by start cell:

@@ -12,7 +12,9 @@ int build_gather_plan(const int* k0, const GatherPlanParams& prm, GatherPlan& ou
   if (M < 0 || T < 2 || (T & (T - 1)) != 0 || T > 64 || L % T != 0 || J < 2 || J > 8 || J > L ||
       prm.entry_bytes == 0 || prm.tab_stride < (T / 2) * (T / 2) + 1 || prm.max_partials < 2)
     return -1;
-  const int TD = L / T, ntiles = TD * TD;
+  const int HT = prm.home_T > 0 ? prm.home_T : T;
+  if ((HT & (HT - 1)) != 0 || HT < 2 || L % HT != 0) return -1;
+  const int TD = L / T, ntiles = TD * TD, HD = L / HT, nhome = HD * HD;
   out = GatherPlan{};
   out.ntiles = ntiles;
   out.tiles_1d = TD;
@@ -23,13 +25,13 @@ int build_gather_plan(const int* k0, const GatherPlanParams& prm, GatherPlan& ou
 
   // counting sort by home tile (stable: keeps the caller's order inside a tile)
   std::vector<int>& cnt = out.home;
-  cnt.assign(ntiles + 1, 0);
+  cnt.assign(nhome + 1, 0);
   out.perm.resize(M);
-  for (int64_t i = 0; i < M; ++i) cnt[(kr_of(i) / T) * TD + kc_of(i) / T + 1]++;
-  for (int t = 0; t < ntiles; ++t) cnt[t + 1] += cnt[t];
+  for (int64_t i = 0; i < M; ++i) cnt[(kr_of(i) / HT) * HD + kc_of(i) / HT + 1]++;
+  for (int t = 0; t < nhome; ++t) cnt[t + 1] += cnt[t];
   {
     std::vector<int> pos(cnt.begin(), cnt.end() - 1);
-    for (int64_t i = 0; i < M; ++i) out.perm[pos[(kr_of(i) / T) * TD + kc_of(i) / T]++] = (int)i;
+    for (int64_t i = 0; i < M; ++i) out.perm[pos[(kr_of(i) / HT) * HD + kc_of(i) / HT]++] = (int)i;
   }
 
   // per-tile lists of sorted indices whose footprint meets the tile
@@ -175,7 +177,7 @@ int build_gather_plan(const int* k0, const GatherPlanParams& prm, GatherPlan& ou
   // order) in chunks of at most dch; dch keeps the number of chunks (one FP64
   // partial-sum slot each) within max_partials: at most ntiles + M / dch
   const int64_t dch = std::max<int64_t>(1024, (2 * M + prm.max_partials - 1) / prm.max_partials);
-  for (int t = 0; t < ntiles; ++t) {
+  for (int t = 0; t < nhome; ++t) {
     const int b = cnt[t], e = cnt[t + 1];
     const int nc = (int)((e - b + dch - 1) / dch);
     for (int k = 0; k < nc; ++k) {

@@ -47,6 +47,7 @@ struct GatherPlanParams {
   int L;                 // grid side
   int J;                 // footprint side (<= 8)
   int T;                 // tile side (power of two, divides L, <= 64)
+  int home_T = 0;        // tile side of the visibility sort and the degridding units (0: T)
   size_t fixed_bytes;    // shared memory of a gridding CTA without its entries
   size_t entry_bytes;    // shared memory per staged entry
   size_t smem_budget;    // target shared memory of a gridding CTA
@@ -55,9 +56,9 @@ struct GatherPlanParams {
 };
 
 struct GatherPlan {
-  int ntiles = 0, tiles_1d = 0;
+  int ntiles = 0, tiles_1d = 0;           // gridding tiles (side T)
   std::vector<int> perm;        // sorted position -> caller index (M)
-  std::vector<int> home;        // ntiles + 1: home visibilities of tile t are sorted [home[t], home[t+1])
+  std::vector<int> home;        // home tiles + 1: home visibilities of tile t (side home_T) are sorted [home[t], home[t+1])
   std::vector<int> list_off;    // ntiles + 1: list entries of tile t are [list_off[t], list_off[t+1])
   std::vector<int> list;        // sorted index of each list entry
   std::vector<int> lkey;        // start-cell key of each list entry

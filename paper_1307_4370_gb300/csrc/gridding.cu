@@ -618,14 +618,14 @@ constexpr int kDegridPerSm = 8;  // CTAs of the SDMM mode per SM (4: 108 us, 8: 
 template <int J>
 static void degrid_J(purify_ctx* c, DegridOut mode, const DegridArgs& a, cudaStream_t s) {
   const int threads = 256;
-  const int W = c->tileT + J - 1;
+  const int W = c->homeT + J - 1;
   const size_t sm = (size_t)W * W * sizeof(float2);
 #define DEG(MD)                                                                                               \
   do {                                                                                                        \
     allow_smem(k_degrid<J, MD>, sm);                                                                          \
     PURIFY_LAUNCH(c, "degrid", s,                                                                             \
                   (pdl_launch(k_degrid<J, MD>, LaunchCfg{MD == kDegridSdmm ? std::min(c->ndchunks, kDegridPerSm * c->sms) : c->ndchunks, threads, sm, s}, c->d_grid, c->d_uv, c->d_perm, a, c->d_dchunks, \
-                                                                    c->ndchunks, c->kb, c->ks, c->L, c->tileT, c->tiles_1d,     \
+                                                                    c->ndchunks, c->kb, c->ks, c->L, c->homeT, c->L / c->homeT, \
                                                                     c->d_partials, c->d_sc)));                     \
   } while (0)
   if (mode == kDegridPerm) DEG(kDegridPerm);
