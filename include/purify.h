@@ -311,7 +311,7 @@ int purify_sdmm_step(purify_ctx* ctx, purify_sdmm_state* st, purify_stream_t str
  * until reweighted by purify_sdmm_reweight with delta / (delta + |grad x_hat|));
  * its prox is `fgp_iters` (1..1000) iterations of Beck & Teboulle's fast
  * gradient projection on the dual (§5), and gamma = beta max |grad Phi^H y|.
- * Call before purify_sdmm_init.  Allocates the prox scratch (7 N complex64)
+ * Call before purify_sdmm_init.  Allocates the prox scratch (9 N complex64)
  * on the context.  PURIFY_E_INVALID_ARG for an unknown prior or iteration
  * count. */
 int purify_sdmm_set_prior(purify_ctx* ctx, purify_sdmm_state* st, int32_t prior,
