@@ -184,6 +184,63 @@ KbPoly fit_kb(int J, int kernel) {
   return kb;
 }
 
+// The same taps for the host's set-up, in double: Chebyshev interpolants of
+// degree 16 in z = 2x - 1, within 1e-12 of the kernels (checked at set-up), at
+// a tenth of the time of the Bessel function, which was a quarter of the
+// set-up at M = 2^21.
+struct TapSeries {
+  static constexpr int kTerms = 17;
+  int J, kernel;
+  bool exact;  // the series is not that good: evaluate g
+  double c[kMaxJ][kTerms];
+};
+
+double tap_value(const double* c, double z) {  // Clenshaw's recurrence
+  double b1 = 0.0, b2 = 0.0;
+  for (int k = TapSeries::kTerms - 1; k >= 1; --k) {
+    const double b0 = c[k] + 2.0 * z * b1 - b2;
+    b2 = b1;
+    b1 = b0;
+  }
+  return c[0] + z * b1 - b2;
+}
+
+TapSeries fit_taps(int J, int kernel) {
+  const double beta = kb_beta(J), i0b = std::cyl_bessel_i(0.0, beta);
+  constexpr int np = TapSeries::kTerms;
+  TapSeries p{};
+  p.J = J;
+  p.kernel = kernel;
+  double err = 0.0;
+  for (int a = 0; a < J; ++a) {
+    double f[np];
+    for (int i = 0; i < np; ++i)
+      f[i] = interp_g(0.5 * (std::cos(M_PI * (i + 0.5) / np) + 1.0) + J / 2 - 1 - a, J, kernel, beta, i0b);
+    for (int k = 0; k < np; ++k) {
+      double sum = 0.0;
+      for (int i = 0; i < np; ++i) sum += f[i] * std::cos(M_PI * k * (i + 0.5) / np);
+      p.c[a][k] = sum * (k == 0 ? 1.0 : 2.0) / np;
+    }
+    for (int t = 0; t < 64; ++t) {
+      const double x = (t + 0.37) / 64.0;
+      err = std::max(err, std::fabs(tap_value(p.c[a], 2.0 * x - 1.0) -
+                                    interp_g(x + J / 2 - 1 - a, J, kernel, beta, i0b)));
+    }
+  }
+  p.exact = !(err < 2e-12);
+  return p;
+}
+
+// Weights of the J taps for the fraction x in [0, 1).
+void tap_weights(const TapSeries& p, double x, double* w) {
+  if (p.exact) {
+    const double beta = kb_beta(p.J), i0b = std::cyl_bessel_i(0.0, beta);
+    for (int a = 0; a < p.J; ++a) w[a] = interp_g(x + p.J / 2 - 1 - a, p.J, p.kernel, beta, i0b);
+    return;
+  }
+  for (int a = 0; a < p.J; ++a) w[a] = tap_value(p.c[a], 2.0 * x - 1.0);
+}
+
 FftPlan make_plan(int L) {
   FftPlan p{};
   p.L = L;
@@ -236,6 +293,16 @@ __global__ void k_list_setup(const int2* __restrict__ lk, const float2* __restri
     split_kappa(u.x, ks, kr, fr);
     split_kappa(u.y, ks, kc, fc);
     out[e] = make_int4(v.x, v.y, __float_as_int(fr), __float_as_int(fc));
+  }
+}
+
+// Caller positions and frequencies in the degridding's order.
+__global__ void k_order_setup(int64_t M, const int* __restrict__ dpos, const int* __restrict__ perm,
+                              const float2* __restrict__ uv_user, int* __restrict__ dperm, float2* __restrict__ uv) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < M; i += (int64_t)gridDim.x * blockDim.x) {
+    const int m = perm[dpos[i]];
+    dperm[i] = m;
+    uv[i] = uv_user[m];
   }
 }
 
@@ -292,7 +359,7 @@ void encode_halo_map(purify_ctx* c) {
 
 void free_ctx(purify_ctx* c) {
   if (!c) return;
-  void* ptrs[] = {c->d_dense_tiles, c->d_H, c->d_gram_chunks, c->d_diff, c->d_twp[0], c->d_twp[1], c->d_deapod, c->d_beam, c->d_tv, c->d_tw, c->d_uv, c->d_perm, c->d_list, c->d_chunks, c->d_chunk_tab, c->d_items, c->d_item_row, c->d_dchunks, c->d_tile_slot0,
+  void* ptrs[] = {c->d_dense_tiles, c->d_H, c->d_gram_chunks, c->d_diff, c->d_twp[0], c->d_twp[1], c->d_deapod, c->d_beam, c->d_tv, c->d_tw, c->d_uv, c->d_dpos, c->d_dperm, c->d_perm, c->d_list, c->d_chunks, c->d_chunk_tab, c->d_items, c->d_item_row, c->d_dchunks, c->d_tile_slot0,
                   c->d_tile_nchunk, c->d_tile_cnt, c->d_slots,
                   c->d_grid, c->d_grid2, c->d_half, c->d_vis, c->d_vis2, c->d_ll[0], c->d_ll[1], c->d_img[0],
                   c->d_img[1], c->d_img[2], c->d_img[3], c->d_partials, c->d_sc};
@@ -315,18 +382,29 @@ constexpr double kDenseEntriesPerSlice = 0.01;
 constexpr size_t kDenseAllBytes = (size_t)8 << 20;
 constexpr size_t kDenseL2Bytes = (size_t)32 << 20;
 
+// Visibilities from which purify_phi_adj sorts its input first.
+constexpr int64_t kPermFirst = (int64_t)1 << 20;
+
+// Threads that build the stencils.
+unsigned pool_threads(const purify::GatherPlan& plan, const std::vector<int>& dense, int J) {
+  double work = 0;  // multiply-adds: J^4 per list entry; a thread starts in the time of a few 10^5
+  for (int t : dense) work += (double)(plan.list_off[t + 1] - plan.list_off[t]) * J * J * J * J;
+  const unsigned hw = std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
+  return std::max(1u, std::min(hw, (unsigned)std::min(16.0, work / 1e6)));
+}
+
 // G^T G restricted to the cells of the dense tiles (§5: G^H G, precomputed
 // and stored, to speed up the CG solve): for cell k of tile t and offset d in
 // [-(J-1), J-1]^2, H[t][d][k] = sum over the tile's list entries m of
 // w_m(k) w_m(k + d), w_m the J x J interpolation weights of visibility m
-// (exact kernel values in double, at the fractions the device uses).  Every
+// (kernel values in double, at the fractions the device uses).  Every
 // visibility whose footprint covers a cell of the tile is on the tile's list,
 // so (G^T G X)(k) = sum_d H[t][d][k] X(k + d) exactly.  Built in double on
 // the host, one tile per thread of a small pool, and stored as float.
 int build_dense_gram(const purify_ctx* c, const purify::GatherPlan& plan, const std::vector<int4>& entries,
                       const std::vector<int>& dense, std::vector<float>& H) {
   const int T = c->tileT, J = c->J, W = T + J - 1, ND = (2 * J - 1) * (2 * J - 1), TT = T * T;
-  const double beta = kb_beta(J), i0b = std::cyl_bessel_i(0.0, beta);
+  const TapSeries taps = fit_taps(J, c->kernel);
   H.assign((size_t)dense.size() * ND * TT, 0.0f);
   std::atomic<size_t> next{0};
   std::atomic<bool> failed{false};
@@ -343,10 +421,8 @@ int build_dense_gram(const purify_ctx* c, const purify::GatherPlan& plan, const 
           std::memcpy(&frf, &le.z, 4);
           std::memcpy(&fcf, &le.w, 4);
           double wr[kMaxJ], wc[kMaxJ];
-          for (int a = 0; a < J; ++a) {
-            wr[a] = interp_g((double)frf + J / 2 - 1 - a, J, c->kernel, beta, i0b);
-            wc[a] = interp_g((double)fcf + J / 2 - 1 - a, J, c->kernel, beta, i0b);
-          }
+          tap_weights(taps, frf, wr);
+          tap_weights(taps, fcf, wc);
           for (int a = 0; a < J; ++a) {
             const int r = kr - (J - 1) + a;
             if (r < 0 || r >= T) continue;
@@ -369,7 +445,7 @@ int build_dense_gram(const purify_ctx* c, const purify::GatherPlan& plan, const 
       failed = true;
     }
   };
-  const unsigned hw = std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
+  const unsigned hw = pool_threads(plan, dense, J);
   std::vector<std::thread> pool;
   try {
     for (unsigned i = 1; i < hw; ++i) pool.emplace_back(work);
@@ -397,7 +473,7 @@ int build_dense_gram_half(const purify_ctx* c, const purify::GatherPlan& plan, c
                            const std::vector<int>& dense, std::vector<float>& H) {
   const int T = c->tileT, J = c->J, W = T + J - 1, NDW = 2 * J - 1;
   const int NH = dense_gram_slices(J), EW = T + 2 * (J - 1), EH = T + J - 1, ES = EW * EH;
-  const double beta = kb_beta(J), i0b = std::cyl_bessel_i(0.0, beta);
+  const TapSeries taps = fit_taps(J, c->kernel);
   H.assign((size_t)dense.size() * NH * ES, 0.0f);
   std::atomic<size_t> next{0};
   std::atomic<bool> failed{false};
@@ -414,10 +490,8 @@ int build_dense_gram_half(const purify_ctx* c, const purify::GatherPlan& plan, c
           std::memcpy(&frf, &le.z, 4);
           std::memcpy(&fcf, &le.w, 4);
           double wr[kMaxJ], wc[kMaxJ];
-          for (int a = 0; a < J; ++a) {
-            wr[a] = interp_g((double)frf + J / 2 - 1 - a, J, c->kernel, beta, i0b);
-            wc[a] = interp_g((double)fcf + J / 2 - 1 - a, J, c->kernel, beta, i0b);
-          }
+          tap_weights(taps, frf, wr);
+          tap_weights(taps, fcf, wc);
           // every ordered pair of footprint cells (a, b) -> (a2, b2) with a
           // lexicographically non-negative offset, accumulated at the first cell
           for (int a = 0; a < J; ++a) {
@@ -446,7 +520,7 @@ int build_dense_gram_half(const purify_ctx* c, const purify::GatherPlan& plan, c
       failed = true;
     }
   };
-  const unsigned hw = std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
+  const unsigned hw = pool_threads(plan, dense, J);
   std::vector<std::thread> pool;
   try {
     for (unsigned i = 1; i < hw; ++i) pool.emplace_back(work);
@@ -506,6 +580,7 @@ int setup_visibilities(purify_ctx* c, const float* uv_in, cudaStream_t s) {
   c->ndchunks = (int)plan.dchunks.size();
   const int nslots = plan.nslots;
   if ((st = dev_alloc(&c->d_uv, M)) == PURIFY_OK && (st = dev_alloc(&c->d_perm, M)) == PURIFY_OK &&
+      (st = dev_alloc(&c->d_dpos, M)) == PURIFY_OK && (st = dev_alloc(&c->d_dperm, M)) == PURIFY_OK &&
       (st = dev_alloc(&c->d_list, c->nlist)) == PURIFY_OK && (st = dev_alloc(&d_lk, c->nlist)) == PURIFY_OK &&
       (st = dev_alloc(&c->d_chunks, c->nchunks)) == PURIFY_OK &&
       (st = dev_alloc(&c->d_chunk_tab, (size_t)c->nchunks * c->chunk_tab_stride)) == PURIFY_OK &&
@@ -524,6 +599,10 @@ int setup_visibilities(purify_ctx* c, const float* uv_in, cudaStream_t s) {
       launch_gather_perm(M, d_uv_user, c->d_perm, c->d_uv, s);
       PURIFY_LAUNCH(c, "list_setup", s,
                     (k_list_setup<<<nblk(c->nlist), 256, 0, s>>>(d_lk, c->d_uv, c->ks, c->nlist, c->d_list)));
+      // the degridding's order, and its frequencies in place of the sorted ones
+      cudaMemcpyAsync(c->d_dpos, plan.dorder.data(), M * sizeof(int), cudaMemcpyHostToDevice, s);
+      PURIFY_LAUNCH(c, "order_setup", s,
+                    (k_order_setup<<<nblk(M), 256, 0, s>>>(M, c->d_dpos, c->d_perm, d_uv_user, c->d_dperm, c->d_uv)));
       if (cudaStreamSynchronize(s) != cudaSuccess) st = PURIFY_E_CUDA;
     }
     static_assert(sizeof(purify::PlanI4) == sizeof(int4), "plan work units have the layout of int4");
@@ -911,7 +990,16 @@ int purify_phi_adj(purify_ctx* c, const float* y, float* x, purify_stream_t stre
   DeviceGuard g(c->device);
   if (!is_device_ptr(x) || !is_device_ptr(y)) return PURIFY_E_NOT_DEVICE_PTR;
   cudaStream_t s = (cudaStream_t)stream;
-  TRY(grid_adjoint(c, kGridPerm, (const float2*)y, s));
+  if (c->M >= kPermFirst) {
+    // many visibilities: brought into sorted order once, instead of by every
+    // tile list that holds them (1024^2, M = 2^21: gridding through the
+    // permutation 168 us, sorted 146 us after 9 us for the gather; below, the
+    // launch costs what it saves)
+    TRY(launch_gather_perm(c->M, (const float2*)y, c->d_perm, c->d_vis, s));
+    TRY(grid_adjoint(c, kGridSorted, c->d_vis, s));
+  } else {
+    TRY(grid_adjoint(c, kGridPerm, (const float2*)y, s));
+  }
   RowOutArgs ra{};
   ra.out = (float2*)x;
   return phi_adjoint_image(c, kRowOutPlain, ra, s);
@@ -1018,9 +1106,7 @@ void purify_sdmm_state_destroy(purify_sdmm_state* st) {
   if (st->side) cudaStreamDestroy(st->side);
   if (st->ev_fork) cudaEventDestroy(st->ev_fork);
   if (st->ev_join) cudaEventDestroy(st->ev_join);
-  void* ptrs[] = {st->xhat, st->r, st->p, st->qp, st->sv, st->x1, st->z3, st->z1, st->u1,
-                  st->w, st->y, st->yb, st->yscale, st->z2, st->s2, st->v,
-                  st->d_block_of, st->d_pos, st->d_bchunks, st->d_beps, st->d_bscale};
+  void* ptrs[] = {st->slab, st->d_block_of, st->d_pos, st->d_bchunks, st->d_beps, st->d_bscale};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   delete st;
@@ -1034,15 +1120,34 @@ int purify_sdmm_state_create(purify_ctx* c, purify_sdmm_state** out) {
   if (!st) return PURIFY_E_ALLOC;
   st->ctx = c;
   const int64_t N = ctx_N(c), D = ctx_D(c), M = c->M;
-  int e;
-  if ((e = dev_alloc(&st->xhat, N)) || (e = dev_alloc(&st->r, N)) || (e = dev_alloc(&st->p, N)) ||
-      (e = dev_alloc(&st->qp, N)) || (e = dev_alloc(&st->sv, N)) || (e = dev_alloc(&st->x1, N)) ||
-      (e = dev_alloc(&st->z3, N)) ||
-      (e = dev_alloc(&st->z1, D)) || (e = dev_alloc(&st->u1, D)) || (e = dev_alloc(&st->w, D)) ||
-      (e = dev_alloc(&st->y, M)) || (e = dev_alloc(&st->yb, 2 * M)) || (e = dev_alloc(&st->yscale, (M + 4095) / 4096)) ||
-      (e = dev_alloc(&st->z2, M)) || (e = dev_alloc(&st->s2, M)) || (e = dev_alloc(&st->v, M))) {
-    purify_sdmm_state_destroy(st);
-    return e;
+  // one allocation; the vectors that purify_sdmm_init clears come first, so
+  // that one memset clears them (a malloc and a free each and twelve memsets
+  // were a fifth of a 64^2 solve's time outside its iterations)
+  {
+    struct Part {
+      void** p;
+      size_t bytes;
+    };
+    const size_t c8 = sizeof(float2);
+    const Part parts[] = {{(void**)&st->xhat, N * c8}, {(void**)&st->r, N * c8},  {(void**)&st->p, N * c8},
+                          {(void**)&st->qp, N * c8},   {(void**)&st->sv, N * c8}, {(void**)&st->x1, N * c8},
+                          {(void**)&st->z3, N * c8},   {(void**)&st->z1, D * c8}, {(void**)&st->u1, D * c8},
+                          {(void**)&st->z2, M * c8},   {(void**)&st->s2, M * c8}, {(void**)&st->v, M * c8},
+                          {(void**)&st->w, D * sizeof(float)}, {(void**)&st->y, M * c8},
+                          {(void**)&st->yb, 2 * M * sizeof(uint16_t)},
+                          {(void**)&st->yscale, (M + 4095) / 4096 * sizeof(float)}};
+    size_t total = 0;
+    for (const Part& q : parts) total += (q.bytes + 255) / 256 * 256;
+    const int e = dev_alloc(&st->slab, total);
+    if (e != PURIFY_OK) {
+      purify_sdmm_state_destroy(st);
+      return e;
+    }
+    char* at = st->slab;
+    for (const Part& q : parts) {
+      *q.p = at;
+      at += (q.bytes + 255) / 256 * 256;
+    }
   }
   if (cudaStreamCreateWithFlags(&st->side, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&st->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
@@ -1082,18 +1187,8 @@ int purify_sdmm_init(purify_ctx* c, purify_sdmm_state* st, const float* y, doubl
   TRY(load_data(c, st, y, s));
   st->eps = eps;
   st->iters = 0;
-  TRY_CUDA(cudaMemsetAsync(st->xhat, 0, N * sizeof(float2), s));
-  TRY_CUDA(cudaMemsetAsync(st->r, 0, N * sizeof(float2), s));
-  TRY_CUDA(cudaMemsetAsync(st->p, 0, N * sizeof(float2), s));
-  TRY_CUDA(cudaMemsetAsync(st->qp, 0, N * sizeof(float2), s));
-  TRY_CUDA(cudaMemsetAsync(st->sv, 0, N * sizeof(float2), s));
-  TRY_CUDA(cudaMemsetAsync(st->x1, 0, N * sizeof(float2), s));
-  TRY_CUDA(cudaMemsetAsync(st->z3, 0, N * sizeof(float2), s));
-  TRY_CUDA(cudaMemsetAsync(st->z1, 0, D * sizeof(float2), s));
-  TRY_CUDA(cudaMemsetAsync(st->u1, 0, D * sizeof(float2), s));
-  TRY_CUDA(cudaMemsetAsync(st->z2, 0, M * sizeof(float2), s));
-  TRY_CUDA(cudaMemsetAsync(st->s2, 0, M * sizeof(float2), s));
-  TRY_CUDA(cudaMemsetAsync(st->v, 0, M * sizeof(float2), s));
+  // x_hat, r, p, w = Qr, s, x1, z3, z1, u1, z2, s2 and v (the slab's first part)
+  TRY_CUDA(cudaMemsetAsync(st->slab, 0, (size_t)((char*)st->w - st->slab), s));
   PURIFY_LAUNCH(c, "fill", s, (k_fill_f32<<<nblk(D), 256, 0, s>>>(D, st->w, 1.0f)));
   TRY_CUDA(cudaGetLastError());
   // scalars: everything zero but eps

@@ -341,7 +341,9 @@ struct purify_ctx {
   float2* d_twp[2];     // per-stage twiddle tables of that engine (8 or 12, 16 or 24 per thread)
 
   // visibility table (sorted by grid tile of the first footprint cell)
-  float2* d_uv;         // M sorted frequencies
+  float2* d_uv;         // M frequencies in the degridding's order
+  int* d_dpos;          // degridding order -> sorted position
+  int* d_dperm;         // degridding order -> caller position
   int* d_perm;          // sorted position -> caller position
   int tileT;            // gridding tile side (cells)
   int homeT;            // tile side of the visibility sort and the degridding
@@ -448,6 +450,7 @@ struct GraphKey {
 
 struct purify_sdmm_state {
   purify_ctx* ctx;
+  char* slab;     // the allocation that holds the vectors below
   // image-size vectors
   float2* xhat;   // N
   float2* r;      // N  CG residual
@@ -551,7 +554,7 @@ int cg_partial_blocks(const purify_ctx* c);
 // one-block kernel after the inverse row pass (many partials: at 256
 // partials, e.g. 1024^2, every block of the 1024-block forward row pass
 // summing them cost 9 us per CG step against ~2 us for the extra launch).
-constexpr int kCgConsumeMaxBlocks = 128;
+constexpr int kCgConsumeMaxBlocks = 192;
 int cg_consumer_blocks(const purify_ctx* c);  // nblk for the consumers: the partial count, or 0
 int launch_cg_scalars(purify_ctx* c, int cg_j, cudaStream_t s);
 int degrid(purify_ctx* c, DegridOut mode, const DegridArgs& a, cudaStream_t s);

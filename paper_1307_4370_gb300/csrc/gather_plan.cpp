@@ -75,20 +75,48 @@ int build_gather_plan(const int* k0, const GatherPlanParams& prm, GatherPlan& ou
     return t >= L - (J - 1) ? t - L : t;
   };
   {
+    // (counting sort by key, stable; a comparison sort was a tenth of the set-up
+    // at M = 2^21)
     std::vector<std::pair<int, int>> seg;
+    std::vector<int> at(W * W + 1);
     for (int t = 0; t < ntiles; ++t) {
+      if (lcnt[t] == lcnt[t + 1]) continue;
       const int R0 = (t / TD) * T, C0 = (t % TD) * T;
       seg.clear();
+      std::fill(at.begin(), at.end(), 0);
       for (int e = lcnt[t]; e < lcnt[t + 1]; ++e) {
         const int64_t i = out.perm[out.list[e]];
         const int key = (rel(kr_of(i), R0) + J - 1) * W + (rel(kc_of(i), C0) + J - 1);
         seg.emplace_back(key, out.list[e]);
+        ++at[key + 1];
       }
-      std::stable_sort(seg.begin(), seg.end(),
-                       [](const std::pair<int, int>& x, const std::pair<int, int>& y) { return x.first < y.first; });
-      for (size_t k = 0; k < seg.size(); ++k) {
-        out.list[lcnt[t] + k] = seg[k].second;
-        out.lkey[lcnt[t] + k] = seg[k].first;
+      for (int k = 0; k < W * W; ++k) at[k + 1] += at[k];
+      for (const auto& v : seg) {
+        const int k = lcnt[t] + at[v.first]++;
+        out.list[k] = v.second;
+        out.lkey[k] = v.first;
+      }
+    }
+  }
+
+  // the degridding's order: the visibilities that start in a gridding tile (key
+  // row and column at least J - 1) are in its list by start cell; the gridding
+  // tiles of a home tile one after the other
+  out.dorder.resize(M);
+  {
+    const int sub = HT / T > 0 ? HT / T : 1;
+    std::vector<int> pos(cnt.begin(), cnt.end() - 1);
+    for (int t = 0; t < ntiles; ++t) {
+      const int h = HT >= T ? (t / TD / sub) * HD + (t % TD) / sub : -1;
+      for (int e = lcnt[t]; e < lcnt[t + 1]; ++e) {
+        const int k = out.lkey[e], si = out.list[e];
+        if (k / W < J - 1 || k % W < J - 1) continue;
+        int hh = h;
+        if (hh < 0) {  // (home tiles smaller than the gridding's)
+          const int64_t i = out.perm[si];
+          hh = (kr_of(i) / HT) * HD + kc_of(i) / HT;
+        }
+        out.dorder[pos[hh]++] = si;
       }
     }
   }

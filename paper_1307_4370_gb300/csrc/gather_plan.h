@@ -71,7 +71,11 @@ struct GatherPlan {
   std::vector<int> item_row;    // per chunk: first row of its items
   std::vector<uint32_t> items;  // rows x kGridThreads: step s of thread j of a chunk at row item_row + s, column j
   int64_t nitem_rows = 0;
-  std::vector<PlanI4> dchunks;  // degridding units (tile, sorted begin, sorted end, 0), heavy first
+  std::vector<PlanI4> dchunks;  // degridding units (home tile, begin, end, 0), heavy first: runs of [home[t], home[t + 1])
+  // sorted positions in the order the degridding takes them: every home tile's
+  // visibilities by gridding tile and first footprint cell, so that the lanes
+  // of a warp read neighbouring (or the same) cells of the staged halo
+  std::vector<int> dorder;
 };
 
 // Returns 0, or -1 for invalid parameters, -2 when the tile lists exceed

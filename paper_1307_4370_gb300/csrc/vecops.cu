@@ -306,7 +306,14 @@ __global__ void k_reweight(int64_t n, const float2* __restrict__ alpha, float* _
 __global__ void k_gather(int64_t n, const float2* __restrict__ src, const int* __restrict__ perm,
                          float2* __restrict__ dst) {
   pdl_sync(src, perm, dst);
-  GRID_STRIDE(i, n) dst[i] = src[perm[i]];
+  const int64_t j0 = (int64_t)blockIdx.x * kPerBlock + threadIdx.x;
+  float2 v[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    if (j0 + q * 256 < n) v[q] = src[perm[j0 + q * 256]];
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    if (j0 + q * 256 < n) dst[j0 + q * 256] = v[q];
 }
 
 // bf16 storage of y: one CTA per block of 4096 visibilities, scale = max |component|.
@@ -405,7 +412,7 @@ int launch_reweight(purify_ctx* c, int64_t count, const float2* alpha, float* w,
 }
 
 int launch_gather_perm(int64_t M, const float2* src, const int* perm, float2* dst, cudaStream_t s) {
-  PURIFY_LAUNCH(nullptr, "gather", s, (pdl_launch(k_gather, LaunchCfg{blocks_for(M), 256, 0, s}, M, src, perm, dst)));
+  PURIFY_LAUNCH(nullptr, "gather", s, (pdl_launch(k_gather, LaunchCfg{blocks_once(M), 256, 0, s}, M, src, perm, dst)));
   return check_cuda(cudaGetLastError());
 }
 
