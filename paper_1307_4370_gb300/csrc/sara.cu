@@ -343,6 +343,215 @@ __global__ void __launch_bounds__(256) k_dwt_level(const float2* __restrict__ in
   }
 }
 
+// ---------------------------------------------------------------------------
+// The coarse levels of small planes in one launch per direction: once a
+// level's side is at most kTailAnalysis (kTailSynthesis), one CTA per plane
+// runs all the levels that remain, the plane's low-low band in shared memory
+// between them.  A level of 8 to 64 pixels a side is bound by its launch and a
+// CTA's dependent loads (4 to 6 us), not by arithmetic: at 64^2 four analysis
+// levels with the prox 26 -> 13 us and three synthesis levels 17 -> 8 us (the
+// iteration 188 -> 176 us, 128^2, M = 20000, 214 -> 209 us).  The sides are
+// where it stops paying: three levels from 96 take 13 us so and 12 us in three
+// launches (analysis), 23 and 13 us (synthesis); two from 64 the same.
+// The filters wrap (also when longer than the signal), so the analysis extends
+// each row, then each column, periodically by the filter's length before it
+// filters; the synthesis reads its few wrapped coefficients by index.
+// ---------------------------------------------------------------------------
+constexpr int kTailAnalysis = 64, kTailSynthesis = 48;
+constexpr int kTailThreads = 512;
+constexpr int kTailExt = 14;  // 2 p - 2 for p = 8
+
+struct TailGeom {
+  int n, L, levels;  // image side; side of the tail's first (analysis) or last (synthesis) level; levels in it
+  int nb, plane0;
+  float scale;
+  int dirac;   // analysis from level 0: plane of the Dirac basis, handled by CTA nb, or -1
+  int f1_off;  // analysis, prox mode
+};
+
+template <int P, int MODE>
+__device__ __forceinline__ float dwt_tail_plane(const float2* __restrict__ src, int src_stride, float2* __restrict__ pl,
+                                                const TailGeom& G, const WaveletTaps& wf, float2* z1, float2* u1,
+                                                const float* w, float gamma) {
+  extern __shared__ float2 sm[];
+  constexpr int taps = 2 * P;
+  const float2 *h = wf.h + P * (P - 1), *g = wf.g + P * (P - 1);
+  const int ST = (G.L + kTailExt) | 1;  // row stride (odd)
+  float2 *A = sm, *B = sm + (G.L + kTailExt) * ST;
+  float f1 = 0.f;
+  int L = G.L;
+  Div dL = make_div(L);
+  for (int e = threadIdx.x; e < L * L; e += kTailThreads) {
+    const int r = udiv(e, dL), c = e - r * L;
+    A[r * ST + c] = src[r * src_stride + c];
+  }
+  __syncthreads();
+  for (int lev = 0; lev < G.levels; ++lev, L /= 2) {
+    const int H = L / 2;
+    const bool last = lev == G.levels - 1;
+    dL = make_div(L);
+    // rows, extended by taps - 2 (an extension longer than the signal repeats it)
+    for (int e = threadIdx.x; e < L * (taps - 2); e += kTailThreads) {
+      const int c = udiv(e, dL), r = e - c * L;
+      A[r * ST + L + c] = A[r * ST + c - udiv(c, dL) * L];
+    }
+    __syncthreads();
+    const int bq = H % 4 == 0 ? 4 : 1;
+    for (int e = threadIdx.x; e < L * (H / bq); e += kTailThreads) {  // lanes take consecutive rows
+      const int q = udiv(e, dL), r = e - q * L;
+      const float2* sp = A + r * ST + 2 * bq * q;
+      float2 a[4], d[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) a[j] = d[j] = make_float2(0.f, 0.f);
+      if (bq == 4) {
+#pragma unroll
+        for (int m = 0; m < taps + 6; ++m) {
+          const float2 v = sp[m];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            if (m - 2 * j >= 0 && m - 2 * j < taps) {
+              a[j] = __ffma2_rn(h[m - 2 * j], v, a[j]);
+              d[j] = __ffma2_rn(g[m - 2 * j], v, d[j]);
+            }
+          }
+        }
+      } else {
+#pragma unroll
+        for (int m = 0; m < taps; ++m) {
+          const float2 v = sp[m];
+          a[0] = __ffma2_rn(h[m], v, a[0]);
+          d[0] = __ffma2_rn(g[m], v, d[0]);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (j >= bq) continue;
+        B[r * ST + bq * q + j] = a[j];
+        B[r * ST + H + bq * q + j] = d[j];
+      }
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < L * (taps - 2); e += kTailThreads) {
+      const int r = udiv(e, dL), c = e - r * L;
+      B[(L + r) * ST + c] = B[(r - udiv(r, dL) * L) * ST + c];
+    }
+    __syncthreads();
+    // columns: low-low to A (or the plane, on the last level), the rest to the
+    // plane; the prox operands of an output are loaded before its filter loop
+    struct Operands {
+      float2 zl, zh;
+      float wl, wh;
+    };
+    const int Hn = H * G.n;
+    auto operands = [&](int i1, int kc) {
+      Operands p{};
+      if (MODE == kSaraProx) {
+        const int o = i1 * G.n + kc;
+        if (kc >= H || last) {
+          p.zl = z1[o];
+          p.wl = w ? w[o] : 1.0f;
+        }
+        p.zh = z1[o + Hn];
+        p.wh = w ? w[o + Hn] : 1.0f;
+      }
+      return p;
+    };
+    auto emit = [&](int i1, int kc, float2 lo, float2 hi, const Operands& p) {
+      const int o = i1 * G.n + kc;  // Mallat position: columns [0, H) of a, [H, L) of d
+      const bool ll = kc < H && !last;
+      if (ll) A[i1 * ST + kc] = lo;
+      const float2 ls = cscale(lo, G.scale), hs = cscale(hi, G.scale);
+      if (MODE == kSaraPlain) {
+        if (!ll) pl[o] = ls;
+        pl[o + Hn] = hs;
+      } else {
+        if (!ll) f1 += sara_prox_v(ls, p.zl, p.wl, o, z1, u1, gamma);
+        f1 += sara_prox_v(hs, p.zh, p.wh, o + Hn, z1, u1, gamma);
+      }
+    };
+    if (H % 2 == 0) {
+      for (int e = threadIdx.x; e < L * (H / 2); e += kTailThreads) {
+        const int j = udiv(e, dL), kc = e - j * L;
+        const float2* cp = B + 4 * j * ST + kc;
+        const Operands p0 = operands(2 * j, kc), p1 = operands(2 * j + 1, kc);
+        float2 lo[2], hi[2];
+        lo[0] = lo[1] = hi[0] = hi[1] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int m = 0; m < taps + 2; ++m) {
+          const float2 v = cp[m * ST];
+          if (m < taps) {
+            lo[0] = __ffma2_rn(h[m], v, lo[0]);
+            hi[0] = __ffma2_rn(g[m], v, hi[0]);
+          }
+          if (m >= 2) {
+            lo[1] = __ffma2_rn(h[m - 2], v, lo[1]);
+            hi[1] = __ffma2_rn(g[m - 2], v, hi[1]);
+          }
+        }
+        emit(2 * j, kc, lo[0], hi[0], p0);
+        emit(2 * j + 1, kc, lo[1], hi[1], p1);
+      }
+    } else {
+      for (int e = threadIdx.x; e < L * H; e += kTailThreads) {
+        const int i1 = udiv(e, dL), kc = e - i1 * L;
+        const float2* cp = B + 2 * i1 * ST + kc;
+        const Operands p0 = operands(i1, kc);
+        float2 lo = make_float2(0.f, 0.f), hi = lo;
+#pragma unroll
+        for (int m = 0; m < taps; ++m) {
+          const float2 v = cp[m * ST];
+          lo = __ffma2_rn(h[m], v, lo);
+          hi = __ffma2_rn(g[m], v, hi);
+        }
+        emit(i1, kc, lo, hi, p0);
+      }
+    }
+    __syncthreads();
+  }
+  return f1;
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(kTailThreads) k_dwt_tail(const float2* __restrict__ in, int in_shared,
+                                                           float2* __restrict__ coef, TailGeom G, BasisList bl,
+                                                           const __grid_constant__ WaveletTaps wf, SaraProxArgs pa,
+                                                           double* partials, DevScalars* sc) {
+  pdl_sync(in, coef, partials, sc);
+  const int k = blockIdx.x;
+  const float gamma = (MODE == kSaraProx) ? (float)sc->gamma : 0.f;
+  float f1 = 0.f;
+  if (k == G.nb) {  // the Dirac plane
+    const size_t base = (size_t)G.dirac * G.n * G.n;
+    for (int e = threadIdx.x; e < G.n * G.n; e += kTailThreads) {
+      const float2 al = cscale(in[e], G.scale);
+      if (MODE == kSaraPlain) coef[base + e] = al;
+      else f1 += sara_prox(al, base + e, pa, gamma);
+    }
+  } else {
+    const size_t base = (size_t)(G.plane0 + k) * G.n * G.n;
+    const float2* src = in_shared ? in : in + (size_t)k * (G.n / 2) * (G.n / 2);
+    float2 *z1 = MODE == kSaraProx ? pa.z1 + base : nullptr, *u1 = MODE == kSaraProx ? pa.u1 + base : nullptr;
+    const float* w = MODE == kSaraProx && pa.w ? pa.w + base : nullptr;
+    float2* pl = coef + base;
+    switch (bl.p(k)) {
+      case 1: f1 = dwt_tail_plane<1, MODE>(src, G.L, pl, G, wf, z1, u1, w, gamma); break;
+      case 2: f1 = dwt_tail_plane<2, MODE>(src, G.L, pl, G, wf, z1, u1, w, gamma); break;
+      case 3: f1 = dwt_tail_plane<3, MODE>(src, G.L, pl, G, wf, z1, u1, w, gamma); break;
+      case 4: f1 = dwt_tail_plane<4, MODE>(src, G.L, pl, G, wf, z1, u1, w, gamma); break;
+      case 5: f1 = dwt_tail_plane<5, MODE>(src, G.L, pl, G, wf, z1, u1, w, gamma); break;
+      case 6: f1 = dwt_tail_plane<6, MODE>(src, G.L, pl, G, wf, z1, u1, w, gamma); break;
+      case 7: f1 = dwt_tail_plane<7, MODE>(src, G.L, pl, G, wf, z1, u1, w, gamma); break;
+      default: f1 = dwt_tail_plane<8, MODE>(src, G.L, pl, G, wf, z1, u1, w, gamma); break;
+    }
+  }
+  if (MODE == kSaraProx) {
+    const FPair f1p{f1, 0.f};
+    double f1d;
+    block_reduce<1>(&f1p, &f1d);
+    if (threadIdx.x == 0) partials[kCntF1 * 2 * kMaxPartials + G.f1_off + blockIdx.x] = f1d;
+  }
+}
+
 // f1 of §4.4 as the sum of the analysis levels' block partials (in index
 // order), and the halting quantity zeta = |f1 - f1_prev| / f1_prev.
 __device__ __forceinline__ void sara_f1_finish(const double* __restrict__ part, int n, DevScalars* sc) {
@@ -629,6 +838,93 @@ __global__ void __launch_bounds__(256, 3) k_idwt_level(const float2* __restrict_
   }
 }
 
+// The synthesis of the coarse levels, one CTA per plane (see k_dwt_tail): from
+// the coarsest level up to the one whose output side is G.L, written to
+// ll_out.  With f1 partials to sum, CTA nb forms f1 and zeta.
+template <int P>
+__device__ __forceinline__ void idwt_tail_plane(const float2* __restrict__ pl, float2* __restrict__ out,
+                                                const TailGeom& G, const WaveletTaps& wf) {
+  extern __shared__ float2 sm[];
+  const float2 *h = wf.h + P * (P - 1), *g = wf.g + P * (P - 1);
+  const int ST = G.L | 1;
+  float2 *A = sm, *B = sm + G.L * ST;
+  int L = G.L >> (G.levels - 1);
+  for (int lev = 0; lev < G.levels; ++lev, L *= 2) {
+    const int H = L / 2;
+    const Div dL = make_div(L), dH = make_div(H);
+    // A: [LL LH; HL HH]; LL of the levels after the first is there already
+    for (int e = threadIdx.x; e < L * L; e += kTailThreads) {
+      const int r = udiv(e, dL), c = e - r * L;
+      if (lev == 0 || r >= H || c >= H) A[r * ST + c] = pl[r * G.n + c];
+    }
+    __syncthreads();
+    auto wrapped = [&](int i) {  // i in (-P, H)
+      if (H >= P) return i < 0 ? i + H : i;
+      i += 8 * H;
+      return i - udiv(i, dH) * H;
+    };
+    // columns, then rows: outputs 2 i and 2 i + 1 from coefficients i - u
+    for (int e = threadIdx.x; e < H * L; e += kTailThreads) {
+      const int i = udiv(e, dL), c = e - i * L;
+      float2 s0 = make_float2(0.f, 0.f), s1 = s0;
+#pragma unroll
+      for (int u = 0; u < P; ++u) {
+        const int t = wrapped(i - u);
+        const float2 lo = A[t * ST + c], hi = A[(H + t) * ST + c];
+        s0 = __ffma2_rn(h[2 * u], lo, __ffma2_rn(g[2 * u], hi, s0));
+        s1 = __ffma2_rn(h[2 * u + 1], lo, __ffma2_rn(g[2 * u + 1], hi, s1));
+      }
+      B[2 * i * ST + c] = s0;
+      B[(2 * i + 1) * ST + c] = s1;
+    }
+    __syncthreads();
+    const bool last = lev == G.levels - 1;
+    for (int e = threadIdx.x; e < H * L; e += kTailThreads) {
+      const int j = udiv(e, dL), r = e - j * L;
+      float2 s0 = make_float2(0.f, 0.f), s1 = s0;
+#pragma unroll
+      for (int u = 0; u < P; ++u) {
+        const int t = wrapped(j - u);
+        const float2 av = B[r * ST + t], dv = B[r * ST + H + t];
+        s0 = __ffma2_rn(h[2 * u], av, __ffma2_rn(g[2 * u], dv, s0));
+        s1 = __ffma2_rn(h[2 * u + 1], av, __ffma2_rn(g[2 * u + 1], dv, s1));
+      }
+      if (last) {
+        out[r * L + 2 * j] = s0;
+        out[r * L + 2 * j + 1] = s1;
+      } else {
+        A[r * ST + 2 * j] = s0;
+        A[r * ST + 2 * j + 1] = s1;
+      }
+    }
+    __syncthreads();
+  }
+}
+
+__global__ void __launch_bounds__(kTailThreads) k_idwt_tail(const float2* __restrict__ coef,
+                                                            float2* __restrict__ ll_out, TailGeom G, BasisList bl,
+                                                            const __grid_constant__ WaveletTaps wf,
+                                                            const double* f1_part, int f1_n, DevScalars* sc) {
+  pdl_sync(coef, ll_out, f1_part, sc);
+  const int k = blockIdx.x;
+  if (k == G.nb) {
+    sara_f1_finish(f1_part, f1_n, sc);
+    return;
+  }
+  const float2* pl = coef + (size_t)(G.plane0 + k) * G.n * G.n;
+  float2* out = ll_out + (size_t)k * (G.n / 2) * (G.n / 2);
+  switch (bl.p(k)) {
+    case 1: idwt_tail_plane<1>(pl, out, G, wf); break;
+    case 2: idwt_tail_plane<2>(pl, out, G, wf); break;
+    case 3: idwt_tail_plane<3>(pl, out, G, wf); break;
+    case 4: idwt_tail_plane<4>(pl, out, G, wf); break;
+    case 5: idwt_tail_plane<5>(pl, out, G, wf); break;
+    case 6: idwt_tail_plane<6>(pl, out, G, wf); break;
+    case 7: idwt_tail_plane<7>(pl, out, G, wf); break;
+    default: idwt_tail_plane<8>(pl, out, G, wf); break;
+  }
+}
+
 __global__ void __launch_bounds__(256) k_f1_finish(const double* __restrict__ part, int n, DevScalars* sc) {
   pdl_sync(part, sc);
   sara_f1_finish(part, n, sc);
@@ -736,6 +1032,24 @@ int sara_analysis(purify_ctx* c, const float2* x, float2* alpha, SaraMode mode, 
   for (int lev = 0; lev < c->levels; ++lev) {
     const int L = c->n >> lev;
     const int H = L / 2;
+    if (L <= kTailAnalysis && lev < c->levels - 1) {  // the levels that remain in one launch
+      TailGeom G{c->n, L, c->levels - lev, nb, plane0, scale, lev == 0 ? dirac_plane : -1, f1_off};
+      const float2* in = (lev == 0) ? x : c->d_ll[(lev - 1) & 1];
+      const int ctas = nb + (G.dirac >= 0 ? 1 : 0);
+      const size_t sm = (size_t)2 * (L + kTailExt) * ((L + kTailExt) | 1) * sizeof(float2);
+      const LaunchCfg lc{ctas, kTailThreads, sm, s, lev > 0};
+      f1_off += ctas;
+      if (mode == kSaraPlain) {
+        allow_smem(k_dwt_tail<kSaraPlain>, sm);
+        PURIFY_LAUNCH(c, "dwt_level", s,
+                      (pdl_launch(k_dwt_tail<kSaraPlain>, lc, in, lev == 0, alpha, G, bl, taps, pa, c->d_partials, c->d_sc)));
+      } else {
+        allow_smem(k_dwt_tail<kSaraProx>, sm);
+        PURIFY_LAUNCH(c, "dwt_level", s,
+                      (pdl_launch(k_dwt_tail<kSaraProx>, lc, in, lev == 0, pa.z1, G, bl, taps, pa, c->d_partials, c->d_sc)));
+      }
+      break;
+    }
     const int TI = tile_for(H, nb + (lev == 0 && dirac_plane >= 0 ? 1 : 0), c->sms);
     LevelGeom G{TI, c->n, L, nb, plane0, lev == c->levels - 1, scale, lev == 0, lev == 0 ? dirac_plane : -1, f1_off};
     const float2* in = (lev == 0) ? x : c->d_ll[(lev - 1) & 1];
@@ -783,7 +1097,22 @@ int sara_synthesis(purify_ctx* c, const float2* alpha, float2* x, cudaStream_t s
   int maxp = 1;
   for (int k = 0; k < nb; ++k) maxp = std::max(maxp, bl.p(k));
   const WaveletTaps taps = wavelet_taps(c->wf);
-  for (int lev = c->levels - 1; lev >= 0; --lev) {
+  // the coarse levels (never the finest, which sums the planes) in one launch
+  int top = c->levels - 1;  // coarsest level left to the per-level launches
+  for (int lev = 1; lev < c->levels; ++lev) {
+    const int L = c->n >> lev;
+    if (L > kTailSynthesis || lev == c->levels - 1) continue;
+    TailGeom G{c->n, L, c->levels - lev, nb, plane0, scale, -1, 0};
+    const size_t sm = (size_t)2 * L * (L | 1) * sizeof(float2);
+    allow_smem(k_idwt_tail, sm);
+    PURIFY_LAUNCH(c, "idwt_level", s,
+                  (pdl_launch(k_idwt_tail, LaunchCfg{nb + (f1_parts > 0 ? 1 : 0), kTailThreads, sm, s}, alpha,
+                              c->d_ll[lev & 1], G, bl, taps, c->d_partials + kCntF1 * 2 * kMaxPartials, f1_parts,
+                              c->d_sc)));
+    top = lev - 1;
+    break;
+  }
+  for (int lev = top; lev >= 0; --lev) {
     const int L = c->n >> lev;  // output side
     const int H = L / 2;
     const int TO = tile_for(H, lev == 0 ? 1 : nb, c->sms);
