@@ -130,7 +130,7 @@ typedef struct {
  * Set-up sorts the visibilities by grid tile and builds the tile lists of
  * the gridding adjoint and its stored gather walk (one 32-bit item per
  * visibility and 2 x 2 cell block its footprint meets, about 12 per
- * visibility for J = 6, so ~50 bytes of device memory per visibility besides
+ * visibility for J = 6, so ~60 bytes of device memory per visibility besides
  * the grids and tables).  For the grid tiles whose lists are dense it also
  * computes G^T G restricted to them (§5: G^H G precomputed for the CG
  * solve), on the host in double with a pool of threads, and keeps it on the

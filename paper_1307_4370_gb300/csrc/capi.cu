@@ -4,6 +4,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <numeric>
 #include <string>
 #include <new>
@@ -385,6 +386,19 @@ constexpr size_t kDenseL2Bytes = (size_t)32 << 20;
 // Visibilities from which purify_phi_adj sorts its input first.
 constexpr int64_t kPermFirst = (int64_t)1 << 20;
 
+// Host floats that their writers touch first (32 MB of stencils and more; a
+// vector would have one thread fill them with zeros before).
+struct HostFloats {
+  std::unique_ptr<float[]> p;
+  size_t n = 0;
+  void resize(size_t count) {
+    p.reset(new float[count]);
+    n = count;
+  }
+  float* data() { return p.get(); }
+  size_t size() const { return n; }
+};
+
 // Threads that build the stencils.
 unsigned pool_threads(const purify::GatherPlan& plan, const std::vector<int>& dense, int J) {
   double work = 0;  // multiply-adds: J^4 per list entry; a thread starts in the time of a few 10^5
@@ -402,10 +416,10 @@ unsigned pool_threads(const purify::GatherPlan& plan, const std::vector<int>& de
 // so (G^T G X)(k) = sum_d H[t][d][k] X(k + d) exactly.  Built in double on
 // the host, one tile per thread of a small pool, and stored as float.
 int build_dense_gram(const purify_ctx* c, const purify::GatherPlan& plan, const std::vector<int4>& entries,
-                      const std::vector<int>& dense, std::vector<float>& H) {
+                      const std::vector<int>& dense, HostFloats& H) {
   const int T = c->tileT, J = c->J, W = T + J - 1, ND = (2 * J - 1) * (2 * J - 1), TT = T * T;
   const TapSeries taps = fit_taps(J, c->kernel);
-  H.assign((size_t)dense.size() * ND * TT, 0.0f);
+  H.resize((size_t)dense.size() * ND * TT);
   std::atomic<size_t> next{0};
   std::atomic<bool> failed{false};
   auto work = [&]() {
@@ -470,11 +484,11 @@ int build_dense_gram(const purify_ctx* c, const purify::GatherPlan& plan, const 
 // dr = 0, dc = 0 .. J - 1; then s = J + (dr - 1)(2J - 1) + dc + J - 1 for
 // dr = 1 .. J - 1, dc = -(J - 1) .. J - 1.
 int build_dense_gram_half(const purify_ctx* c, const purify::GatherPlan& plan, const std::vector<int4>& entries,
-                           const std::vector<int>& dense, std::vector<float>& H) {
+                           const std::vector<int>& dense, HostFloats& H) {
   const int T = c->tileT, J = c->J, W = T + J - 1, NDW = 2 * J - 1;
   const int NH = dense_gram_slices(J), EW = T + 2 * (J - 1), EH = T + J - 1, ES = EW * EH;
   const TapSeries taps = fit_taps(J, c->kernel);
-  H.assign((size_t)dense.size() * NH * ES, 0.0f);
+  H.resize((size_t)dense.size() * NH * ES);
   std::atomic<size_t> next{0};
   std::atomic<bool> failed{false};
   auto work = [&]() {
@@ -661,7 +675,7 @@ int setup_visibilities(purify_ctx* c, const float* uv_in, cudaStream_t s) {
       if (!is_dense[plan.chunks[q].x]) gram_chunks.push_back(q);
     c->n_dense = (int)dense.size();
     c->n_gram_chunks = (int)gram_chunks.size();
-    std::vector<float> H;
+    HostFloats H;
     if (c->n_dense > 0) {
       std::vector<int4> entries(c->nlist);
       if (cudaMemcpy(entries.data(), c->d_list, c->nlist * sizeof(int4), cudaMemcpyDeviceToHost) != cudaSuccess)

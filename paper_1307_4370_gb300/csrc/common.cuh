@@ -338,7 +338,7 @@ struct purify_ctx {
   float* d_deapod;      // n: 1 / g_hat((r - n/2) / 2n)
   float2* d_tw;         // L: exp(-2 pi i m / L)
   int fft_engine;       // 1: compile-time engine (fft_fixed_side), 0: generic Stockham
-  float2* d_twp[2];     // per-stage twiddle tables of that engine (8 or 12, 16 or 24 per thread)
+  float2* d_twp[2];     // per-stage twiddle tables of that engine (8 or 12, 16 per thread)
 
   // visibility table (sorted by grid tile of the first footprint cell)
   float2* d_uv;         // M frequencies in the degridding's order
@@ -551,9 +551,10 @@ int fft_prepare(purify_ctx* c);  // its tables (at context creation)
 int phi_forward_grid(purify_ctx* c, RowInMode mode, const RowInArgs& a, cudaStream_t s, int cg_j = 0);
 int cg_partial_blocks(const purify_ctx* c);
 // CG step sizes formed by the consuming kernels (few partials) or by a
-// one-block kernel after the inverse row pass (many partials: at 256
-// partials, e.g. 1024^2, every block of the 1024-block forward row pass
-// summing them cost 9 us per CG step against ~2 us for the extra launch).
+// one-block kernel after the inverse row pass.  Measured: 192 partials and 192
+// consumers (384^2) 513 -> 495 us an iteration without the extra kernel; 256
+// and 1024 (1024^2) row_fwd +4.6 us against 6 us for the kernel, no difference
+// in the iteration, so the line lies between.
 constexpr int kCgConsumeMaxBlocks = 192;
 int cg_consumer_blocks(const purify_ctx* c);  // nblk for the consumers: the partial count, or 0
 int launch_cg_scalars(purify_ctx* c, int cg_j, cudaStream_t s);

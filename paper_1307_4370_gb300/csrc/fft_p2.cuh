@@ -9,8 +9,8 @@
 // (j / Ns) Ns R + k; natural-order output), specialised so that
 //  * every index split is by a constant, every loop is unrolled;
 //  * each thread runs E / R butterflies of a stage, E = elements per thread
-//    (8 or 16; 12 or 24 where 3 divides L, whose first radix, 12 or 24, takes
-//    the factor 3 by a prime-factor map, without inner twiddles);
+//    (8 or 16; 12 where 3 divides L, whose first radix takes the factor 3 by a
+//    prime-factor map, without inner twiddles);
 //  * shared memory is padded by one complex value per 16, so the strided
 //    writes of the first stages and the strided reads of the column layout
 //    fall in distinct banks;
@@ -66,52 +66,41 @@ __device__ __forceinline__ void dft_small<16>(float2* v) {
   }
 }
 
-// 3 Q-point DFT (Q = 4 or 8, coprime to 3): with j = (Q j1 + 3 j2) mod 3 Q and
-// k = (A k1 + 9 k2) mod 3 Q, A = 4 (Q = 4) or 16 (Q = 8) (A = 1 mod 3, 0 mod Q;
-// 9 = 0 mod 3, 1 mod Q), the transform is a Q-point DFT along j2 and a 3-point
-// one along j1 with no twiddles between (Good-Thomas prime-factor map).
-template <int Q>
-__device__ __forceinline__ void dft_3q(float2* v) {
-  constexpr int N = 3 * Q, A = Q == 4 ? 4 : 16;
-  float2 a[3][Q];
+// 12-point DFT: with j = (4 j1 + 3 j2) mod 12 and k = (4 k1 + 9 k2) mod 12
+// (4 = 1 mod 3, 0 mod 4; 9 = 0 mod 3, 1 mod 4) the transform is a 4-point DFT
+// along j2 and a 3-point one along j1 with no twiddles between (Good-Thomas
+// prime-factor map).
+template <>
+__device__ __forceinline__ void dft_small<12>(float2* v) {
+  float2 a[3][4];
 #pragma unroll
   for (int j1 = 0; j1 < 3; ++j1) {
 #pragma unroll
-    for (int j2 = 0; j2 < Q; ++j2) a[j1][j2] = v[(Q * j1 + 3 * j2) % N];
-    dft_small<Q>(a[j1]);
+    for (int j2 = 0; j2 < 4; ++j2) a[j1][j2] = v[(4 * j1 + 3 * j2) % 12];
+    dft_small<4>(a[j1]);
   }
 #pragma unroll
-  for (int k2 = 0; k2 < Q; ++k2) {
+  for (int k2 = 0; k2 < 4; ++k2) {
     float2 t[3] = {a[0][k2], a[1][k2], a[2][k2]};
     dft_small<3>(t);
 #pragma unroll
-    for (int k1 = 0; k1 < 3; ++k1) v[(A * k1 + 9 * k2) % N] = t[k1];
+    for (int k1 = 0; k1 < 3; ++k1) v[(4 * k1 + 9 * k2) % 12] = t[k1];
   }
 }
-template <>
-__device__ __forceinline__ void dft_small<12>(float2* v) { dft_3q<4>(v); }
-template <>
-__device__ __forceinline__ void dft_small<24>(float2* v) { dft_3q<8>(v); }
 
 constexpr int p2_min(int a, int b) { return a < b ? a : b; }
 constexpr int p2_max(int a, int b) { return a > b ? a : b; }
-// First radix: E, or for L = 3 2^p and E = 24 the one of 24 and 12 that leaves
-// 8^a or 4 8^a (the pruned last stage needs a radix of at least 4).
-constexpr int p2_first(int L, int E) {
-  if (L % 3 != 0) return p2_min(E, L);
-  if (E == 12) return 12;
-  int rem = L / 24;
-  while (rem >= 8) rem /= 8;
-  return rem == 2 ? 12 : 24;
-}
-// Radix of stage st: after the first, E (8 or 4 of 24 or 12) until fewer remain.
+// First radix: E (12 for L = 3 2^p).
+constexpr int p2_first(int L, int E) { return L % 3 != 0 ? p2_min(E, L) : 12; }
+// Radix of stage st: after the first, E (4 of 12) until fewer remain.
 constexpr int p2_radix(int L, int E, int st) {
   const int cap = L % 3 != 0 ? E : E / 3;
   int rem = L, r = p2_first(L, E);
   for (int i = 0; i < st; ++i) {
     rem /= r;
-    // (8, 4, 4 at 128: the pruned last stage needs a radix of at least 4)
-    r = rem == 2 * cap && cap == 8 ? 4 : p2_min(cap, rem);
+    // (the pruned last stage needs a radix of at least 4: 8, 4, 4 at 128 points,
+    // 12, 4, 2, 4 at 384)
+    r = rem == 2 * cap && cap <= 8 ? cap / 2 : p2_min(cap, rem);
   }
   return r;
 }

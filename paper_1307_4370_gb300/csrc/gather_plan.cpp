@@ -155,6 +155,8 @@ int build_gather_plan(const int* k0, const GatherPlanParams& prm, GatherPlan& ou
   out.tab.assign((size_t)nchunks * prm.tab_stride, 0);
   out.item_row.assign(nchunks, 0);
   std::vector<int> off(NK + 1);
+  // (about (J + 1)^2 / 4 items per entry; growing the vector copied it over and over)
+  out.items.reserve((size_t)nlist * ((J + 1) * (J + 1) / 4 + 1) + (size_t)nchunks * NT);
   int64_t rows = 0;
   for (int q = 0; q < nchunks; ++q) {
     const PlanI4 ch = out.chunks[q];

@@ -373,7 +373,9 @@ __global__ void __launch_bounds__(256) k_row_inv(const float2* __restrict__ half
 // inverse row pass of the CG leaves one pair of partial sums per CTA, which
 // every CTA of the next pass adds up.  Eight elements per thread up to 512
 // points: a lone warp issues an instruction every six clocks, so shorter
-// threads win there (128 points, CG epilogue: 16 elements 6.4 us, 8 4.5 us).
+// threads win there (128 points, CG epilogue: 16 elements 6.4 us, 8 4.5 us;
+// 3 2^p points: 24 elements 281, 341, 495 and 1105 us an iteration at 96^2,
+// 192^2, 384^2 and 768^2, 12 elements 230, 293, 480 and 1074 us).
 constexpr int p2_rows(int L, int E, int max_threads) {
   const int per = L / E;                        // threads per row
   int ns = p2_max(1, L / 2 / 128);              // about 128 CTAs
@@ -386,7 +388,7 @@ constexpr int p2_rows(int L, int E, int max_threads) {
 template <int L>
 struct P2Cfg {
   static constexpr bool T3 = L % 3 == 0;
-  static constexpr int E = T3 ? 24 : (L >= 1024 ? 16 : 8);  // plain row, column and inverse row passes
+  static constexpr int E = T3 ? 12 : (L >= 1024 ? 16 : 8);  // plain row, column and inverse row passes
   static constexpr int E_CG = T3 ? 12 : 8;                              // forward row pass with the CG update
   static constexpr int NS_ROW = p2_rows(L, E, 256);
   static constexpr int NS_ROWCG = p2_rows(L, E_CG, 256);
@@ -501,7 +503,7 @@ bool fft_fixed_side(int L) {
 // Concatenated twiddle tables of the engine for (L, E) (device, owned by the context).
 template <int L, int E>
 static int p2_table(purify_ctx* c, const float2** out) {
-  const int idx = (E == 16 || E == 24) ? 1 : 0;
+  const int idx = E == 16 ? 1 : 0;
   if (!c->d_twp[idx]) {
     std::vector<float2> t(std::max(1, p2_twsize(L, E)));
     p2_twiddles<L, E>(t.data());
