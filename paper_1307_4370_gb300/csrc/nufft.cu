@@ -526,7 +526,7 @@ static int p2_prepare_L(purify_ctx* c) {
   return p2_table<L, P2Cfg<L>::E_CG>(c, &t);
 }
 
-// Twiddle tables of the power-of-two engine, built when the context is
+// Twiddle tables of the compile-time engine, built when the context is
 // created (never inside a stream capture).
 int fft_prepare(purify_ctx* c) {
   if (c->fft_engine != 1) return PURIFY_OK;
