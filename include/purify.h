@@ -109,8 +109,8 @@ typedef enum {
  *   tile        side of the grid tiles that organise G and G^T (a schedule
  *               choice, not part of the method): 0 picks a default from the
  *               grid size; otherwise 8, 16, 32 or 64, at least J and dividing
- *               2n.  The autotuner of the Python package measures the
- *               candidates.
+ *               2n (2n itself: one tile).  The autotuner of the Python
+ *               package measures the candidates.
  *   kernel      a purify_kernel (0, the zero-initialised default, is
  *               Kaiser-Bessel).  */
 typedef struct {

@@ -13,7 +13,7 @@ int build_gather_plan(const int* k0, const GatherPlanParams& prm, GatherPlan& ou
       prm.entry_bytes == 0 || prm.tab_stride < (T / 2) * (T / 2) + 1 || prm.max_partials < 2)
     return -1;
   const int HT = prm.home_T > 0 ? prm.home_T : T;
-  if ((HT & (HT - 1)) != 0 || HT < 2 || L % HT != 0) return -1;
+  if ((HT & (HT - 1)) != 0 || HT < T || L % HT != 0) return -1;
   const int TD = L / T, ntiles = TD * TD, HD = L / HT, nhome = HD * HD;
   out = GatherPlan{};
   out.ntiles = ntiles;
@@ -34,22 +34,36 @@ int build_gather_plan(const int* k0, const GatherPlanParams& prm, GatherPlan& ou
     for (int64_t i = 0; i < M; ++i) out.perm[pos[(kr_of(i) / HT) * HD + kc_of(i) / HT]++] = (int)i;
   }
 
-  // per-tile lists of sorted indices whose footprint meets the tile
-  auto tiles_of = [&](int64_t si, int* tl) {
+  // Per-tile lists of sorted indices whose footprint meets the tile, each entry
+  // with the key of the footprint's first cell relative to the tile.  Per axis
+  // a footprint is at most two parts: one in the tile it starts in and, past
+  // that tile's end, one in the next (the first one again where the grid is a
+  // single tile) starting at a negative offset.
+  const int W = T + J - 1;
+  auto parts_of = [&](int64_t si, int* tl, int* key) {
     const int64_t i = out.perm[si];
-    const int r0 = kr_of(i) / T, r1 = ((kr_of(i) + J - 1) % L) / T;
-    const int c0 = kc_of(i) / T, c1 = ((kc_of(i) + J - 1) % L) / T;
-    int nt = 0;
-    const int rs[2] = {r0, r1}, cs[2] = {c0, c1};
-    for (int a = 0; a < (r1 != r0 ? 2 : 1); ++a)
-      for (int b = 0; b < (c1 != c0 ? 2 : 1); ++b) tl[nt++] = rs[a] * TD + cs[b];
-    return nt;
+    const int k[2] = {kr_of(i), kc_of(i)};
+    int at[2][2], start[2][2], np[2];
+    for (int x = 0; x < 2; ++x) {
+      at[x][0] = k[x] / T;
+      start[x][0] = k[x] - at[x][0] * T;
+      at[x][1] = (at[x][0] + 1) % TD;
+      start[x][1] = start[x][0] - T;
+      np[x] = start[x][0] + J > T ? 2 : 1;
+    }
+    int n = 0;
+    for (int a = 0; a < np[0]; ++a)
+      for (int b = 0; b < np[1]; ++b) {
+        tl[n] = at[0][a] * TD + at[1][b];
+        key[n++] = (start[0][a] + J - 1) * W + start[1][b] + J - 1;
+      }
+    return n;
   };
   // (list positions are 32-bit on the device: at most 2^31 - 1 entries)
   std::vector<int64_t> lcnt64(ntiles + 1, 0);
-  int tl[4];
+  int tl[4], key[4];
   for (int64_t si = 0; si < M; ++si) {
-    const int nt = tiles_of(si, tl);
+    const int nt = parts_of(si, tl, key);
     for (int k = 0; k < nt; ++k) lcnt64[tl[k] + 1]++;
   }
   for (int t = 0; t < ntiles; ++t) lcnt64[t + 1] += lcnt64[t];
@@ -62,33 +76,27 @@ int build_gather_plan(const int* k0, const GatherPlanParams& prm, GatherPlan& ou
   {
     std::vector<int> pos(lcnt.begin(), lcnt.end() - 1);
     for (int64_t si = 0; si < M; ++si) {
-      const int nt = tiles_of(si, tl);
-      for (int k = 0; k < nt; ++k) out.list[pos[tl[k]]++] = (int)si;
+      const int nt = parts_of(si, tl, key);
+      for (int k = 0; k < nt; ++k) {
+        const int e = pos[tl[k]]++;
+        out.list[e] = (int)si;
+        out.lkey[e] = key[k];
+      }
     }
   }
-  // order each tile's list by the footprint start cell relative to the tile:
-  // the visibilities starting at a given cell form one run
-  const int W = T + J - 1;
-  auto rel = [&](int k, int origin) {  // start offset in [-(J-1), L - J + 1)
-    int t = (k - origin) % L;
-    if (t < 0) t += L;
-    return t >= L - (J - 1) ? t - L : t;
-  };
+  // order each tile's list by that key: the visibilities starting at a given
+  // cell form one run (counting sort, stable; a comparison sort was a tenth of
+  // the set-up at M = 2^21)
   {
-    // (counting sort by key, stable; a comparison sort was a tenth of the set-up
-    // at M = 2^21)
     std::vector<std::pair<int, int>> seg;
     std::vector<int> at(W * W + 1);
     for (int t = 0; t < ntiles; ++t) {
       if (lcnt[t] == lcnt[t + 1]) continue;
-      const int R0 = (t / TD) * T, C0 = (t % TD) * T;
       seg.clear();
       std::fill(at.begin(), at.end(), 0);
       for (int e = lcnt[t]; e < lcnt[t + 1]; ++e) {
-        const int64_t i = out.perm[out.list[e]];
-        const int key = (rel(kr_of(i), R0) + J - 1) * W + (rel(kc_of(i), C0) + J - 1);
-        seg.emplace_back(key, out.list[e]);
-        ++at[key + 1];
+        seg.emplace_back(out.lkey[e], out.list[e]);
+        ++at[out.lkey[e] + 1];
       }
       for (int k = 0; k < W * W; ++k) at[k + 1] += at[k];
       for (const auto& v : seg) {
@@ -99,24 +107,18 @@ int build_gather_plan(const int* k0, const GatherPlanParams& prm, GatherPlan& ou
     }
   }
 
-  // the degridding's order: the visibilities that start in a gridding tile (key
-  // row and column at least J - 1) are in its list by start cell; the gridding
-  // tiles of a home tile one after the other
+  // the degridding's order: a visibility has one part that starts in the tile
+  // (key row and column at least J - 1), in its first cell's tile; the parts of
+  // that kind by start cell, the gridding tiles of a home tile one after the other
   out.dorder.resize(M);
   {
-    const int sub = HT / T > 0 ? HT / T : 1;
+    const int sub = HT / T;
     std::vector<int> pos(cnt.begin(), cnt.end() - 1);
     for (int t = 0; t < ntiles; ++t) {
-      const int h = HT >= T ? (t / TD / sub) * HD + (t % TD) / sub : -1;
+      const int h = (t / TD / sub) * HD + (t % TD) / sub;
       for (int e = lcnt[t]; e < lcnt[t + 1]; ++e) {
-        const int k = out.lkey[e], si = out.list[e];
-        if (k / W < J - 1 || k % W < J - 1) continue;
-        int hh = h;
-        if (hh < 0) {  // (home tiles smaller than the gridding's)
-          const int64_t i = out.perm[si];
-          hh = (kr_of(i) / HT) * HD + kc_of(i) / HT;
-        }
-        out.dorder[pos[hh]++] = si;
+        const int k = out.lkey[e];
+        if (k / W >= J - 1 && k % W >= J - 1) out.dorder[pos[h]++] = out.list[e];
       }
     }
   }

@@ -9,7 +9,8 @@
 //     (stable), and per tile the run of its "home" visibilities;
 //   - per tile, the list of sorted indices whose footprint meets the tile,
 //     ordered by the footprint's first cell relative to the tile (key =
-//     (dr + J - 1) * W + (dc + J - 1), W = T + J - 1);
+//     (dr + J - 1) * W + (dc + J - 1), W = T + J - 1); where one tile is the
+//     whole grid, a footprint that wraps has an entry for each of its parts;
 //   - the gridding work units ("chunks": a run of one tile's list), with
 //     per chunk the prefix of the 2 x 2 cell blocks' ("owners'") gather work
 //     and the gather items of each of the kernel's threads (see grid_item);
@@ -47,7 +48,7 @@ struct GatherPlanParams {
   int L;                 // grid side
   int J;                 // footprint side (<= 8)
   int T;                 // tile side (power of two, divides L, <= 64)
-  int home_T = 0;        // tile side of the visibility sort and the degridding units (0: T)
+  int home_T = 0;        // tile side of the visibility sort and the degridding units (at least T; 0: T)
   size_t fixed_bytes;    // shared memory of a gridding CTA without its entries
   size_t entry_bytes;    // shared memory per staged entry
   size_t smem_budget;    // target shared memory of a gridding CTA
