@@ -6,6 +6,8 @@
 // depend on block scheduling, and no extra kernel launch is needed.
 #pragma once
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace purify {
@@ -48,13 +50,34 @@ struct FPair {
 // 16 clocks, and the ten of a warp's shuffle tree over two values, for every
 // warp of a block, cost more than the kernel's own work (degridding with the
 // norms of the l2 branch at 1024^2, M = 2^21: 98 us against 63 us without).
-// So the lanes of a warp are summed as float pairs by error-free TwoSum
-// merges (FP32 unit; the dropped terms are below 2^-47 of one warp's sum,
-// itself a 10^-3..10^-5 part of the total, i.e. at the rounding of an FP64
-// total), and only the sums across warps and blocks are FP64.  A warp that
-// holds a value which could overflow the pair (or is not finite) takes the
-// FP64 tree instead.
+// So the lanes of a warp are summed in FP32 as well, in triples whose three
+// components hold what every addition rounds off (the terms dropped are below
+// 2^-68 of the largest partial sum, so the one rounding to FP64 at the end is
+// the only error that FP64 can show; a pair, 2^-47, would lose bits that an
+// FP64 tree keeps), and only the sums across warps and blocks are FP64.  A
+// warp that holds a value which could overflow the triple (or is not finite)
+// takes the FP64 tree instead.
 constexpr float kPairMax = 1.2676506e30f;  // 2^100: 32 such values stay far below FP32's maximum
+
+// a + b = two_sum + e, exactly (Knuth's TwoSum)
+__device__ __forceinline__ float two_sum(float a, float b, float& e) {
+  const float s = a + b;
+  const float bb = s - a;
+  e = (a - (s - bb)) + (b - bb);
+  return s;
+}
+
+struct FTriple {
+  float a = 0.f, b = 0.f, c = 0.f;
+  __device__ __forceinline__ void add(float ta, float tb, float tc) {
+    float e1, e2, e3;
+    a = two_sum(a, ta, e1);
+    b = two_sum(b, tb, e2);
+    b = two_sum(b, e1, e3);
+    c += tc + (e2 + e3);
+  }
+  __device__ __forceinline__ double value() const { return (double)a + ((double)b + (double)c); }
+};
 
 // Tree over the first `valid` lanes of a warp whose first `present` lanes
 // exist (any block size, including a partial last warp); every present lane
@@ -70,29 +93,69 @@ __device__ __forceinline__ double warp_tree(double v, int lane, int present, int
   return v;
 }
 
-__device__ __forceinline__ double warp_tree(FPair v, int lane, int present, int valid) {
+__device__ __forceinline__ double warp_tree(FTriple v, int lane, int present, int valid) {
   const unsigned mask = present >= 32 ? 0xffffffffu : ((1u << present) - 1u);
-  if (__any_sync(mask, !(fabsf(v.hi) < kPairMax))) return warp_tree(v.value(), lane, present, valid);
+  if (__any_sync(mask, !(fabsf(v.a) < kPairMax))) return warp_tree(v.value(), lane, present, valid);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     if (o >= valid) continue;
-    const float h = __shfl_down_sync(mask, v.hi, o), l = __shfl_down_sync(mask, v.lo, o);
-    if (lane + o < valid) v.add(h, l);
+    const float a = __shfl_down_sync(mask, v.a, o), b = __shfl_down_sync(mask, v.b, o);
+    const float c = __shfl_down_sync(mask, v.c, o);
+    if (lane + o < valid) v.add(a, b, c);
   }
   return v.value();
 }
 
-// Sum of NV values (FPair or double) over the block; out is valid in thread 0.
+__device__ __forceinline__ double warp_tree(FPair v, int lane, int present, int valid) {
+  return warp_tree(FTriple{v.hi, v.lo, 0.f}, lane, present, valid);
+}
+
+// Two sums over a full warp at once: the halves of the warp first exchange what
+// the other one takes, then the lower half adds the first value and the upper
+// half the second: five triple additions instead of ten.  With one warp per
+// scheduler, as in the row passes of the CG, the time goes by instructions
+// (256^2, CG of ten steps: two trees of pairs 275.6 us, two trees of triples
+// 2.3 % more, this one 272.8 us).  The first sum is valid in lane 0, the second in lane 16.
+__device__ __forceinline__ double warp_tree2(FTriple v0, FTriple v1, int lane) {
+  const unsigned mask = 0xffffffffu;
+  const bool up = (lane & 16) != 0;
+  if (__any_sync(mask, !(fabsf(v0.a) < kPairMax && fabsf(v1.a) < kPairMax))) {
+    const double s0 = warp_tree(v0, lane, 32, 32), s1 = warp_tree(v1, lane, 32, 32);
+    const double s1b = __shfl_sync(mask, s1, 0);
+    return up ? s1b : s0;
+  }
+  FTriple v = up ? v1 : v0;
+  const FTriple w = up ? v0 : v1;
+  v.add(__shfl_xor_sync(mask, w.a, 16), __shfl_xor_sync(mask, w.b, 16), __shfl_xor_sync(mask, w.c, 16));
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1)  // (lanes past a half's first o are not used any more)
+    v.add(__shfl_down_sync(mask, v.a, o), __shfl_down_sync(mask, v.b, o), __shfl_down_sync(mask, v.c, o));
+  return v.value();
+}
+
+__device__ __forceinline__ FTriple to_triple(FPair v) { return FTriple{v.hi, v.lo, 0.f}; }
+__device__ __forceinline__ FTriple to_triple(FTriple v) { return v; }
+
+// Sum of NV values (FPair, FTriple or double) over the block; out is valid in thread 0.
 template <int NV, class V>
 __device__ __forceinline__ void block_reduce(const V* v, double* out) {
   __shared__ double sh[NV][32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int nw = (blockDim.x + 31) >> 5;
   const int mylanes = min(32, (int)blockDim.x - wid * 32);
+  bool two = false;  // (uniform per warp) out[0] holds the first sum in lane 0, the second in lane 16
+  if constexpr (NV == 2 && !std::is_same<V, double>::value) two = mylanes == 32;
+  if constexpr (NV == 2 && !std::is_same<V, double>::value) {
+    if (two) out[0] = warp_tree2(to_triple(v[0]), to_triple(v[1]), lane);
+  }
+  if (!two) {
 #pragma unroll
-  for (int k = 0; k < NV; ++k) out[k] = warp_tree(v[k], lane, mylanes, mylanes);
+    for (int k = 0; k < NV; ++k) out[k] = warp_tree(v[k], lane, mylanes, mylanes);
+  }
   __syncthreads();
-  if (lane == 0) {
+  if (two) {
+    if ((lane & 15) == 0) sh[NV == 2 ? lane >> 4 : 0][wid] = out[0];
+  } else if (lane == 0) {
 #pragma unroll
     for (int k = 0; k < NV; ++k) sh[k][wid] = out[k];
   }
