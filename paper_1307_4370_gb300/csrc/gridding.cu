@@ -32,7 +32,7 @@ __global__ void __launch_bounds__(256) k_degrid(const float2* __restrict__ X, co
   constexpr int NT = 256;
   const int W = T + J - 1, NW = W * W;
   const float inv_w = 1.0f / (float)W;
-  FPair part[2];  // per-thread exact sums of a few terms; FP64 across threads
+  FTriple norms[2];  // this thread's part of the SDMM mode's norms over its chunks
   // One chunk per CTA; in the SDMM mode a CTA takes every gridDim-th chunk
   // (heavy chunks come first, so the shares are even): the norms' partial
   // sums then end in a few hundred tickets and terms for the last CTA instead
@@ -41,6 +41,7 @@ __global__ void __launch_bounds__(256) k_degrid(const float2* __restrict__ X, co
     const int4 ch = dchunks[q0];
     const int tr = ch.x / tiles_1d, tc = ch.x - tr * tiles_1d;
     const int R0 = tr * T, C0 = tc * T;
+    FPair part[2];  // ... over this chunk: a few terms, exactly
     // the first frequencies of this thread, in flight with the halo loads
     constexpr int QV = 4;
     float2 uq[QV];
@@ -162,11 +163,14 @@ __global__ void __launch_bounds__(256) k_degrid(const float2* __restrict__ X, co
     }
     for (int i = ch.y + threadIdx.x + QV * NT; i < ch.z; i += NT) visit(i, __ldg(&to[i]), __ldg(&uv[i]));
     if (MODE != kDegridSdmm) break;
+    // (one pair over all chunks would drop bits below 2^-47 of the sum)
+#pragma unroll
+    for (int k = 0; k < 2; ++k) norms[k].add(part[k].hi, part[k].lo, 0.f);
     __syncthreads();  // the halo is reused
   }
   if (MODE == kDegridSdmm) {
     double tot[2];
-    if (reduce_last_block<2>(part, partials + kCntL2 * 2 * kMaxPartials, &sc->counter[kCntL2], tot)) {
+    if (reduce_last_block<2>(norms, partials + kCntL2 * 2 * kMaxPartials, &sc->counter[kCntL2], tot)) {
       sc->l2_dn2 = tot[0];
       sc->l2_res2 = tot[1];
       sc->nu = sqrt(tot[1]) / sc->eps;

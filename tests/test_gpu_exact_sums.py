@@ -31,9 +31,9 @@ def test_norm(count, at):
     assert float(nrm.item()) == math.sqrt(int(BIG) ** 2 + (count - 1) * int(SMALL) ** 2)
 
 
-@pytest.mark.parametrize("n,M,at", [(64, 3000, 11)])
+@pytest.mark.parametrize("n,M,at", [(64, 3000, 11), (768, 60000, 7), (768, 60000, 30000), (768, 60000, 59999)])
 def test_sdmm_norms(n, M, at):
-    """nu of an iteration at x_hat = 0 (no CG step): ||y|| alone."""
+    """nu of an iteration at x_hat = 0 (no CG step): ||y|| alone, over one and over several units per CTA."""
     torch = require_gpu()
     from paper_1307_4370_gb300 import binding
 
