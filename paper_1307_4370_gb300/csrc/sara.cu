@@ -370,15 +370,14 @@ struct TailGeom {
 };
 
 template <int P, int MODE>
-__device__ __forceinline__ float dwt_tail_plane(const float2* __restrict__ src, int src_stride, float2* __restrict__ pl,
-                                                const TailGeom& G, const WaveletTaps& wf, float2* z1, float2* u1,
-                                                const float* w, float gamma) {
+__device__ __forceinline__ void dwt_tail_plane(const float2* __restrict__ src, int src_stride, float2* __restrict__ pl,
+                                               const TailGeom& G, const WaveletTaps& wf, float2* z1, float2* u1,
+                                               const float* w, float gamma, FPair& f1) {
   extern __shared__ float2 sm[];
   constexpr int taps = 2 * P;
   const float2 *h = wf.h + P * (P - 1), *g = wf.g + P * (P - 1);
   const int ST = (G.L + kTailExt) | 1;  // row stride (odd)
   float2 *A = sm, *B = sm + (G.L + kTailExt) * ST;
-  float f1 = 0.f;
   int L = G.L;
   Div dL = make_div(L);
   for (int e = threadIdx.x; e < L * L; e += kTailThreads) {
@@ -465,8 +464,8 @@ __device__ __forceinline__ float dwt_tail_plane(const float2* __restrict__ src, 
         if (!ll) pl[o] = ls;
         pl[o + Hn] = hs;
       } else {
-        if (!ll) f1 += sara_prox_v(ls, p.zl, p.wl, o, z1, u1, gamma);
-        f1 += sara_prox_v(hs, p.zh, p.wh, o + Hn, z1, u1, gamma);
+        if (!ll) f1.add(sara_prox_v(ls, p.zl, p.wl, o, z1, u1, gamma), 0.f);
+        f1.add(sara_prox_v(hs, p.zh, p.wh, o + Hn, z1, u1, gamma), 0.f);
       }
     };
     if (H % 2 == 0) {
@@ -508,7 +507,6 @@ __device__ __forceinline__ float dwt_tail_plane(const float2* __restrict__ src, 
     }
     __syncthreads();
   }
-  return f1;
 }
 
 template <int MODE>
@@ -519,13 +517,13 @@ __global__ void __launch_bounds__(kTailThreads) k_dwt_tail(const float2* __restr
   pdl_sync(in, coef, partials, sc);
   const int k = blockIdx.x;
   const float gamma = (MODE == kSaraProx) ? (float)sc->gamma : 0.f;
-  float f1 = 0.f;
+  FPair f1;  // (a thread has a dozen terms, summed exactly; one to four a level in k_dwt_level)
   if (k == G.nb) {  // the Dirac plane
     const size_t base = (size_t)G.dirac * G.n * G.n;
     for (int e = threadIdx.x; e < G.n * G.n; e += kTailThreads) {
       const float2 al = cscale(in[e], G.scale);
       if (MODE == kSaraPlain) coef[base + e] = al;
-      else f1 += sara_prox(al, base + e, pa, gamma);
+      else f1.add(sara_prox(al, base + e, pa, gamma), 0.f);
     }
   } else {
     const size_t base = (size_t)(G.plane0 + k) * G.n * G.n;
@@ -534,20 +532,19 @@ __global__ void __launch_bounds__(kTailThreads) k_dwt_tail(const float2* __restr
     const float* w = MODE == kSaraProx && pa.w ? pa.w + base : nullptr;
     float2* pl = coef + base;
     switch (bl.p(k)) {
-      case 1: f1 = dwt_tail_plane<1, MODE>(src, G.L, pl, G, wf, z1, u1, w, gamma); break;
-      case 2: f1 = dwt_tail_plane<2, MODE>(src, G.L, pl, G, wf, z1, u1, w, gamma); break;
-      case 3: f1 = dwt_tail_plane<3, MODE>(src, G.L, pl, G, wf, z1, u1, w, gamma); break;
-      case 4: f1 = dwt_tail_plane<4, MODE>(src, G.L, pl, G, wf, z1, u1, w, gamma); break;
-      case 5: f1 = dwt_tail_plane<5, MODE>(src, G.L, pl, G, wf, z1, u1, w, gamma); break;
-      case 6: f1 = dwt_tail_plane<6, MODE>(src, G.L, pl, G, wf, z1, u1, w, gamma); break;
-      case 7: f1 = dwt_tail_plane<7, MODE>(src, G.L, pl, G, wf, z1, u1, w, gamma); break;
-      default: f1 = dwt_tail_plane<8, MODE>(src, G.L, pl, G, wf, z1, u1, w, gamma); break;
+      case 1: dwt_tail_plane<1, MODE>(src, G.L, pl, G, wf, z1, u1, w, gamma, f1); break;
+      case 2: dwt_tail_plane<2, MODE>(src, G.L, pl, G, wf, z1, u1, w, gamma, f1); break;
+      case 3: dwt_tail_plane<3, MODE>(src, G.L, pl, G, wf, z1, u1, w, gamma, f1); break;
+      case 4: dwt_tail_plane<4, MODE>(src, G.L, pl, G, wf, z1, u1, w, gamma, f1); break;
+      case 5: dwt_tail_plane<5, MODE>(src, G.L, pl, G, wf, z1, u1, w, gamma, f1); break;
+      case 6: dwt_tail_plane<6, MODE>(src, G.L, pl, G, wf, z1, u1, w, gamma, f1); break;
+      case 7: dwt_tail_plane<7, MODE>(src, G.L, pl, G, wf, z1, u1, w, gamma, f1); break;
+      default: dwt_tail_plane<8, MODE>(src, G.L, pl, G, wf, z1, u1, w, gamma, f1); break;
     }
   }
   if (MODE == kSaraProx) {
-    const FPair f1p{f1, 0.f};
     double f1d;
-    block_reduce<1>(&f1p, &f1d);
+    block_reduce<1>(&f1, &f1d);
     if (threadIdx.x == 0) partials[kCntF1 * 2 * kMaxPartials + G.f1_off + blockIdx.x] = f1d;
   }
 }

@@ -1,6 +1,6 @@
 """Reductions whose exact value an FP64 sum holds (needs a GB300).
 
-The terms are integers that need more than the 48 bits
+The terms are integers (or multiples of 2^-25) that need more than the 48 bits
 of a float pair but fit FP64's 53, so the library's sums, FP64 once they leave
 a thread's few terms, must be exact: no tolerance.
 """
@@ -57,3 +57,28 @@ def test_sdmm_norms_beyond_float():
     st.init(dev(np.full(M, 2.0 ** 62, np.complex64), torch), 1.0, cg_iters=0)
     st.step()
     assert st.report()["nu"] == math.sqrt(M * 2.0 ** 124)
+
+
+HEADER = 48  # bytes before x_hat in an exported state
+
+
+@pytest.mark.parametrize("n,levels", [(64, 4), (32, 3)])
+def test_f1(n, levels):
+    """f1 = sum w |Psi^H x_hat| with the weights of the Dirac plane alone, moduli 1 and 2^-25 mixed."""
+    torch = require_gpu()
+    from paper_1307_4370_gb300 import binding
+
+    rng = np.random.default_rng(n)
+    M, N = 40, n * n
+    ctx = binding.Context(n, inputs.uniform_uv(M, rng).astype(np.float32), J=4, levels=levels, bases_mask=0xF)
+    st = ctx.sdmm_state()
+    st.init(dev(inputs.random_vis(M, rng), torch), 1.0, cg_iters=0)
+    one = rng.integers(0, 2, N).astype(bool)
+    blob = bytearray(st.export())
+    blob[HEADER:HEADER + 8 * N] = np.where(one, 2.0, 2.0 ** -24).astype(np.complex64).tobytes()  # x / sqrt(4 planes)
+    st.import_(bytes(blob))
+    w = np.zeros((4, N), np.float32)
+    w[0] = 1.0
+    st.set_weights(dev(w, torch))
+    st.step()
+    assert st.report()["f1"] == float(one.sum()) + float((~one).sum()) * 2.0 ** -25
