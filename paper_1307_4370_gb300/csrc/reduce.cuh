@@ -254,8 +254,9 @@ __device__ __forceinline__ CgStep cg_consume(const double* __restrict__ part, in
     return CgStep{(float)sc->alpha, (float)sc->beta, sc->cg_step_first != 0};
   }
   // the first warp adds the partials (fixed order) and forms the step sizes:
-  // one FP64 division each on lanes 0 and 1 while the partials arrive (the
-  // reciprocals of step j - 1's gamma and alpha), one after (gamma / den)
+  // gamma's quotients by step j - 1's gamma and alpha on lanes 0 and 1 together
+  // (an FP64 division takes 560 clocks), then alpha.  Reciprocals formed while
+  // the partials arrive would save one division, at a rounding more per quotient.
   if (threadIdx.x < 32) {  // (blocks have at least two threads)
     const int lane = threadIdx.x, present = min(32, (int)blockDim.x);
     const unsigned mask = present >= 32 ? 0xffffffffu : ((1u << present) - 1u);
@@ -268,15 +269,16 @@ __device__ __forceinline__ CgStep cg_consume(const double* __restrict__ part, in
       v[1] += __ldcg(&part[kMaxPartials + i]);
     }
     const unsigned zero = __ballot_sync(mask, old == 0.0);
-    const double inv = 1.0 / old;
-    const double inv_al = __shfl_sync(mask, inv, 1);
     v[0] = warp_tree(v[0], lane, present, min(present, nblk));
+    const double gamma = __shfl_sync(mask, v[0], 0);
+    const double quot = gamma / old;
+    const double quot_al = __shfl_sync(mask, quot, 1);
     v[1] = warp_tree(v[1], lane, present, min(present, nblk));
     if (lane == 0) {
-      const double gamma = v[0], delta = v[1];
+      const double delta = v[1];
       const bool first = j == 0 || (zero & 3u) != 0u;
-      const double beta = first ? 0.0 : gamma * inv;
-      const double den = first ? delta : delta - beta * gamma * inv_al;
+      const double beta = first ? 0.0 : quot;
+      const double den = first ? delta : delta - beta * quot_al;
       const double alpha = den > 0.0 ? gamma / den : 0.0;
       s_al = (float)alpha;
       s_be = (float)beta;

@@ -82,3 +82,22 @@ def test_f1(n, levels):
     st.set_weights(dev(w, torch))
     st.step()
     assert st.report()["f1"] == float(one.sum()) + float((~one).sum()) * 2.0 ** -25
+
+
+def test_cg_direction_update_is_the_fp64_quotient():
+    """beta of the last CG step of an iteration, against the two <r, r> it is the quotient of."""
+    torch = require_gpu()
+    from paper_1307_4370_gb300 import binding
+
+    rng = np.random.default_rng(3)
+    n, M = 32, 500
+    ctx = binding.Context(n, inputs.uniform_uv(M, rng).astype(np.float32), J=4, levels=3)
+    st = ctx.sdmm_state()
+    st.init(dev(inputs.random_vis(M, rng), torch), 1.0, cg_iters=3)
+    N, D = n * n, 9 * n * n
+    st.step()  # (starts from a zero residual)
+    for _ in range(24):
+        st.step()
+        # the scalars end the exported state: beta is the third, the last steps' <r, r> the 19th (even steps) and 20th
+        sc = np.frombuffer(st.export()[HEADER + 8 * (5 * N + D + 2 * M) + 4 * D:], np.float64, 22)
+        assert sc[2] == sc[18] / sc[19]
