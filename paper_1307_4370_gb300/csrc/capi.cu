@@ -14,6 +14,7 @@
 #include <cudaTypedefs.h>
 
 #include "common.cuh"
+#include "kernel_taps.h"
 
 using namespace purify;
 
@@ -88,26 +89,6 @@ int dev_alloc(T** p, size_t count) {
   return PURIFY_OK;
 }
 
-// ---------------------------------------------------------------------------
-// Kaiser-Bessel: beta of Beatty et al. (2005) for oversampling 2, the kernel
-// g(t) = I0(beta sqrt(1 - (2t/J)^2)) / I0(beta) and its closed-form transform.
-// ---------------------------------------------------------------------------
-double kb_beta(int J) {
-  const double a = 2.0;
-  return M_PI * std::sqrt((J / a) * (J / a) * (a - 0.5) * (a - 0.5) - 0.8);
-}
-
-double kb_g(double t, int J, double beta, double i0b) {
-  const double s = 2.0 * t / J;
-  if (std::fabs(s) > 1.0) return 0.0;
-  return std::cyl_bessel_i(0.0, beta * std::sqrt(std::max(0.0, 1.0 - s * s))) / i0b;
-}
-
-double kb_ghat(double f, int J, double beta, double i0b) {
-  const double a = std::sqrt(beta * beta - (M_PI * J * f) * (M_PI * J * f));
-  return J * std::sinh(a) / (i0b * a);
-}
-
 // Solve V c = f (Gaussian elimination with partial pivoting, long double).
 void solve_dense(std::vector<long double>& A, std::vector<long double>& b, int n) {
   for (int k = 0; k < n; ++k) {
@@ -129,24 +110,6 @@ void solve_dense(std::vector<long double>& A, std::vector<long double>& b, int n
     for (int j = k + 1; j < n; ++j) s -= A[k * n + j] * b[j];
     b[k] = s / A[k * n + k];
   }
-}
-
-// The paper's Gaussian kernel (§5): g(t) = exp(-b t^2) on |t| <= J/2 with
-// b = pi (alpha - 1/2) / (alpha J / 2), alpha = 2 (the width of Greengard &
-// Lee 2004 in grid cells); g_hat is the transform of the untruncated Gaussian.
-double gauss_b(int J) { return M_PI * 1.5 / (2.0 * (J / 2.0)); }
-double gauss_g(double t, int J) { return std::fabs(t) <= J / 2.0 ? std::exp(-gauss_b(J) * t * t) : 0.0; }
-double gauss_ghat(double f, int J) {
-  const double b = gauss_b(J);
-  return std::sqrt(M_PI / b) * std::exp(-M_PI * M_PI * f * f / b);
-}
-
-// g and g_hat of the context's kernel.
-double interp_g(double t, int J, int kernel, double beta, double i0b) {
-  return kernel == PURIFY_KERNEL_GAUSS ? gauss_g(t, J) : kb_g(t, J, beta, i0b);
-}
-double interp_ghat(double f, int J, int kernel, double beta, double i0b) {
-  return kernel == PURIFY_KERNEL_GAUSS ? gauss_ghat(f, J) : kb_ghat(f, J, beta, i0b);
 }
 
 // Fit each tap's weight, as a function of z = 2x - 1 on [-1, 1], by the
@@ -183,63 +146,6 @@ KbPoly fit_kb(int J, int kernel) {
   }
   kb.max_err = err;
   return kb;
-}
-
-// The same taps for the host's set-up, in double: Chebyshev interpolants of
-// degree 16 in z = 2x - 1, within 1e-12 of the kernels (checked at set-up), at
-// a tenth of the time of the Bessel function, which was a quarter of the
-// set-up at M = 2^21.
-struct TapSeries {
-  static constexpr int kTerms = 17;
-  int J, kernel;
-  bool exact;  // the series is not that good: evaluate g
-  double c[kMaxJ][kTerms];
-};
-
-double tap_value(const double* c, double z) {  // Clenshaw's recurrence
-  double b1 = 0.0, b2 = 0.0;
-  for (int k = TapSeries::kTerms - 1; k >= 1; --k) {
-    const double b0 = c[k] + 2.0 * z * b1 - b2;
-    b2 = b1;
-    b1 = b0;
-  }
-  return c[0] + z * b1 - b2;
-}
-
-TapSeries fit_taps(int J, int kernel) {
-  const double beta = kb_beta(J), i0b = std::cyl_bessel_i(0.0, beta);
-  constexpr int np = TapSeries::kTerms;
-  TapSeries p{};
-  p.J = J;
-  p.kernel = kernel;
-  double err = 0.0;
-  for (int a = 0; a < J; ++a) {
-    double f[np];
-    for (int i = 0; i < np; ++i)
-      f[i] = interp_g(0.5 * (std::cos(M_PI * (i + 0.5) / np) + 1.0) + J / 2 - 1 - a, J, kernel, beta, i0b);
-    for (int k = 0; k < np; ++k) {
-      double sum = 0.0;
-      for (int i = 0; i < np; ++i) sum += f[i] * std::cos(M_PI * k * (i + 0.5) / np);
-      p.c[a][k] = sum * (k == 0 ? 1.0 : 2.0) / np;
-    }
-    for (int t = 0; t < 64; ++t) {
-      const double x = (t + 0.37) / 64.0;
-      err = std::max(err, std::fabs(tap_value(p.c[a], 2.0 * x - 1.0) -
-                                    interp_g(x + J / 2 - 1 - a, J, kernel, beta, i0b)));
-    }
-  }
-  p.exact = !(err < 2e-12);
-  return p;
-}
-
-// Weights of the J taps for the fraction x in [0, 1).
-void tap_weights(const TapSeries& p, double x, double* w) {
-  if (p.exact) {
-    const double beta = kb_beta(p.J), i0b = std::cyl_bessel_i(0.0, beta);
-    for (int a = 0; a < p.J; ++a) w[a] = interp_g(x + p.J / 2 - 1 - a, p.J, p.kernel, beta, i0b);
-    return;
-  }
-  for (int a = 0; a < p.J; ++a) w[a] = tap_value(p.c[a], 2.0 * x - 1.0);
 }
 
 FftPlan make_plan(int L) {
@@ -846,6 +752,7 @@ static int purify_create_impl(purify_ctx** out, const purify_desc* d, const floa
   *out = nullptr;
   if (!d || !uv) return PURIFY_E_INVALID_ARG;
   if (d->oversample != 2) return PURIFY_E_SIZE;
+  static_assert(kTapsMaxJ == kMaxJ, "the host's taps cover every support of the kernels");
   if (d->J != 2 && d->J != 4 && d->J != 6 && d->J != 8) return PURIFY_E_SIZE;
   if (d->levels < 1 || d->levels > 6) return PURIFY_E_SIZE;
   if (d->n < 8 || d->n > 2048 || d->n % (1 << d->levels) != 0 || d->n % 2 != 0) return PURIFY_E_SIZE;
