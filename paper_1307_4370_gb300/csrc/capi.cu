@@ -792,11 +792,15 @@ static int purify_create_impl(purify_ctx** out, const purify_desc* d, const floa
   } else {
     c->homeT = c->L >= 512 ? 32 : (c->L >= 64 ? 16 : 8);
     while (c->homeT < c->J || c->L % c->homeT) c->homeT *= 2;
-    // gridding tiles of a 512 grid: 32 would leave 256 tiles, not two per SM
-    // (SDMM iteration at 256^2, M = 65536: tiles of 32 325 us, of 16 303 us; on
-    // 768 and larger grids 32 is the faster one, 384^2: 527 against 547 us).
-    // The sort keeps its tile: exported states and bf16 blocks follow it.
-    c->tileT = c->L == 512 ? 16 : c->homeT;
+    // gridding tiles of 32 halve to 16 while they would leave fewer than two
+    // per SM (the 512 grid: 256 tiles on 152 SMs; SDMM iteration at 256^2, M =
+    // 65536: tiles of 32 325 us, of 16 303 us; from the 768 grid on, 576 tiles,
+    // 32 is the faster one, 384^2: 527 against 547 us).  Contexts that fill the
+    // GPU together lose a little by it (a batch of six up to 512^2: 7.32 ms with
+    // tiles of 32, 7.50 ms so).  The sort keeps its tile: exported states and
+    // bf16 blocks follow it.
+    c->tileT = c->homeT;
+    while (c->tileT > 16 && (int64_t)(c->L / c->tileT) * (c->L / c->tileT) < 2 * (int64_t)c->sms) c->tileT /= 2;
   }
   c->tiles_1d = c->L / c->tileT;
   c->ntiles = c->tiles_1d * c->tiles_1d;
