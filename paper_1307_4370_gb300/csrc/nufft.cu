@@ -20,22 +20,21 @@
 namespace purify {
 
 // ---------------------------------------------------------------------------
-// Launch shapes
+// Launch shapes of the runtime engine: grid sides 16, 24, 32, 48, 64 and 96
+// (the compile-time engine has every other supported one, P2_SIDES)
 // ---------------------------------------------------------------------------
 struct FftShape {
-  int ept;      // elements per thread (8, 12 or 16)
+  int ept;      // elements per thread (8 or 12)
   int nsig;     // signals per CTA
   int threads;  // nsig * L / ept
 };
 
 static int pick_ept(int L) { return (L % 3 == 0) ? 12 : 8; }
 
-// Row passes: nsig rows per CTA, at most 256 threads (16 elements per thread
-// for L = 4096), nsig divides n.
+// Row passes: nsig rows per CTA, at most 128 threads, nsig divides n.
 static FftShape row_shape(const purify_ctx* c) {
   FftShape f;
   f.ept = pick_ept(c->L);
-  if (f.ept == 8 && c->L / 8 > 256) f.ept = 16;
   int nsig = 1;
   while (nsig * 2 * c->L / f.ept <= 128 && c->n % (nsig * 2) == 0) nsig *= 2;
   f.nsig = nsig;
@@ -43,13 +42,13 @@ static FftShape row_shape(const purify_ctx* c) {
   return f;
 }
 
-// Column passes: nsig adjacent columns per CTA (>= 4 for 32-byte segments).
+// Column passes: nsig adjacent columns per CTA (>= 4 for 32-byte segments), at
+// most 128 threads.
 static FftShape col_shape(const purify_ctx* c) {
   FftShape f;
   f.ept = pick_ept(c->L);
   int nsig = 4;
   while (nsig * 2 * c->L / f.ept <= 256 && c->L % (nsig * 2) == 0 && nsig < 16) nsig *= 2;
-  while (nsig > 1 && nsig * c->L / f.ept > 1024) nsig /= 2;  // at most 1024 threads
   f.nsig = nsig;
   f.threads = nsig * c->L / f.ept;
   return f;
@@ -453,12 +452,12 @@ __global__ void __launch_bounds__(NSIG * L / E) k_col_inv_p2(const float2* __res
 
 // Register cap: two CTAs per SM for the CG and plain epilogues; the SDMM
 // epilogue (five operands per pixel) keeps its registers.
-constexpr int p2_rinv_minb(int T, int E, int MODE) {
-  return MODE == kRowOutSdmm || E > 16 || 1024 / T <= 1 ? 1 : p2_min(1024 / T, 16);
+constexpr int p2_rinv_minb(int T, int MODE) {
+  return MODE == kRowOutSdmm || 1024 / T <= 1 ? 1 : p2_min(1024 / T, 16);
 }
 
 template <int L, int E, int NSIG, int MODE>
-__global__ void __launch_bounds__(NSIG * L / E, p2_rinv_minb(NSIG * L / E, E, MODE)) k_row_inv_p2(const float2* __restrict__ half, RowOutArgs a,
+__global__ void __launch_bounds__(NSIG * L / E, p2_rinv_minb(NSIG * L / E, MODE)) k_row_inv_p2(const float2* __restrict__ half, RowOutArgs a,
                                                              const float* __restrict__ dz,
                                                              const float* __restrict__ beam,
                                                              const float2* __restrict__ twt, int n,
@@ -534,7 +533,7 @@ int fft_prepare(purify_ctx* c) {
 #define P2_CASE(S) case S: return p2_prepare_L<S>(c);
     P2_SIDES(P2_CASE)
 #undef P2_CASE
-    default: c->fft_engine = 0; return PURIFY_OK;
+    default: return PURIFY_E_UNSUPPORTED;  // (fft_fixed_side has these sides only)
   }
 }
 
@@ -649,7 +648,7 @@ int phi_forward_grid(purify_ctx* c, RowInMode mode, const RowInArgs& a, cudaStre
   const float* beam = c->beam_on ? c->d_beam : nullptr;
   if (c->fft_engine == 1) {
     switch (c->L) {
-  #define P2_CASE(S) case S: return p2_forward<S>(c, mode, a, s, cg_j, beam);
+#define P2_CASE(S) case S: return p2_forward<S>(c, mode, a, s, cg_j, beam);
     P2_SIDES(P2_CASE)
 #undef P2_CASE
     default: break;
@@ -672,10 +671,6 @@ int phi_forward_grid(purify_ctx* c, RowInMode mode, const RowInArgs& a, cudaStre
     if (mode == kRowInPlain) ROWF(8, kRowInPlain);
     else if (mode == kRowInCgUpd) ROWF(8, kRowInCgUpd);
     else ROWF(8, kRowInCgFinish);
-  } else if (rs.ept == 16) {
-    if (mode == kRowInPlain) ROWF(16, kRowInPlain);
-    else if (mode == kRowInCgUpd) ROWF(16, kRowInCgUpd);
-    else ROWF(16, kRowInCgFinish);
   } else {
     if (mode == kRowInPlain) ROWF(12, kRowInPlain);
     else if (mode == kRowInCgUpd) ROWF(12, kRowInCgUpd);
@@ -701,7 +696,7 @@ int phi_adjoint_image(purify_ctx* c, RowOutMode mode, const RowOutArgs& a, cudaS
   const float2* Xg = grid ? grid : c->d_grid;
   if (c->fft_engine == 1) {
     switch (c->L) {
-  #define P2_CASE(S) case S: return p2_adjoint<S>(c, mode, a, s, Xg, before_rows, beam);
+#define P2_CASE(S) case S: return p2_adjoint<S>(c, mode, a, s, Xg, before_rows, beam);
     P2_SIDES(P2_CASE)
 #undef P2_CASE
     default: break;
@@ -736,10 +731,6 @@ int phi_adjoint_image(purify_ctx* c, RowOutMode mode, const RowOutArgs& a, cudaS
     if (mode == kRowOutPlain) ROWI(8, kRowOutPlain);
     else if (mode == kRowOutCgQ) ROWI(8, kRowOutCgQ);
     else ROWI(8, kRowOutSdmm);
-  } else if (rs.ept == 16) {
-    if (mode == kRowOutPlain) ROWI(16, kRowOutPlain);
-    else if (mode == kRowOutCgQ) ROWI(16, kRowOutCgQ);
-    else ROWI(16, kRowOutSdmm);
   } else {
     if (mode == kRowOutPlain) ROWI(12, kRowOutPlain);
     else if (mode == kRowOutCgQ) ROWI(12, kRowOutCgQ);
