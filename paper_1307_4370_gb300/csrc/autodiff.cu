@@ -357,7 +357,8 @@ __global__ void k_b2_bwd1(int64_t n, const float2* __restrict__ g, const float* 
 // z2bar = abar2, t = w o abar2 (gridded into x_bar next)
 __global__ void k_b2_bwd2(int64_t n, const float2* __restrict__ a2, const float* __restrict__ w,
                           const float2* __restrict__ y, int outside, float c, const BwdScalars* __restrict__ S,
-                          const float2* __restrict__ rb, float2* __restrict__ ab, const float2* __restrict__ phx, float* __restrict__ wb,
+                          const float2* __restrict__ rb, float2* __restrict__ ab, const float2* __restrict__ phx,
+                              float* __restrict__ wb,
                           float2* __restrict__ z2b_i, float2* __restrict__ t) {
   pdl_sync(a2, w, y, S, rb, ab, phx, wb, z2b_i, t);
   const float k2 = outside ? (float)S->k2 : 0.f;
@@ -519,7 +520,8 @@ size_t tape_bytes(const purify_ctx* c, int k) {
 int diff_scratch(purify_ctx* c, float2** m, float2** im, float2** dv, BwdScalars** bs = nullptr) {
   const int64_t N = nN(c), M = c->M, D = nD(c);
   if (!c->d_diff) {
-    if (cudaMalloc((void**)&c->d_diff, (size_t)(3 * M + 4 * N + D) * sizeof(float2) + sizeof(BwdScalars)) != cudaSuccess) {
+    if (cudaMalloc((void**)&c->d_diff,
+        (size_t)(3 * M + 4 * N + D) * sizeof(float2) + sizeof(BwdScalars)) != cudaSuccess) {
       cudaGetLastError();
       c->d_diff = nullptr;
       return PURIFY_E_ALLOC;
@@ -552,7 +554,8 @@ int phi_adj_into(purify_ctx* c, const float2* u, float2* out, cudaStream_t s) {
 
 int host_dot(purify_ctx* c, int64_t n, const float2* a, const float2* b, double* out, cudaStream_t s) {
   double* slot = &c->d_sc->norm2;
-  pdl_launch(k_dot, LaunchCfg{dblocks(n), 256, 0, s}, n, a, b, c->d_partials + kCntNorm * 2 * kMaxPartials, &c->d_sc->counter[kCntNorm],
+  pdl_launch(k_dot, LaunchCfg{dblocks(n), 256, 0, s}, n, a, b, c->d_partials + kCntNorm * 2 * kMaxPartials,
+      &c->d_sc->counter[kCntNorm],
                                   slot);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   if (int rc = check_cuda(cudaGetLastError())) return rc;
@@ -627,7 +630,8 @@ int diff_forward(purify_ctx* c, const DiffArgs& A, float2* const* in, float2* co
   RowOutArgs ra{};
   ra.out = im[1];
   if (int rc = apply_ww(c, x, A.w, T.PhiX0, m[0], kRowOutPlain, ra, s)) return rc;
-  LAUNCH((pdl_launch(k_resid0, LaunchCfg{dblocks(N), 256, 0, s}, N, b, im[1], x, T.R, k > 0 ? T.P : nullptr, k, part, cnt, H)));
+  LAUNCH((pdl_launch(k_resid0, LaunchCfg{dblocks(N), 256, 0, s}, N, b, im[1], x, T.R, k > 0 ? T.P : nullptr, k, part,
+      cnt, H)));
   // rho_0 = 0 (the zero state of the first iteration): no step is run, as in the oracle
   double rho0 = 0.0;
   if (k > 0) {
@@ -642,7 +646,8 @@ int diff_forward(purify_ctx* c, const DiffArgs& A, float2* const* in, float2* co
     ra.out = qj;
     ra.p = pj;
     if (int rc = apply_ww(c, pj, A.w, T.PhiP + (int64_t)j * M, m[0], kRowOutCgQ, ra, s)) return rc;
-    LAUNCH((pdl_launch(k_cg_upd, LaunchCfg{dblocks(N), 256, 0, s}, N, c->d_partials + kCntDot * 2 * kMaxPartials + kMaxPartials,
+    LAUNCH((pdl_launch(k_cg_upd, LaunchCfg{dblocks(N), 256, 0, s}, N,
+        c->d_partials + kCntDot * 2 * kMaxPartials + kMaxPartials,
                                                 cg_partial_blocks(c), j, x, pj, rj, qj, rj + N, part, cnt, H)));
     if (j + 1 < k) LAUNCH((pdl_launch(k_cg_dir, LaunchCfg{dblocks(N), 256, 0, s}, N, H, j, rj + N, pj, pj + N)));
   }
@@ -653,7 +658,8 @@ int diff_forward(purify_ctx* c, const DiffArgs& A, float2* const* in, float2* co
   if (int rc = sara_synthesis(c, T.U1, out[4], s)) return rc;
   // ---- i = 2: a2 = w o Phi x_hat' + z2; projection onto the ball around y_w
   if (int rc = phi_into(c, x, T.PhiXh, s)) return rc;
-  LAUNCH((pdl_launch(k_b2_a, LaunchCfg{dblocks(M), 256, 0, s}, M, T.PhiXh, A.w, in[2], A.y, T.A2, A.eps, part, cnt, H)));
+  LAUNCH((pdl_launch(k_b2_a, LaunchCfg{dblocks(M), 256, 0, s}, M, T.PhiXh, A.w, in[2], A.y, T.A2, A.eps, part, cnt,
+      H)));
   LAUNCH((pdl_launch(k_b2_b, LaunchCfg{dblocks(M), 256, 0, s}, M, T.A2, A.w, A.y, H, out[2], T.U2, m[1])));
   if (int rc = phi_adj_into(c, m[1], out[5], s)) return rc;
   // ---- i = 3
@@ -694,7 +700,8 @@ int diff_backward(purify_ctx* c, const DiffArgs& A, float2* const* in, const voi
   const int outside = H.nd > A.eps ? 1 : 0;
   if (outside)  // <d, rbar2>, d = a2 - y_w (FP64): the ball's Jacobian needs it
     LAUNCH((pdl_launch(k_dot_wdiff, LaunchCfg{dblocks(M), 256, 0, s}, M, T.A2, A.w, A.y, m[1], part, cnt, dH, S)));
-  LAUNCH((pdl_launch(k_b2_bwd2, LaunchCfg{dblocks(M), 256, 0, s}, M, T.A2, A.w, A.y, outside, (float)H.cball, S, m[1], m[2], T.PhiXh,
+  LAUNCH((pdl_launch(k_b2_bwd2, LaunchCfg{dblocks(M), 256, 0, s}, M, T.A2, A.w, A.y, outside, (float)H.cball, S,
+      m[1], m[2], T.PhiXh,
                                                wb, ib[2], m[0])));
   if (int rc = phi_adj_into(c, m[0], im[1], s)) return rc;
   LAUNCH((pdl_launch(k_add, LaunchCfg{dblocks(N), 256, 0, s}, N, xacc, im[1], xacc)));
@@ -708,15 +715,18 @@ int diff_backward(purify_ctx* c, const DiffArgs& A, float2* const* in, const voi
   RowOutArgs ra{};
   ra.out = vN;
   if (H.steps > 0)
-    LAUNCH((pdl_launch(k_cgb_first, LaunchCfg{dblocks(N), 256, 0, s}, N, xacc, T.P + (int64_t)(H.steps - 1) * N, part, cnt, S)));
+    LAUNCH((pdl_launch(k_cgb_first, LaunchCfg{dblocks(N), 256, 0, s}, N, xacc, T.P + (int64_t)(H.steps - 1) * N,
+        part, cnt, S)));
   for (int j = H.steps - 1; j >= 0; --j) {
     const float2* pj = T.P + (int64_t)j * N;
     const float2* qj = T.Qp + (int64_t)j * N;
-    LAUNCH((pdl_launch(k_cgb_r, LaunchCfg{dblocks(N), 256, 0, s}, N, rb, pb, T.R + (int64_t)(j + 1) * N, qj, j, part, cnt, dH, S)));
+    LAUNCH((pdl_launch(k_cgb_r, LaunchCfg{dblocks(N), 256, 0, s}, N, rb, pb, T.R + (int64_t)(j + 1) * N, qj, j, part,
+        cnt, dH, S)));
     LAUNCH((pdl_launch(k_cgb_q, LaunchCfg{dblocks(N), 256, 0, s}, N, dH, S, j, rb, pj, qb)));
     // v = Phi_w^H Phi_w qbar; w_bar += 2 w Re(conj(Phi qbar) Phi p_j)
     if (int rc = apply_ww(c, qb, A.w, nullptr, m[1], kRowOutPlain, ra, s, T.PhiP + (int64_t)j * M, 2.f, wb)) return rc;
-    LAUNCH((pdl_launch(k_cgb_p, LaunchCfg{dblocks(N), 256, 0, s}, N, dH, j, pb, xacc, qj, vN, qb, j > 0 ? pj - N : nullptr, part, cnt, S)));
+    LAUNCH((pdl_launch(k_cgb_p, LaunchCfg{dblocks(N), 256, 0, s}, N, dH, j, pb, xacc, qj, vN, qb,
+        j > 0 ? pj - N : nullptr, part, cnt, S)));
   }
   // p_0 = r_0 and rho_0 = <r_0, r_0>
   LAUNCH((pdl_launch(k_cgb_r, LaunchCfg{dblocks(N), 256, 0, s}, N, rb, pb, T.R, nullptr, 0, part, cnt, dH, S)));
@@ -818,7 +828,8 @@ int purify_diff_penalty(purify_ctx* c, const float* y, const float* wvis, double
     if (rc == PURIFY_OK) rc = sara_analysis(c, im[0], dv, kSaraPlain, pa, s);
     if (rc == PURIFY_OK) rc = launch_max_abs(c, nD(c), dv, s);
     double amax = 0.0;
-    if (rc == PURIFY_OK) rc = check_cuda(cudaMemcpyAsync(&amax, &c->d_sc->amax, sizeof(double), cudaMemcpyDeviceToHost, s));
+    if (rc == PURIFY_OK) rc = check_cuda(cudaMemcpyAsync(&amax, &c->d_sc->amax, sizeof(double),
+        cudaMemcpyDeviceToHost, s));
     if (rc == PURIFY_OK) rc = check_cuda(cudaStreamSynchronize(s));
     if (rc == PURIFY_OK) *gamma = beta * amax;
   }
@@ -833,7 +844,8 @@ int purify_vjp_soft_threshold(int64_t count, const float* a, const float* w, flo
   if (!ok_dev(a) || !ok_dev(rbar) || !ok_dev(abar) || (w && !ok_dev(w)) || (wbar && !ok_dev(wbar)))
     return PURIFY_E_NOT_DEVICE_PTR;
   cudaStream_t s = (cudaStream_t)stream;
-  pdl_launch(k_vjp_soft, LaunchCfg{dblocks(count), 256, 0, s}, count, (const float2*)a, w, gamma, (const float2*)rbar, (float2*)abar,
+  pdl_launch(k_vjp_soft, LaunchCfg{dblocks(count), 256, 0, s}, count, (const float2*)a, w, gamma,
+      (const float2*)rbar, (float2*)abar,
                                             wbar);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return check_cuda(cudaGetLastError());
@@ -844,7 +856,8 @@ int purify_vjp_positive(int64_t count, const float* a, const float* rbar, float*
   if (count == 0) return PURIFY_OK;
   if (!ok_dev(a) || !ok_dev(rbar) || !ok_dev(abar)) return PURIFY_E_NOT_DEVICE_PTR;
   cudaStream_t s = (cudaStream_t)stream;
-  pdl_launch(k_vjp_pos, LaunchCfg{dblocks(count), 256, 0, s}, count, (const float2*)a, (const float2*)rbar, (float2*)abar);
+  pdl_launch(k_vjp_pos, LaunchCfg{dblocks(count), 256, 0, s}, count, (const float2*)a, (const float2*)rbar,
+      (float2*)abar);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return check_cuda(cudaGetLastError());
 }
@@ -857,7 +870,8 @@ int purify_vjp_l2ball(purify_ctx* c, int64_t count, const float* a, const float*
   cudaGetDevice(&prev);
   if (prev != c->device) cudaSetDevice(c->device);
   int rc = PURIFY_OK;
-  if (!ok_dev(a) || !ok_dev(y) || !ok_dev(rbar) || !ok_dev(abar) || (ybar && !ok_dev(ybar))) rc = PURIFY_E_NOT_DEVICE_PTR;
+  if (!ok_dev(a) || !ok_dev(y) || !ok_dev(rbar) || !ok_dev(abar) ||
+      (ybar && !ok_dev(ybar))) rc = PURIFY_E_NOT_DEVICE_PTR;
   cudaStream_t s = (cudaStream_t)stream;
   if (rc == PURIFY_OK) {
     // ||a - y||^2 and <a - y, rbar> = <a, rbar> - <y, rbar> in FP64
@@ -874,7 +888,8 @@ int purify_vjp_l2ball(purify_ctx* c, int64_t count, const float* a, const float*
       const int outside = nd > eps ? 1 : 0;
       const double cb = outside ? eps / nd : 1.0;
       const float k2 = outside ? (float)(cb * (ar - yr) / nd2) : 0.f;
-      pdl_launch(k_vjp_ball, LaunchCfg{dblocks(count), 256, 0, s}, count, A, Y, outside, (float)cb, k2, RB, (float2*)abar,
+      pdl_launch(k_vjp_ball, LaunchCfg{dblocks(count), 256, 0, s}, count, A, Y, outside, (float)cb, k2, RB,
+          (float2*)abar,
                                                  (float2*)ybar);
       g_launches.fetch_add(1, std::memory_order_relaxed);
       rc = check_cuda(cudaGetLastError());

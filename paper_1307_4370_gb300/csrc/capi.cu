@@ -266,7 +266,9 @@ void encode_halo_map(purify_ctx* c) {
 
 void free_ctx(purify_ctx* c) {
   if (!c) return;
-  void* ptrs[] = {c->d_dense_tiles, c->d_H, c->d_gram_chunks, c->d_diff, c->d_twp[0], c->d_twp[1], c->d_deapod, c->d_beam, c->d_tv, c->d_tw, c->d_uv, c->d_dpos, c->d_dperm, c->d_perm, c->d_list, c->d_chunks, c->d_chunk_tab, c->d_items, c->d_item_row, c->d_dchunks, c->d_tile_slot0,
+  void* ptrs[] = {c->d_dense_tiles, c->d_H, c->d_gram_chunks, c->d_diff, c->d_twp[0], c->d_twp[1], c->d_deapod,
+      c->d_beam, c->d_tv, c->d_tw, c->d_uv, c->d_dpos, c->d_dperm, c->d_perm, c->d_list, c->d_chunks, c->d_chunk_tab,
+      c->d_items, c->d_item_row, c->d_dchunks, c->d_tile_slot0,
                   c->d_tile_nchunk, c->d_tile_cnt, c->d_slots,
                   c->d_grid, c->d_grid2, c->d_half, c->d_vis, c->d_vis2, c->d_ll[0], c->d_ll[1], c->d_img[0],
                   c->d_img[1], c->d_img[2], c->d_img[3], c->d_partials, c->d_sc};
@@ -596,7 +598,8 @@ int setup_visibilities(purify_ctx* c, const float* uv_in, cudaStream_t s) {
       ;
     if (st == PURIFY_OK) {
       if ((c->n_dense > 0 &&
-           (cudaMemcpy(c->d_dense_tiles, dense.data(), dense.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
+           (cudaMemcpy(c->d_dense_tiles, dense.data(), dense.size() * sizeof(int),
+               cudaMemcpyHostToDevice) != cudaSuccess ||
             cudaMemcpy(c->d_H, H.data(), H.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess)) ||
           (c->n_gram_chunks > 0 && cudaMemcpy(c->d_gram_chunks, gram_chunks.data(), gram_chunks.size() * sizeof(int),
                                               cudaMemcpyHostToDevice) != cudaSuccess))
@@ -808,7 +811,8 @@ static int purify_create_impl(purify_ctx** out, const purify_desc* d, const floa
   int st = PURIFY_OK;
   auto fail = [&](int code) { free_ctx(c); return code; };
   if ((st = dev_alloc(&c->d_deapod, c->n)) || (st = dev_alloc(&c->d_tw, c->L)) ||
-      (st = dev_alloc(&c->d_grid, (size_t)c->L * c->L)) || (st = dev_alloc(&c->d_grid2, (size_t)c->L * c->L)) || (st = dev_alloc(&c->d_half, (size_t)c->n * c->L)) ||
+      (st = dev_alloc(&c->d_grid, (size_t)c->L * c->L)) || (st = dev_alloc(&c->d_grid2, (size_t)c->L * c->L)) ||
+          (st = dev_alloc(&c->d_half, (size_t)c->n * c->L)) ||
       (st = dev_alloc(&c->d_vis, c->M)) || (st = dev_alloc(&c->d_vis2, c->M)) ||
       (st = dev_alloc(&c->d_ll[0], c->q * n2)) || (st = dev_alloc(&c->d_ll[1], c->q * n2)) ||
       (st = dev_alloc(&c->d_img[0], N)) || (st = dev_alloc(&c->d_img[1], N)) || (st = dev_alloc(&c->d_img[2], N)) ||
@@ -816,12 +820,14 @@ static int purify_create_impl(purify_ctx** out, const purify_desc* d, const floa
       (st = dev_alloc(&c->d_partials, (size_t)kNumCounters * 2 * kMaxPartials)) ||
       (st = dev_alloc(&c->d_sc, 1)))
     return fail(st);
-  if (cudaMallocHost((void**)&c->h_sc, sizeof(DevScalars)) != cudaSuccess) { cudaGetLastError(); return fail(PURIFY_E_ALLOC); }
+  if (cudaMallocHost((void**)&c->h_sc,
+      sizeof(DevScalars)) != cudaSuccess) { cudaGetLastError(); return fail(PURIFY_E_ALLOC); }
   // deapodisation 1 / g_hat((r - n/2) / 2n) and twiddles exp(-2 pi i m / L), in double
   {
     const double beta = kb_beta(c->J), i0b = std::cyl_bessel_i(0.0, beta);
     std::vector<float> dz(c->n);
-    for (int r = 0; r < c->n; ++r) dz[r] = (float)(1.0 / interp_ghat((double)(r - c->n / 2) / c->L, c->J, c->kernel, beta, i0b));
+    for (int r = 0; r < c->n; ++r) dz[r] = (float)(1.0 / interp_ghat((double)(r - c->n / 2) / c->L, c->J, c->kernel,
+        beta, i0b));
     std::vector<float2> tw(c->L);
     for (int m = 0; m < c->L; ++m) {
       const double a = -2.0 * M_PI * (double)m / c->L;

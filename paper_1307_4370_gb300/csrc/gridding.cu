@@ -25,8 +25,8 @@ namespace purify {
 template <int J, int MODE>
 __global__ void __launch_bounds__(256) k_degrid(const float2* __restrict__ X, const float2* __restrict__ uv,
                                                 const int* __restrict__ dpos, const int* __restrict__ dperm,
-                                                DegridArgs a, const int4* __restrict__ dchunks, int nchunks, KbPoly kb, KappaScale ks,
-                                                int L, int T, int tiles_1d, double* partials, DevScalars* sc) {
+                                                DegridArgs a, const int4* __restrict__ dchunks, int nchunks,
+                                                KbPoly kb, KappaScale ks, int L, int T, int tiles_1d, double* partials, DevScalars* sc) {
   pdl_sync(X, uv, dpos, dperm, dchunks, partials, sc);
   extern __shared__ float2 halo[];
   constexpr int NT = 256;
@@ -273,7 +273,8 @@ __global__ void __launch_bounds__(kGridThreads, MINB) k_grid(float2* __restrict_
                                                        const int* __restrict__ dense_tiles,
                                                        const float* __restrict__ H,
                                                        const int* __restrict__ gram_chunks, int dense_half) {
-  pdl_sync(X, Xin, perm, vis, list, chunks, tab, items, item_row, tile_slot0, tile_nchunk, tile_cnt, slots, sc, dense_tiles, H, gram_chunks);
+  pdl_sync(X, Xin, perm, vis, list, chunks, tab, items, item_row, tile_slot0, tile_nchunk, tile_cnt, slots, sc,
+           dense_tiles, H, gram_chunks);
   constexpr int NT = kGridThreads;
   constexpr int S = grid_wstride(J);  // [0 wr_0 .. wr_{J-1} 0 | 0 wc_0 .. wc_{J-1} 0 | pad]
   extern __shared__ __align__(128) float4 sm4[];
@@ -627,19 +628,22 @@ __global__ void __launch_bounds__(kGridThreads, MINB) k_grid(float2* __restrict_
   if (threadIdx.x == 0) tile_cnt[tile] = 0u;
 }
 
-constexpr int kDegridPerSm = 8;  // CTAs of the SDMM mode per SM (4: 108 us, 8: 97 us, a CTA per chunk: 119 us, beside the prior branch)
+// CTAs of the SDMM mode per SM (4: 108 us, 8: 97 us, a CTA per chunk: 119 us, beside the prior branch)
+constexpr int kDegridPerSm = 8;
 template <int J>
 static void degrid_J(purify_ctx* c, DegridOut mode, const DegridArgs& a, cudaStream_t s) {
   const int threads = 256;
   const int W = c->homeT + J - 1;
   const size_t sm = (size_t)W * W * sizeof(float2);
-#define DEG(MD)                                                                                               \
-  do {                                                                                                        \
-    allow_smem(k_degrid<J, MD>, sm);                                                                          \
-    PURIFY_LAUNCH(c, "degrid", s,                                                                             \
-                  (pdl_launch(k_degrid<J, MD>, LaunchCfg{MD == kDegridSdmm ? std::min(c->ndchunks, kDegridPerSm * c->sms) : c->ndchunks, threads, sm, s}, c->d_grid, c->d_uv, c->d_dpos, c->d_dperm, a, c->d_dchunks, \
-                                                                    c->ndchunks, c->kb, c->ks, c->L, c->homeT, c->L / c->homeT, \
-                                                                    c->d_partials, c->d_sc)));                     \
+  const int ctas = mode == kDegridSdmm ? std::min(c->ndchunks, kDegridPerSm * c->sms) : c->ndchunks;
+  const LaunchCfg lc{ctas, threads, sm, s};
+#define DEG(MD)                                                                                             \
+  do {                                                                                                      \
+    allow_smem(k_degrid<J, MD>, sm);                                                                        \
+    PURIFY_LAUNCH(c, "degrid", s,                                                                           \
+                  (pdl_launch(k_degrid<J, MD>, lc, c->d_grid, c->d_uv, c->d_dpos, c->d_dperm, a, c->d_dchunks, \
+                              c->ndchunks, c->kb, c->ks, c->L, c->homeT, c->L / c->homeT, c->d_partials,    \
+                              c->d_sc)));                                                                   \
   } while (0)
   if (mode == kDegridPerm) DEG(kDegridPerm);
   else if (mode == kDegridSorted) DEG(kDegridSorted);
@@ -668,17 +672,18 @@ static size_t grid_smem(const purify_ctx* c) {
 // shared memory) keep more registers.
 template <int J, int MINB>
 static void grid_JB(purify_ctx* c, GridIn mode, const float2* vis, size_t sm, cudaStream_t s) {
-#define GRD(MD, NAME, OUT, IN)                                                                                 \
-  do {                                                                                                         \
-    allow_smem(k_grid<J, MD, MINB>, sm);                                                                       \
-    PURIFY_LAUNCH(c, NAME, s,                                                                                  \
-                  (pdl_launch(k_grid<J, MD, MINB>, LaunchCfg{MD == kGridGram ? c->n_dense + c->n_gram_chunks : c->nchunks, kGridThreads, sm, s},                                                \
-                      OUT, IN, c->d_perm, vis, c->d_list, c->d_chunks, c->d_chunk_tab, c->chunk_tab_stride,     \
-                      c->d_items, c->d_item_row,                                                                \
-                      c->d_tile_slot0, c->d_tile_nchunk,                                                        \
-                      c->d_tile_cnt, c->d_slots, c->kb, c->ks, c->L, c->tileT, c->tiles_1d, c->chunk_max,      \
-                      c->halo_map, c->halo_map_ok, c->d_sc, c->n_dense, c->d_dense_tiles, c->d_H,             \
-                      c->d_gram_chunks, c->dense_half)));                                                       \
+  const int ctas = mode == kGridGram ? c->n_dense + c->n_gram_chunks : c->nchunks;
+  const LaunchCfg lc{ctas, kGridThreads, sm, s};
+#define GRD(MD, NAME, OUT, IN)                                                                              \
+  do {                                                                                                      \
+    allow_smem(k_grid<J, MD, MINB>, sm);                                                                    \
+    PURIFY_LAUNCH(c, NAME, s,                                                                               \
+                  (pdl_launch(k_grid<J, MD, MINB>, lc, OUT, IN, c->d_perm, vis, c->d_list, c->d_chunks,     \
+                              c->d_chunk_tab, c->chunk_tab_stride, c->d_items, c->d_item_row,               \
+                              c->d_tile_slot0, c->d_tile_nchunk, c->d_tile_cnt, c->d_slots, c->kb, c->ks,   \
+                              c->L, c->tileT, c->tiles_1d, c->chunk_max, c->halo_map, c->halo_map_ok,       \
+                              c->d_sc, c->n_dense, c->d_dense_tiles, c->d_H, c->d_gram_chunks,              \
+                              c->dense_half)));                                                             \
   } while (0)
   if (mode == kGridPerm) GRD(kGridPerm, "grid", c->d_grid, nullptr);
   else if (mode == kGridSorted) GRD(kGridSorted, "grid", c->d_grid, nullptr);

@@ -457,11 +457,9 @@ constexpr int p2_rinv_minb(int T, int MODE) {
 }
 
 template <int L, int E, int NSIG, int MODE>
-__global__ void __launch_bounds__(NSIG * L / E, p2_rinv_minb(NSIG * L / E, MODE)) k_row_inv_p2(const float2* __restrict__ half, RowOutArgs a,
-                                                             const float* __restrict__ dz,
-                                                             const float* __restrict__ beam,
-                                                             const float2* __restrict__ twt, int n,
-                                                             double* partials) {
+__global__ void __launch_bounds__(NSIG * L / E, p2_rinv_minb(NSIG * L / E, MODE))
+    k_row_inv_p2(const float2* __restrict__ half, RowOutArgs a, const float* __restrict__ dz,
+                 const float* __restrict__ beam, const float2* __restrict__ twt, int n, double* partials) {
   pdl_sync(half, dz, beam, twt, partials);
   extern __shared__ float2 sm[];
   const int r0 = blockIdx.x * NSIG;
@@ -561,7 +559,7 @@ static int p2_forward(purify_ctx* c, RowInMode mode, const RowInArgs& a, cudaStr
   do {                                                                                                    \
     allow_smem(k_row_fwd_p2<L, C::E_CG, NS, MD>, sm);                                                     \
     PURIFY_LAUNCH(c, "row_fwd", s,                                                                        \
-                  (pdl_launch(k_row_fwd_p2<L, C::E_CG, NS, MD>, LaunchCfg{n / NS, NS * L / C::E_CG, sm, s},                   \
+                  (pdl_launch(k_row_fwd_p2<L, C::E_CG, NS, MD>, LaunchCfg{n / NS, NS * L / C::E_CG, sm, s},            \
                       a, c->d_half, c->d_deapod, beam, twcg, n, c->d_sc, cgpart, cg_nblk, cg_j)));          \
   } while (0)
     if (mode == kRowInCgUpd) ROWCG(kRowInCgUpd);
@@ -573,7 +571,8 @@ static int p2_forward(purify_ctx* c, RowInMode mode, const RowInArgs& a, cudaStr
     constexpr size_t sm = p2_smem_bytes<L, NS>();
     allow_smem(k_col_fwd_p2<L, C::E, NS>, sm);
     PURIFY_LAUNCH(c, "col_fwd", s,
-                  (pdl_launch(k_col_fwd_p2<L, C::E, NS>, LaunchCfg{L / NS, NS * L / C::E, sm, s}, c->d_half, c->d_grid, tw, n)));
+                  (pdl_launch(k_col_fwd_p2<L, C::E, NS>, LaunchCfg{L / NS, NS * L / C::E, sm, s}, c->d_half,
+                      c->d_grid, tw, n)));
   }
   return check_cuda(cudaGetLastError());
 }
@@ -589,7 +588,8 @@ static int p2_adjoint(purify_ctx* c, RowOutMode mode, const RowOutArgs& a, cudaS
     constexpr int NS = C::NS_COL;
     constexpr size_t sm = p2_smem_bytes<L, NS>();
     allow_smem(k_col_inv_p2<L, C::E, NS>, sm);
-    PURIFY_LAUNCH(c, "col_inv", s, (pdl_launch(k_col_inv_p2<L, C::E, NS>, LaunchCfg{L / NS, NS * L / C::E, sm, s}, Xg, c->d_half, tw, n)));
+    PURIFY_LAUNCH(c, "col_inv", s, (pdl_launch(k_col_inv_p2<L, C::E, NS>, LaunchCfg{L / NS, NS * L / C::E, sm, s},
+        Xg, c->d_half, tw, n)));
   }
   if (before_rows) {
     const int rc = check_cuda(cudaStreamWaitEvent(s, before_rows, 0));
@@ -601,7 +601,8 @@ static int p2_adjoint(purify_ctx* c, RowOutMode mode, const RowOutArgs& a, cudaS
   do {                                                                                                     \
     allow_smem(k_row_inv_p2<L, C::E, NS, MD>, sm);                                                         \
     PURIFY_LAUNCH(c, "row_inv", s,                                                                         \
-                  (pdl_launch(k_row_inv_p2<L, C::E, NS, MD>, LaunchCfg{n / NS, NS * L / C::E, sm, s, !before_rows}, c->d_half, a, c->d_deapod, \
+                  (pdl_launch(k_row_inv_p2<L, C::E, NS, MD>, LaunchCfg{n / NS, NS * L / C::E, sm, s, !before_rows},    \
+                      c->d_half, a, c->d_deapod,                                                                       \
                                                                                      beam, tw, n,            \
                                                                                      c->d_partials)));       \
   } while (0)
@@ -639,7 +640,8 @@ __global__ void __launch_bounds__(256) k_cg_scalars(const double* __restrict__ p
 
 int launch_cg_scalars(purify_ctx* c, int cg_j, cudaStream_t s) {
   PURIFY_LAUNCH(c, "cg_scalars", s,
-                (pdl_launch(k_cg_scalars, LaunchCfg{1, 256, 0, s}, c->d_partials + kCntDot * 2 * kMaxPartials, cg_partial_blocks(c), cg_j,
+                (pdl_launch(k_cg_scalars, LaunchCfg{1, 256, 0, s}, c->d_partials + kCntDot * 2 * kMaxPartials,
+                    cg_partial_blocks(c), cg_j,
                                                c->d_sc)));
   return check_cuda(cudaGetLastError());
 }
@@ -664,7 +666,8 @@ int phi_forward_grid(purify_ctx* c, RowInMode mode, const RowInArgs& a, cudaStre
   do {                                                                                                     \
     allow_smem(k_row_fwd<E, MD>, smr);                                                                     \
     PURIFY_LAUNCH(c, "row_fwd", s,                                                                         \
-                  (pdl_launch(k_row_fwd<E, MD>, LaunchCfg{gr, rs.threads, smr, s, !a.first}, a, c->d_half, c->d_deapod, beam, c->d_tw, c->plan, \
+                  (pdl_launch(k_row_fwd<E, MD>, LaunchCfg{gr, rs.threads, smr, s, !a.first}, a, c->d_half,             \
+                      c->d_deapod, beam, c->d_tw, c->plan,                                                             \
                                                                 c->n, rs.nsig, c->d_sc, cgpart, cg_nblk, cg_j)));   \
   } while (0)
   if (rs.ept == 8) {
@@ -680,11 +683,13 @@ int phi_forward_grid(purify_ctx* c, RowInMode mode, const RowInArgs& a, cudaStre
   if (cs.ept == 8) {
     allow_smem(k_col_fwd<8>, smc);
     PURIFY_LAUNCH(c, "col_fwd", s,
-                  (pdl_launch(k_col_fwd<8>, LaunchCfg{gc, cs.threads, smc, s}, c->d_half, c->d_grid, c->d_tw, c->plan, c->n, cs.nsig)));
+                  (pdl_launch(k_col_fwd<8>, LaunchCfg{gc, cs.threads, smc, s}, c->d_half, c->d_grid, c->d_tw,
+                      c->plan, c->n, cs.nsig)));
   } else {
     allow_smem(k_col_fwd<12>, smc);
     PURIFY_LAUNCH(c, "col_fwd", s,
-                  (pdl_launch(k_col_fwd<12>, LaunchCfg{gc, cs.threads, smc, s}, c->d_half, c->d_grid, c->d_tw, c->plan, c->n, cs.nsig)));
+                  (pdl_launch(k_col_fwd<12>, LaunchCfg{gc, cs.threads, smc, s}, c->d_half, c->d_grid, c->d_tw,
+                      c->plan, c->n, cs.nsig)));
   }
   return check_cuda(cudaGetLastError());
 }
@@ -709,11 +714,13 @@ int phi_adjoint_image(purify_ctx* c, RowOutMode mode, const RowOutArgs& a, cudaS
   if (cs.ept == 8) {
     allow_smem(k_col_inv<8>, smc);
     PURIFY_LAUNCH(c, "col_inv", s,
-                  (pdl_launch(k_col_inv<8>, LaunchCfg{gc, cs.threads, smc, s}, Xg, c->d_half, c->d_tw, c->plan, c->n, cs.nsig)));
+                  (pdl_launch(k_col_inv<8>, LaunchCfg{gc, cs.threads, smc, s}, Xg, c->d_half, c->d_tw, c->plan, c->n,
+                      cs.nsig)));
   } else {
     allow_smem(k_col_inv<12>, smc);
     PURIFY_LAUNCH(c, "col_inv", s,
-                  (pdl_launch(k_col_inv<12>, LaunchCfg{gc, cs.threads, smc, s}, Xg, c->d_half, c->d_tw, c->plan, c->n, cs.nsig)));
+                  (pdl_launch(k_col_inv<12>, LaunchCfg{gc, cs.threads, smc, s}, Xg, c->d_half, c->d_tw, c->plan,
+                      c->n, cs.nsig)));
   }
   // the row pass may read operands of another stream (the SDMM prior branch)
   if (before_rows) {
@@ -724,7 +731,8 @@ int phi_adjoint_image(purify_ctx* c, RowOutMode mode, const RowOutArgs& a, cudaS
   do {                                                                                                       \
     allow_smem(k_row_inv<E, MD>, smr);                                                                       \
     PURIFY_LAUNCH(c, "row_inv", s,                                                                           \
-                  (pdl_launch(k_row_inv<E, MD>, LaunchCfg{gr, rs.threads, smr, s, !before_rows}, c->d_half, a, c->d_deapod, beam, c->d_tw, c->plan, \
+                  (pdl_launch(k_row_inv<E, MD>, LaunchCfg{gr, rs.threads, smr, s, !before_rows}, c->d_half, a,         \
+                      c->d_deapod, beam, c->d_tw, c->plan,                                                             \
                                                                 c->n, rs.nsig, c->d_partials, c->d_sc)));     \
   } while (0)
   if (rs.ept == 8) {

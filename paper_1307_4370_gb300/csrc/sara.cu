@@ -102,8 +102,9 @@ __global__ void k_dirac(const float2* __restrict__ x, float2* __restrict__ alpha
 // FAST (tiles of a multiple of four): a thread filters four adjacent outputs
 // of a row, then two of a column, from one window of inputs, (2P + 6) / 8 and
 // (2P + 2) / 4 shared-memory loads per output instead of P (one output pair
-// per thread: all four levels at 1024^2 83 us; 74 us so, issue-bound), and lanes take consecutive rows of an odd stride, so neither pass has
-// bank conflicts.
+// per thread: all four levels at 1024^2 83 us; 74 us so, issue-bound), and
+// lanes take consecutive rows of an odd stride, so neither pass has bank
+// conflicts.
 template <int P, int MODE, bool FAST>
 __device__ __forceinline__ float dwt_plane(const float2* __restrict__ in, int in_shared, float2* __restrict__ ll_out,
                                            float2* __restrict__ coef, const LevelGeom& G, const WaveletTaps& wf,
@@ -1012,14 +1013,17 @@ int sara_analysis(purify_ctx* c, const float2* x, float2* alpha, SaraMode mode, 
     int blocks = (int)std::min<int64_t>((N + 255) / 256, 1024);
     if (mode == kSaraPlain)
       PURIFY_LAUNCH(c, "dirac", s,
-                    (pdl_launch(k_dirac<kSaraPlain>, LaunchCfg{blocks, 256, 0, s, false}, x, alpha + (size_t)dirac_plane * N, N, scale, pa,
+                    (pdl_launch(k_dirac<kSaraPlain>, LaunchCfg{blocks, 256, 0, s, false}, x,
+                        alpha + (size_t)dirac_plane * N, N, scale, pa,
                                                                 c->d_partials, c->d_sc)));
     else
       PURIFY_LAUNCH(c, "dirac", s,
-                    (pdl_launch(k_dirac<kSaraProx>, LaunchCfg{blocks, 256, 0, s, false}, x, nullptr, N, scale, pa, c->d_partials, c->d_sc)));
+                    (pdl_launch(k_dirac<kSaraProx>, LaunchCfg{blocks, 256, 0, s, false}, x, nullptr, N, scale, pa,
+                        c->d_partials, c->d_sc)));
   }
   if (nb == 0) {
-    if (mode == kSaraProx) PURIFY_LAUNCH(c, "finish_zeta", s, (pdl_launch(k_finish_zeta, LaunchCfg{1, 1, 0, s}, c->d_sc)));
+    if (mode == kSaraProx) PURIFY_LAUNCH(c, "finish_zeta", s, (pdl_launch(k_finish_zeta, LaunchCfg{1, 1, 0, s},
+        c->d_sc)));
     return check_cuda(cudaGetLastError());
   }
   int maxp = 1;
@@ -1039,11 +1043,13 @@ int sara_analysis(purify_ctx* c, const float2* x, float2* alpha, SaraMode mode, 
       if (mode == kSaraPlain) {
         allow_smem(k_dwt_tail<kSaraPlain>, sm);
         PURIFY_LAUNCH(c, "dwt_level", s,
-                      (pdl_launch(k_dwt_tail<kSaraPlain>, lc, in, lev == 0, alpha, G, bl, taps, pa, c->d_partials, c->d_sc)));
+                      (pdl_launch(k_dwt_tail<kSaraPlain>, lc, in, lev == 0, alpha, G, bl, taps, pa, c->d_partials,
+                          c->d_sc)));
       } else {
         allow_smem(k_dwt_tail<kSaraProx>, sm);
         PURIFY_LAUNCH(c, "dwt_level", s,
-                      (pdl_launch(k_dwt_tail<kSaraProx>, lc, in, lev == 0, pa.z1, G, bl, taps, pa, c->d_partials, c->d_sc)));
+                      (pdl_launch(k_dwt_tail<kSaraProx>, lc, in, lev == 0, pa.z1, G, bl, taps, pa, c->d_partials,
+                          c->d_sc)));
       }
       break;
     }
@@ -1074,7 +1080,8 @@ int sara_analysis(purify_ctx* c, const float2* x, float2* alpha, SaraMode mode, 
       *f1_parts = f1_off;
     } else {  // no synthesis follows to finish f1: one block does
       PURIFY_LAUNCH(c, "f1_finish", s,
-                    (pdl_launch(k_f1_finish, LaunchCfg{1, 256, 0, s}, c->d_partials + kCntF1 * 2 * kMaxPartials, f1_off, c->d_sc)));
+                    (pdl_launch(k_f1_finish, LaunchCfg{1, 256, 0, s}, c->d_partials + kCntF1 * 2 * kMaxPartials,
+                        f1_off, c->d_sc)));
     }
   }
   return check_cuda(cudaGetLastError());
@@ -1088,7 +1095,8 @@ int sara_synthesis(purify_ctx* c, const float2* alpha, float2* x, cudaStream_t s
   const float scale = 1.0f / sqrtf((float)c->q);
   if (nb == 0) {
     int blocks = (int)std::min<int64_t>((N + 255) / 256, 1024);
-    PURIFY_LAUNCH(c, "dirac", s, (pdl_launch(k_dirac_syn, LaunchCfg{blocks, 256, 0, s}, alpha + (size_t)dirac_plane * N, x, N, scale)));
+    PURIFY_LAUNCH(c, "dirac", s, (pdl_launch(k_dirac_syn, LaunchCfg{blocks, 256, 0, s},
+        alpha + (size_t)dirac_plane * N, x, N, scale)));
     return check_cuda(cudaGetLastError());
   }
   int maxp = 1;

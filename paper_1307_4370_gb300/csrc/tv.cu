@@ -251,7 +251,8 @@ static int tv_fgp(purify_ctx* c, float2* scratch, const float2* xa, const float2
   int a = 0;  // the set that holds the current dual variables
   if (iters == 0)
     PURIFY_LAUNCH(c, "tv_init", s,
-                  (pdl_launch(k_tv_init, LaunchCfg{tv_blocks(N), 256, 0, s, chained}, N, xa, xb, b, set[0].p, set[0].q)));
+                  (pdl_launch(k_tv_init, LaunchCfg{tv_blocks(N), 256, 0, s, chained}, N, xa, xb, b, set[0].p,
+                      set[0].q)));
   // tiles of 32 once they give every SM one, of 16 (a region of 26 x 26, 2.6
   // times the arithmetic) on smaller images
   const int t32 = (c->n + 31) / 32, t16 = (c->n + 15) / 16;
@@ -311,7 +312,8 @@ int tv_sdmm_branch(purify_ctx* c, purify_sdmm_state* st, cudaStream_t s) {
 int tv_gradmag(purify_ctx* c, const float2* x, float2** g, cudaStream_t s) {
   float2* sc_buf = nullptr;
   TV_TRY(tv_scratch_ready(c, &sc_buf));
-  PURIFY_LAUNCH(c, "tv_gradmag", s, (pdl_launch(k_tv_gradmag, LaunchCfg{tv_blocks(((int64_t)c->n * c->n)), 256, 0, s}, c->n, x, sc_buf)));
+  PURIFY_LAUNCH(c, "tv_gradmag", s, (pdl_launch(k_tv_gradmag, LaunchCfg{tv_blocks(((int64_t)c->n * c->n)), 256, 0,
+      s}, c->n, x, sc_buf)));
   *g = sc_buf;
   return check_cuda(cudaGetLastError());
 }

@@ -341,56 +341,65 @@ __global__ void __launch_bounds__(256) k_quantize_bf16(int64_t M, const float2* 
 
 __global__ void k_set_gamma(DevScalars* sc, double beta) {
   pdl_sync(sc);
-  sc->gamma = beta * sc->amax; }
+  sc->gamma = beta * sc->amax;
+}
 
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
 int launch_soft_threshold(int64_t count, const float2* in, const float* w, const double* gamma_dev, float gamma,
                           float2* out, cudaStream_t s) {
-  PURIFY_LAUNCH(nullptr, "soft", s, (pdl_launch(k_soft, LaunchCfg{blocks_once(count), 256, 0, s}, count, in, w, gamma_dev, gamma, out)));
+  PURIFY_LAUNCH(nullptr, "soft", s, (pdl_launch(k_soft, LaunchCfg{blocks_once(count), 256, 0, s}, count, in, w,
+      gamma_dev, gamma, out)));
   return check_cuda(cudaGetLastError());
 }
 
 int launch_l2_norm_diff(purify_ctx* c, int64_t count, const float2* a, const float2* b, cudaStream_t s) {
-  PURIFY_LAUNCH(c, "norm_diff", s, (pdl_launch(k_norm_diff, LaunchCfg{blocks_for(count), 256, 0, s}, count, a, b, c->d_partials, c->d_sc)));
+  PURIFY_LAUNCH(c, "norm_diff", s, (pdl_launch(k_norm_diff, LaunchCfg{blocks_for(count), 256, 0, s}, count, a, b,
+      c->d_partials, c->d_sc)));
   return check_cuda(cudaGetLastError());
 }
 
 int launch_l2_project(int64_t count, const float2* in, const float2* y, double eps, const double* norm2_dev,
                       float2* out, cudaStream_t s) {
-  PURIFY_LAUNCH(nullptr, "l2_project", s, (pdl_launch(k_l2_project, LaunchCfg{blocks_for(count), 256, 0, s}, count, in, y, eps, norm2_dev, out)));
+  PURIFY_LAUNCH(nullptr, "l2_project", s, (pdl_launch(k_l2_project, LaunchCfg{blocks_for(count), 256, 0, s}, count,
+      in, y, eps, norm2_dev, out)));
   return check_cuda(cudaGetLastError());
 }
 
 int launch_positive(int64_t count, const float2* in, float2* out, cudaStream_t s) {
-  PURIFY_LAUNCH(nullptr, "positive", s, (pdl_launch(k_positive, LaunchCfg{blocks_for(count), 256, 0, s}, count, in, out)));
+  PURIFY_LAUNCH(nullptr, "positive", s, (pdl_launch(k_positive, LaunchCfg{blocks_for(count), 256, 0, s}, count, in,
+      out)));
   return check_cuda(cudaGetLastError());
 }
 
 int launch_cg_apply(purify_ctx* c, float2* x, float2* r, float2* p, float2* sv, const float2* w, int cg_j,
                     cudaStream_t s) {
   const int64_t N = (int64_t)c->n * c->n;
-  PURIFY_LAUNCH(c, "cg_apply", s, (pdl_launch(k_cg_apply, LaunchCfg{blocks_for(N), 256, 0, s}, N, x, r, p, sv, w, c->d_partials, c->d_sc,
+  PURIFY_LAUNCH(c, "cg_apply", s, (pdl_launch(k_cg_apply, LaunchCfg{blocks_for(N), 256, 0, s}, N, x, r, p, sv, w,
+      c->d_partials, c->d_sc,
                                                                            cg_consumer_blocks(c), cg_j)));
   return check_cuda(cudaGetLastError());
 }
 
 int launch_cg_residual_init(purify_ctx* c, const float2* b, const float2* qx, float2* r, cudaStream_t s) {
   const int64_t N = (int64_t)c->n * c->n;
-  PURIFY_LAUNCH(c, "cg_residual_init", s, (pdl_launch(k_cg_residual_init, LaunchCfg{blocks_for(N), 256, 0, s}, N, b, qx, r, c->d_sc)));
+  PURIFY_LAUNCH(c, "cg_residual_init", s, (pdl_launch(k_cg_residual_init, LaunchCfg{blocks_for(N), 256, 0, s}, N, b,
+      qx, r, c->d_sc)));
   return check_cuda(cudaGetLastError());
 }
 
 int launch_max_abs(purify_ctx* c, int64_t count, const float2* a, cudaStream_t s) {
-  PURIFY_LAUNCH(c, "max_abs", s, (pdl_launch(k_max_abs, LaunchCfg{blocks_for(count), 256, 0, s}, count, a, c->d_partials, c->d_sc)));
+  PURIFY_LAUNCH(c, "max_abs", s, (pdl_launch(k_max_abs, LaunchCfg{blocks_for(count), 256, 0, s}, count, a,
+      c->d_partials, c->d_sc)));
   return check_cuda(cudaGetLastError());
 }
 
 int launch_sdmm_l2_update(purify_sdmm_state* st, cudaStream_t s) {
   purify_ctx* c = st->ctx;
   const bool blk = st->nblocks > 0;
-  PURIFY_LAUNCH(st->ctx, "sdmm_l2", s, (pdl_launch(k_sdmm_l2, LaunchCfg{blocks_for(c->M), 256, 0, s}, c->M, st->s2, st->z2, st->y_bf16 ? nullptr : st->y, st->yb,
+  PURIFY_LAUNCH(st->ctx, "sdmm_l2", s, (pdl_launch(k_sdmm_l2, LaunchCfg{blocks_for(c->M), 256, 0, s}, c->M, st->s2,
+      st->z2, st->y_bf16 ? nullptr : st->y, st->yb,
                                              st->yscale, st->v, c->d_sc, blk ? st->d_block_of : nullptr,
                                              blk ? st->d_bscale : nullptr)));
   return check_cuda(cudaGetLastError());
@@ -399,7 +408,8 @@ int launch_sdmm_l2_update(purify_sdmm_state* st, cudaStream_t s) {
 int launch_block_norms(purify_sdmm_state* st, cudaStream_t s) {
   purify_ctx* c = st->ctx;
   PURIFY_LAUNCH(c, "block_norms", s,
-                (pdl_launch(k_block_norms, LaunchCfg{st->nbchunks, 256, 0, s}, st->d_bchunks, st->nbchunks, st->d_pos, st->s2, st->z2,
+                (pdl_launch(k_block_norms, LaunchCfg{st->nbchunks, 256, 0, s}, st->d_bchunks, st->nbchunks,
+                    st->d_pos, st->s2, st->z2,
                                                             st->y_bf16 ? nullptr : st->y, st->yb, st->yscale,
                                                             st->nblocks, st->d_beps, st->d_bscale,
                                                             c->d_partials + kCntBlk * 2 * kMaxPartials, c->d_sc)));
@@ -407,7 +417,8 @@ int launch_block_norms(purify_sdmm_state* st, cudaStream_t s) {
 }
 
 int launch_reweight(purify_ctx* c, int64_t count, const float2* alpha, float* w, int round, cudaStream_t s) {
-  PURIFY_LAUNCH(c, "reweight", s, (pdl_launch(k_reweight, LaunchCfg{blocks_for(count), 256, 0, s}, count, alpha, w, round, c->d_sc)));
+  PURIFY_LAUNCH(c, "reweight", s, (pdl_launch(k_reweight, LaunchCfg{blocks_for(count), 256, 0, s}, count, alpha, w,
+      round, c->d_sc)));
   return check_cuda(cudaGetLastError());
 }
 
@@ -418,7 +429,8 @@ int launch_gather_perm(int64_t M, const float2* src, const int* perm, float2* ds
 
 int launch_quantize_bf16(int64_t M, const float2* y, uint16_t* yb, float* yscale, cudaStream_t s) {
   const int64_t blocks = (M + 4095) / 4096;
-  PURIFY_LAUNCH(nullptr, "quantize_bf16", s, (pdl_launch(k_quantize_bf16, LaunchCfg{(unsigned)blocks, 256, 0, s}, M, y, reinterpret_cast<uint32_t*>(yb), yscale)));
+  PURIFY_LAUNCH(nullptr, "quantize_bf16", s, (pdl_launch(k_quantize_bf16, LaunchCfg{(unsigned)blocks, 256, 0, s}, M,
+      y, reinterpret_cast<uint32_t*>(yb), yscale)));
   return check_cuda(cudaGetLastError());
 }
 
