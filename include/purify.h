@@ -137,6 +137,11 @@ typedef struct {
  * device as float stencils: (2J - 1)^2 values per cell, or about half that
  * when the stencils fit a quarter of L2 (at most 4 (2J - 1)^2 bytes per grid
  * cell of the dense tiles; 200 MB for the 1024 x 1024, M = 2^21 workload).
+ * With J <= 4 lists count as dense from a few entries on, as far as 32 MB of
+ * stencils hold them; that takes 1 to 8 % of this call's time (512 x 512, M =
+ * 235293, J = 4: 26.6 ms, 25.7 without; 1024 x 1024, M = 400000, J = 2: 47.6
+ * and 44.2).  The stencils serve purify_cg_solve and the SDMM only; a context
+ * that is used for Phi and Phi^H or differentiated builds them all the same.
  * This call synchronises `stream`.  PURIFY_E_SIZE if a gridding work unit
  * does not fit the walk's encoding (not reached for the supported sizes),
  * PURIFY_E_ALLOC if device or host memory runs out.
