@@ -850,7 +850,6 @@ static int purify_create_impl(purify_ctx** out, const purify_desc* d, const floa
     st = PURIFY_E_ALLOC;
   }
   if (st != PURIFY_OK) return fail(st);
-  // shared memory above 48 KB needs an opt-in per kernel; sizes here stay below it
   *out = c;
   return PURIFY_OK;
 }

@@ -199,10 +199,14 @@ struct DevScalars {
 
 
 // Static plus dynamic shared memory above 48 KB needs a per-kernel opt-in
-// (the kernels' static shared memory is well under 8 KB).
+// (the kernels' static shared memory is well under 8 KB).  The limit belongs to
+// the kernel, so it is the same for every launch: a launch's own size as the
+// limit would let another thread's smaller launch lower it before this one
+// (the kernel's footprint and occupancy follow the launch, not the limit).
+constexpr int kMaxDynamicSmem = (227 - 8) * 1024;
 template <class K>
 inline void allow_smem(K kernel, size_t bytes) {
-  if (bytes > 40 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (bytes > 40 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynamicSmem);
 }
 
 // ---------------------------------------------------------------------------
