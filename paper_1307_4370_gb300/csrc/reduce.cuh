@@ -16,8 +16,8 @@ namespace purify {
 // Per-thread accumulation without FP64 arithmetic (GB300 has little FP64
 // throughput): terms are formed exactly with error-free transformations
 // (TwoSum for a difference, an FMA for a product's rounding error) and summed
-// into a float pair (hi, lo); the pair goes to FP64 once per thread, and the
-// sums across threads and blocks are FP64.  With the few terms each thread
+// into a float pair (hi, lo); the pairs of a warp are added as triples (below),
+// and the sums across warps and blocks are FP64.  With the few terms each thread
 // holds, the per-thread error is far below FP64 rounding of the total.
 // ---------------------------------------------------------------------------
 struct FPair {
